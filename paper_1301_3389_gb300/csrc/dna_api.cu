@@ -55,6 +55,10 @@ struct dna_ctx {
     // split plans (pass 1 and pass 2 / KL) for the H view and the W view
     int sp1[2] = {1, 1}, sp2[2] = {1, 1};
     int64_t per1[2] = {0, 0}, per2[2] = {0, 0};
+    // splits of pass 1 in the differentiation form (its sums over s run in ascending order
+    // within a split)
+    int dsp1[2] = {1, 1};
+    int64_t dper1[2] = {0, 0};
     // tensor-core (BF16) path
     bool tc = false;
     bool split = false;              // FP32 form on the tensor cores (hi + lo bf16 operands)
@@ -202,6 +206,27 @@ void plan_split(int64_t S, int64_t nblocks_os, int slots, int chunk, int* splits
     *splits = (int)((S + *per - 1) / *per);
 }
 
+// Splits of a float32 pass on the CUDA cores (f32_pass.cuh: chunks and o-blocks of 64), by
+// the time they should take in microseconds: an SM works its share of the CTAs off at
+// chunk_us per chunk whether one or two of them are resident, but a lone CTA hides its own
+// latencies less well (1.3); a CTA costs about 1 us to start and end, the partial sums of a
+// split part_us, and reading several splits back one more launch.
+void plan_f2(int64_t S, int64_t nob, int sms, double chunk_us, double part_us, int* splits,
+             int64_t* per) {
+    const int64_t chunks = (S + 63) / 64;
+    int64_t best = chunks;
+    double best_us = 1e300;
+    for (int64_t sp = 1; sp <= std::min<int64_t>(chunks, 64); ++sp) {
+        const int64_t pc = (chunks + sp - 1) / sp;
+        const int64_t load = (nob * ((chunks + pc - 1) / pc) + sms - 1) / sms;
+        const double us = (double)load * ((double)pc * chunk_us + 1.0) * (load == 1 ? 1.3 : 1.0) +
+                          (double)sp * part_us + (sp > 4 ? 3.0 : 0.5 * (double)(sp - 1));
+        if (us < best_us) { best_us = us; best = pc; }
+    }
+    *per = best * 64;
+    *splits = (int)((S + *per - 1) / *per);
+}
+
 // Chunks of 128 that one pass-1 CTA of the split FP32 form accumulates in tensor memory
 // (1024 values of s: the accumulation error stays near 1e-6 relative).
 constexpr int64_t SPLIT_CHUNK = 128;
@@ -218,12 +243,27 @@ void plan_all(dna_ctx* c) {
     const int ob = S::oblock(), ch = S::chunk();
     const int rb = S::rblock(c->R);
     const int64_t nrb = (c->R + rb - 1) / rb;
-    const int b1 = S::pass1_blocks_per_sm(c->R), b2 = S::pass2_blocks_per_sm(c->R);
+    const int b1 = S::pass1_blocks_per_sm(c->R);
+    const bool f2 = sizeof(Tp) == 4 && c->R <= dna::f2::MAX_R;   // the passes of f32_pass.cuh
     for (int w = 0; w < 2; ++w) {
         const int64_t Sdim = w ? c->T : c->N, Odim = w ? c->N : c->T;
         const int64_t nob = (Odim + ob - 1) / ob;
-        plan_split(Sdim, nob * nrb, c->num_sms * b1, ch, &c->sp1[w], &c->per1[w]);
-        plan_split(Sdim, nob, c->num_sms * b2, ch, &c->sp2[w], &c->per2[w]);
+        plan_split(Sdim, nob * nrb, c->num_sms * b1, ch, &c->dsp1[w], &c->dper1[w]);
+        c->sp1[w] = c->dsp1[w];
+        c->per1[w] = c->dper1[w];
+        if (f2) {
+            // a chunk of pass 1 (pass 2) takes about 0.9 (0.55) us per 16 ranks and 0.8 us for
+            // the rest; a split writes and reads 2 R values (2 float64) per column at 4 TB/s
+            const double r16 = (double)((c->R + 15) / 16), o = (double)Odim;
+            if (!c->tc)
+                plan_f2(Sdim, nob, c->num_sms, 0.9 * r16 + 0.8, 16e-6 / 4.0 * (double)c->R * o,
+                        &c->sp1[w], &c->per1[w]);
+            plan_f2(Sdim, nob, c->num_sms, 0.55 * r16 + 0.8, 32e-6 / 4.0 * o, &c->sp2[w],
+                    &c->per2[w]);
+        } else {
+            plan_split(Sdim, nob, c->num_sms * S::pass2_blocks_per_sm(c->R), ch, &c->sp2[w],
+                       &c->per2[w]);
+        }
         if (c->tc) {
             const int tob = dna::TcBf16::oblock(), tch = dna::TcBf16::chunk();
             c->pad_o[w] = (Odim + tob - 1) / tob * tob;
@@ -284,7 +324,8 @@ int alloc_workspace(dna_ctx* c) {
     int64_t ap = 0, dp = 0;
     for (int w = 0; w < 2; ++w) {
         const int64_t O = w ? N : T;
-        ap = std::max<int64_t>(ap, (int64_t)std::max(c->sp1[w], c->tsp1[w]) * R * O);
+        ap = std::max<int64_t>(
+            ap, (int64_t)std::max(std::max(c->sp1[w], c->dsp1[w]), c->tsp1[w]) * R * O);
         dp = std::max<int64_t>(dp, (int64_t)std::max(c->sp2[w], c->tsp2[w]) * 2 * O);
     }
     c->ldvt = (N + 3) / 4 * 4;
@@ -544,10 +585,10 @@ int step_h_fixed(dna_ctx* c, uint8_t* choice_out) {
     Tp* Xdna = static_cast<Tp*>(c->Xdna);
     int e = phase(c, DNA_PHASE_SUMS, 1, [&] { return S::factor_sums_y(v, c->o.lambda, c->c, c->fwork, st); });
     if (!e) e = phase(c, DNA_PHASE_PASS1, 1, [&] {
-        return S::pass1(v, A, B, c->sp1[0], c->per1[0], true, c->status, st);
+        return S::pass1(v, A, B, c->dsp1[0], c->dper1[0], true, c->status, st, nullptr, true);
     });
     if (!e) e = phase(c, DNA_PHASE_CANDIDATES, 1, [&] {
-        return S::candidates(v, c->c, A, B, c->sp1[0], Xmu, Xdna, c->o.eps, c->o.alpha, st);
+        return S::candidates(v, c->c, A, B, c->dsp1[0], Xmu, Xdna, c->o.eps, c->o.alpha, st);
     });
     if (!e) e = phase(c, DNA_PHASE_PASS2, 1, [&] {
         return S::pass2(v, Xmu, Xdna, c->dpart, c->sp2[0], c->per2[0], c->status, st);
@@ -584,10 +625,10 @@ int step_h_adjoint(dna_ctx* c, const Tp* Hk, const uint8_t* choice, const Tp* Hb
     Tp* Abar = static_cast<Tp*>(c->Xmu);
     Tp* Bbar = static_cast<Tp*>(c->Xdna);
     int e = S::factor_sums_y(v, c->o.lambda, c->c, c->fwork, st);
-    if (!e) e = S::pass1(v, A, B, c->sp1[0], c->per1[0], true, c->status, st);
+    if (!e) e = S::pass1(v, A, B, c->dsp1[0], c->dper1[0], true, c->status, st, nullptr, true);
     if (!e)
-        e = S::adjoint_h(v, c->c, A, B, c->sp1[0], choice, Hbar_next, Hbar_out, Abar, Bbar,
-                         c->dpart, A, c->sp1[0], c->per1[0], Vbar, c->T, c->o.eps, c->o.alpha,
+        e = S::adjoint_h(v, c->c, A, B, c->dsp1[0], choice, Hbar_next, Hbar_out, Abar, Bbar,
+                         c->dpart, A, c->dsp1[0], c->dper1[0], Vbar, c->T, c->o.eps, c->o.alpha,
                          c->status, st, Wbar ? c->wg_cpart : nullptr);
     if (!e && Wbar)
         e = S::adjoint_w(v, Abar, Bbar, c->wg_cpart, static_cast<Tp*>(c->wg_part), c->wsp,
@@ -693,7 +734,7 @@ int step_core(dna_ctx* c, int w, bool mu_only, bool prepared, int stop) {
         // (in the candidates kernel each further split is another round of dependent loads;
         // the sums are the same, ascending split order either way)
         const int parts = stop == STOP_PASS2 ? 1 : sp1;
-        const bool presum = (int64_t)parts * v.O >= 32768 && parts > 1;
+        const bool presum = parts > 4 || ((int64_t)parts * v.O >= 32768 && parts > 1);
         e = phase(c, DNA_PHASE_CANDIDATES, presum ? 2 : 1, [&] {
             if (presum)
                 if (int r = S::split_sum(A, B, c->R, v.O, parts, st)) return r;
@@ -859,9 +900,9 @@ int kl_backward(dna_ctx* c, double scale, Tp* dW, Tp* dH, Tp* dV) {
         if (!G) continue;
         const View v = make_view(c, w == 1);
         int e = S::factor_sums_y(v, 0.0, c->c, c->fwork, st);
-        if (!e) e = S::pass1(v, A, A, c->sp1[w], c->per1[w], false, c->status, st);
-        if (!e) e = w ? S::grad_x(v, c->c, A, c->sp1[w], scale, G, 1, c->R, st)
-                      : S::grad_x(v, c->c, A, c->sp1[w], scale, G, c->T, 1, st);
+        if (!e) e = S::pass1(v, A, A, c->dsp1[w], c->dper1[w], false, c->status, st, nullptr, true);
+        if (!e) e = w ? S::grad_x(v, c->c, A, c->dsp1[w], scale, G, 1, c->R, st)
+                      : S::grad_x(v, c->c, A, c->dsp1[w], scale, G, c->T, 1, st);
         if (e) return e;
     }
     if (dV) return S::grad_v(make_view(c, false), scale, dV, c->T, c->status, st);

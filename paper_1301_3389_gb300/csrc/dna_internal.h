@@ -68,7 +68,8 @@ template <typename Tp> struct Simt {
     // pass 1: raw sums Apart = sum_s y q, Bpart = sum_s y^2 qbar (split over s); with dcur,
     // also the starting factor's per-column costs [splits][O] (descent selection)
     static int pass1(const View& v, Tp* Apart, Tp* Bpart, int splits, int64_t s_per,
-                     bool with_b, int* status, cudaStream_t st, double* dcur = nullptr);
+                     bool with_b, int* status, cudaStream_t st, double* dcur = nullptr,
+                     bool ascending = false);
     // candidates: MU and renormalised Newton candidates, laid out [R][O]
     static int candidates(const View& v, const double* c, const Tp* Apart, const Tp* Bpart,
                           int splits, Tp* Xmu, Tp* Xdna, double eps, double alpha,
@@ -177,6 +178,22 @@ template <typename Tp> struct Simt {
     static int oblock();  // the o-block of passes 1 and 2
     static int rblock(int64_t R);  // the r-block of pass 1
 };
+
+// The passes in float32 at ranks up to MAX_R (f32_pass.cuh): Simt<float> takes them where
+// they apply, with the same arguments.
+namespace f2 {
+constexpr int64_t MAX_R = 128;
+// ascending: every sum over s in ascending order within a split (the order of the
+// differentiation form), else the faster grouping of s at ranks up to 64
+int pass1(const View& v, float* Apart, float* Bpart, int splits, int64_t s_per, bool with_b,
+          bool ascending, int* status, cudaStream_t st);
+int pass2(const View& v, const float* Xmu, const float* Xdna, double* dpart, int splits,
+          int64_t s_per, int* status, cudaStream_t st);
+int pass2_one(const View& v, const float* X, double* dpart, int splits, int64_t s_per,
+              int* status, cudaStream_t st);
+int kl_columns(const View& v, double* dpart, int splits, int64_t s_per, int* status,
+               cudaStream_t st);
+}  // namespace f2
 
 // Tensor-core (tcgen05) operands of one half-step, bf16, zero-padded:
 //   Xk [O_pad][RP]  x(r, o) K-major (GEMM1 A)      Yk   [S_pad][RP] y(s, r) (GEMM1 B)

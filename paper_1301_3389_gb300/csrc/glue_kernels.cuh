@@ -378,6 +378,46 @@ __global__ void __launch_bounds__(256) k_split_sum(Tp* __restrict__ A, Tp* __res
     }
 }
 
+// The same sums for many splits of a small matrix: CTA = 32 values (or float4s) x 8 groups of
+// threads, group g adding the contiguous splits [g k, (g + 1) k) (k = ceil(splits / 8), up
+// to eight loads in flight) and the eight group sums added in order.  blockIdx.y picks A or
+// B.  With one thread per value the loads of the splits follow one another in rounds of
+// L2 latency: 64 splits of 80 x 165 values take 16 rounds there and one here.
+template <typename Tp, int VEC>
+__global__ void __launch_bounds__(256) k_split_sum_par(Tp* __restrict__ A, Tp* __restrict__ B,
+                                                       int64_t n, int splits) {
+    __shared__ Tp red[8][32][VEC];
+    Tp* M = blockIdx.y ? B : A;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int64_t i = ((int64_t)blockIdx.x * 32 + tx) * VEC;
+    const int k = (splits + 7) / 8, s0 = ty * k, s1 = min(splits, s0 + k);
+    Tp acc[VEC];
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) acc[q] = Tp(0);
+    if (i < n)
+#pragma unroll 8
+        for (int sp = s0; sp < s1; ++sp) {
+            const Tp* p = M + (int64_t)sp * n + i;
+            if constexpr (VEC == 4) {
+                const float4 t = *reinterpret_cast<const float4*>(p);
+                acc[0] += t.x; acc[1] += t.y; acc[2] += t.z; acc[3] += t.w;
+            } else {
+                acc[0] += *p;
+            }
+        }
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) red[ty][tx][q] = acc[q];
+    __syncthreads();
+    if (ty == 0 && i < n)
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) {
+            Tp t = red[0][tx][q];
+#pragma unroll
+            for (int g = 1; g < 8; ++g) t += red[g][tx][q];
+            M[i + q] = t;
+        }
+}
+
 template <typename Tp>
 constexpr size_t select_smem(int64_t R) {
     return sizeof(Tp) * (size_t)R * (TO + 1) + 32 * sizeof(int);

@@ -59,14 +59,13 @@ int pass2_rb(const View& v, const Tp* X0, const Tp* X1, int64_t xr, int64_t xo, 
 template <typename Tp, int NC, bool FULL>
 int pass2_any(const View& v, const Tp* X0, const Tp* X1, int64_t xr, int64_t xo, double* dpart,
               int splits, int64_t s_per, int* status, cudaStream_t st) {
-    switch (rblock_for<Tp>(v.R)) {
-        case 32: return pass2_rb<Tp, 32, NC, FULL>(v, X0, X1, xr, xo, dpart, splits, s_per, status, st);
-        case 64: return pass2_rb<Tp, 64, NC, FULL>(v, X0, X1, xr, xo, dpart, splits, s_per, status, st);
-        default:
-            if constexpr (sizeof(Tp) == 4)
-                return pass2_rb<Tp, 128, NC, FULL>(v, X0, X1, xr, xo, dpart, splits, s_per, status, st);
-            return DNA_ERR_UNSUPPORTED;
-    }
+    // float32 at ranks up to f2::MAX_R runs in f32_pass.cuh
+    if constexpr (sizeof(Tp) == 4)
+        return pass2_rb<Tp, 128, NC, FULL>(v, X0, X1, xr, xo, dpart, splits, s_per, status, st);
+    else if (rblock_for<Tp>(v.R) == 32)
+        return pass2_rb<Tp, 32, NC, FULL>(v, X0, X1, xr, xo, dpart, splits, s_per, status, st);
+    else
+        return pass2_rb<Tp, 64, NC, FULL>(v, X0, X1, xr, xo, dpart, splits, s_per, status, st);
 }
 
 template <typename Tp, int RB>
@@ -142,7 +141,10 @@ int Simt<Tp>::rescale(const View& v, const double* f, cudaStream_t st) {
 
 template <typename Tp>
 int Simt<Tp>::pass1(const View& v, Tp* A, Tp* B, int splits, int64_t s_per, bool with_b,
-                    int* status, cudaStream_t st, double* dcur) {
+                    int* status, cudaStream_t st, double* dcur, bool ascending) {
+    if constexpr (sizeof(Tp) == 4)
+        if (v.R <= f2::MAX_R && !dcur)
+            return f2::pass1(v, A, B, splits, s_per, with_b, ascending, status, st);
     switch (simt::rblock_for<Tp>(v.R)) {
         case 32: return simt::pass1_rb<Tp, 32>(v, A, B, splits, s_per, with_b, status, st, dcur);
         case 64: return simt::pass1_rb<Tp, 64>(v, A, B, splits, s_per, with_b, status, st, dcur);
@@ -170,12 +172,16 @@ int Simt<Tp>::mu_apply(const View& v, const double* c, const Tp* A, int splits, 
 template <typename Tp>
 int Simt<Tp>::pass2(const View& v, const Tp* Xmu, const Tp* Xdna, double* dpart, int splits,
                     int64_t s_per, int* status, cudaStream_t st) {
+    if constexpr (sizeof(Tp) == 4)
+        if (v.R <= f2::MAX_R) return f2::pass2(v, Xmu, Xdna, dpart, splits, s_per, status, st);
     return simt::pass2_any<Tp, 2, false>(v, Xmu, Xdna, v.O, 1, dpart, splits, s_per, status, st);
 }
 
 template <typename Tp>
 int Simt<Tp>::pass2_one(const View& v, const Tp* X, double* dpart, int splits, int64_t s_per,
                         int* status, cudaStream_t st) {
+    if constexpr (sizeof(Tp) == 4)
+        if (v.R <= f2::MAX_R) return f2::pass2_one(v, X, dpart, splits, s_per, status, st);
     return simt::pass2_any<Tp, 1, false>(v, X, X, v.O, 1, dpart, splits, s_per, status, st);
 }
 
@@ -190,6 +196,8 @@ int Simt<Tp>::select(const View& v, const Tp* Xmu, const Tp* Xdna, const double*
 template <typename Tp>
 int Simt<Tp>::kl_columns(const View& v, double* dpart, int splits, int64_t s_per, int* status,
                          cudaStream_t st) {
+    if constexpr (sizeof(Tp) == 4)
+        if (v.R <= f2::MAX_R) return f2::kl_columns(v, dpart, splits, s_per, status, st);
     const Tp* X = static_cast<const Tp*>(v.X);
     return simt::pass2_any<Tp, 1, true>(v, X, X, v.xr, v.xo, dpart, splits, s_per, status, st);
 }
@@ -365,6 +373,18 @@ template <typename Tp>
 int Simt<Tp>::split_sum(Tp* A, Tp* B, int64_t R, int64_t O, int splits, cudaStream_t st) {
     if (splits <= 1) return DNA_OK;
     const int64_t n = R * O;
+    // above four splits the loads of one thread would be rounds of dependent latency
+    if (splits > 4) {
+        const bool vec = sizeof(Tp) == 4 && n % 4 == 0;
+        const dim3 grid((unsigned)((n / (vec ? 4 : 1) + 31) / 32), B ? 2 : 1);
+        if constexpr (sizeof(Tp) == 4)
+            if (vec) {
+                glue::k_split_sum_par<Tp, 4><<<grid, dim3(32, 8), 0, st>>>(A, B, n, splits);
+                return simt::launch_status();
+            }
+        glue::k_split_sum_par<Tp, 1><<<grid, dim3(32, 8), 0, st>>>(A, B, n, splits);
+        return simt::launch_status();
+    }
     const int64_t work = (sizeof(Tp) == 4 && n % 4 == 0) ? n / 4 : n;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 8));
     glue::k_split_sum<Tp><<<(unsigned)blocks, 256, 0, st>>>(A, B, n, splits);
@@ -480,13 +500,10 @@ int Simt<Tp>::pass1_blocks_per_sm(int64_t R) {
 
 template <typename Tp>
 int Simt<Tp>::pass2_blocks_per_sm(int64_t R) {
-    switch (simt::rblock_for<Tp>(R)) {
-        case 32: return simt::occupancy_pass2<Tp, 32>();
-        case 64: return simt::occupancy_pass2<Tp, 64>();
-        default:
-            if constexpr (sizeof(Tp) == 4) return simt::occupancy_pass2<Tp, 128>();
-            return 1;
-    }
+    if constexpr (sizeof(Tp) == 4)
+        return simt::occupancy_pass2<Tp, 128>();
+    else
+        return R <= 32 ? simt::occupancy_pass2<Tp, 32>() : simt::occupancy_pass2<Tp, 64>();
 }
 
 template <typename Tp> int Simt<Tp>::chunk() { return simt::SB; }
