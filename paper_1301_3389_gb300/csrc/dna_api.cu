@@ -731,13 +731,14 @@ int step_core(dna_ctx* c, int w, bool mu_only, bool prepared, int stop) {
     int slots = sp2;
     if (stop <= STOP_PASS2) {
         // split partials over many columns: one streaming pass sums them into split 0 first
-        // (in the candidates kernel each further split is another round of dependent loads;
-        // the sums are the same, ascending split order either way)
+        // (in the candidates kernel each further split is another round of dependent loads);
+        // the tensor-core forms keep the ascending order of splits, since bf16 operands make
+        // a selection near a tie depend on the last bit
         const int parts = stop == STOP_PASS2 ? 1 : sp1;
         const bool presum = parts > 4 || ((int64_t)parts * v.O >= 32768 && parts > 1);
         e = phase(c, DNA_PHASE_CANDIDATES, presum ? 2 : 1, [&] {
             if (presum)
-                if (int r = S::split_sum(A, B, c->R, v.O, parts, st)) return r;
+                if (int r = S::split_sum(A, B, c->R, v.O, parts, st, tc)) return r;
             return S::cand_fused(v, c->c, A, B, presum ? 1 : parts, Xmu, Xdna, c->o.eps,
                                  c->o.alpha, tc ? c->Xmk : nullptr, tc ? c->Xdk : nullptr, c->rp,
                                  c->pad_o[w], c->plane, st);
@@ -1034,7 +1035,7 @@ int shard_W_pass1(dna_ctx* c, const double* hsum, void* AB) {
     const int sp1 = c->tc ? c->tsp1[1] : c->sp1[1];
     Tp* A = static_cast<Tp*>(c->Apart);
     Tp* B = static_cast<Tp*>(c->Bpart);
-    if (int e = S::split_sum(A, B, c->R, c->N, sp1, c->stream)) return e;
+    if (int e = S::split_sum(A, B, c->R, c->N, sp1, c->stream, c->tc)) return e;
     const size_t n = sizeof(Tp) * (size_t)(c->R * c->N);
     if (int e = d2d(AB, A, n, c->stream)) return e;
     return d2d(static_cast<char*>(AB) + n, B, n, c->stream);
@@ -1048,7 +1049,7 @@ int shard_W_pass2(dna_ctx* c, const void* AB, double* cost) {
     if (int e = step_core<Tp>(c, 1, false, true, STOP_PASS2)) return e;
     const int sp2 = c->tc ? c->tsp2[1] : c->sp2[1];
     // the cost slots [sp2][2][N] summed into slot 0 (float64, ascending slot order)
-    if (int e = dna::Simt<double>::split_sum(c->dpart, nullptr, 1, 2 * c->N, sp2, c->stream))
+    if (int e = dna::Simt<double>::split_sum(c->dpart, nullptr, 1, 2 * c->N, sp2, c->stream, true))
         return e;
     return d2d(cost, c->dpart, sizeof(double) * 2 * c->N, c->stream);
 }

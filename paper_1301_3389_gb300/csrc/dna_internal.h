@@ -118,8 +118,10 @@ template <typename Tp> struct Simt {
                           int splits, Tp* Xmu, Tp* Xdna, double eps, double alpha, void* Xmk,
                           void* Xdk, int64_t rp, int64_t O_pad, int64_t plane,
                           cudaStream_t st);
-    // A[0] = sum over the splits of A[sp] (and B, if given), each [R][O]: ascending order.
-    static int split_sum(Tp* A, Tp* B, int64_t R, int64_t O, int splits, cudaStream_t st);
+    // A[0] = sum over the splits of A[sp] (and B, if given), each [R][O]: in ascending order,
+    // or (ascending = false, more than four splits) as eight ranges of splits
+    static int split_sum(Tp* A, Tp* B, int64_t R, int64_t O, int splits, cudaStream_t st,
+                         bool ascending);
     // cand_fused keeps a thread's candidates in registers and sums the split partials as
     // they stream in (no split_sum pass needed)
     static bool cand_in_registers(int64_t R);

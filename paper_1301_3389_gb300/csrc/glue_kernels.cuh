@@ -341,37 +341,24 @@ __global__ void __launch_bounds__(512) k_cand_reg(View v, const double* __restri
 // A[0][i] = A[0][i] + A[1][i] + ... + A[splits-1][i] (ascending, the order the candidates
 // kernel uses, so results are unchanged), and the same for B (may be null): the split
 // partials of pass 1 streamed once with wide loads before the candidates read them.
-template <typename Tp>
+// blockIdx.y picks A or B; up to eight splits' loads of a thread are in flight.
+template <typename Tp, int VEC>
 __global__ void __launch_bounds__(256) k_split_sum(Tp* __restrict__ A, Tp* __restrict__ B,
                                                    int64_t n, int splits) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    if constexpr (sizeof(Tp) == 4) {
-        if (n % 4 == 0) {   // float4 path (slots are 16-byte aligned when n % 4 == 0)
-            const int64_t n4 = n / 4;
-            for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-#pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    float4* M = reinterpret_cast<float4*>(m ? B : A);
-                    if (!M) continue;
-                    float4 acc = M[i];
-#pragma unroll 4
-                    for (int sp = 1; sp < splits; ++sp) {
-                        const float4 t = M[(int64_t)sp * n4 + i];
-                        acc.x += t.x; acc.y += t.y; acc.z += t.z; acc.w += t.w;
-                    }
-                    M[i] = acc;
-                }
+    Tp* M = blockIdx.y ? B : A;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * VEC;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * VEC; i < n; i += stride) {
+        if constexpr (VEC == 4) {   // slots are 16-byte aligned when n % 4 == 0
+            float4 acc = *reinterpret_cast<const float4*>(M + i);
+#pragma unroll 8
+            for (int sp = 1; sp < splits; ++sp) {
+                const float4 t = *reinterpret_cast<const float4*>(M + (int64_t)sp * n + i);
+                acc.x += t.x; acc.y += t.y; acc.z += t.z; acc.w += t.w;
             }
-            return;
-        }
-    }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-#pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            Tp* M = m ? B : A;
-            if (!M) continue;
+            *reinterpret_cast<float4*>(M + i) = acc;
+        } else {
             Tp acc = M[i];
-#pragma unroll 4
+#pragma unroll 8
             for (int sp = 1; sp < splits; ++sp) acc += M[(int64_t)sp * n + i];
             M[i] = acc;
         }

@@ -19,6 +19,7 @@
 
 #include "dna.h"
 #include "dna_internal.h"
+#include "f32_pass.cuh"
 #include "glue_kernels.cuh"
 #include "simt_kernels.cuh"
 
@@ -39,48 +40,57 @@ struct GProb {
     int64_t per1[2], per2[2];  // rows of s per split
     int sp1[2], sp2[2];
     int nslot[2];              // cost slots per column that the selection adds
-    int rclass;                // rank class: 0: R <= 16, 1: R <= 32, 2: R <= 64
 };
 
 struct GTile {
     int32_t prob, a, b, pad;
 };
 
-constexpr int NCLASS = 3;   // r-blocks of 16, 32 and 64 (rank padding at most 2x past R = 8)
-constexpr int class_of_rb(int rb) { return rb == 16 ? 0 : rb == 32 ? 1 : 2; }
 constexpr int64_t MIN_SPLIT_ROWS = 256;   // smallest s-range per split (bounds the workspace)
 
-template <int RB, bool WITH_B>
-__global__ void __launch_bounds__(simt::NT, 2)
-    k_g_pass1(const GProb* __restrict__ P, const GTile* __restrict__ tl, int n, int w,
+// FP32 form, pass 1 of every problem: CTA b takes tile b (problem, o-block, split) with the
+// kernel body of its rank (multiples of 16 up to 64).  The tiles are listed longest first
+// and the hardware hands them to the SMs as they come free, so one launch serves all ranks
+// and only short tiles are left at its end.
+__global__ void __launch_bounds__(f2::NT, 2)
+    k_g_pass1(const GProb* __restrict__ P, const GTile* __restrict__ tl, int w,
               int* __restrict__ status) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    for (int t = blockIdx.x; t < n; t += gridDim.x) {
-        const GTile tt = tl[t];
-        const GProb& p = P[tt.prob];
-        const View v = p.v[w];
-        simt::pass1_tile<float, RB, WITH_B>(v, p.A, p.B, p.per1[w], status, tt.a, 0, tt.b, smem);
-        __syncthreads();
+    extern __shared__ __align__(16) float smem_g1[];
+    const GTile tt = tl[blockIdx.x];
+    const GProb& p = P[tt.prob];
+    const View v = p.v[w];
+    switch ((v.R + 15) / 16) {
+        case 1: f2::pass1_tile<1, true, f2::s_groups(1)>(v, p.A, p.B, p.per1[w], status, tt.a, tt.b, smem_g1); break;
+        case 2: f2::pass1_tile<2, true, f2::s_groups(2)>(v, p.A, p.B, p.per1[w], status, tt.a, tt.b, smem_g1); break;
+        case 3: f2::pass1_tile<3, true, f2::s_groups(3)>(v, p.A, p.B, p.per1[w], status, tt.a, tt.b, smem_g1); break;
+        default: f2::pass1_tile<4, true, f2::s_groups(4)>(v, p.A, p.B, p.per1[w], status, tt.a, tt.b, smem_g1);
     }
 }
 
-template <int RB, int NC, bool FULL>
-__global__ void __launch_bounds__(simt::NT, 2)
-    k_g_pass2(const GProb* __restrict__ P, const GTile* __restrict__ tl, int n, int w,
+// Pass 2 of every problem, or (FULL) d_KL's column sums, over tiles as above.
+template <int RPT, bool FULL>
+__device__ __forceinline__ void g_pass2(const GProb& p, const View& v, int w, const GTile& tt,
+                                        int* __restrict__ status, float* sm) {
+    const float* X = static_cast<const float*>(v.X);
+    if constexpr (FULL)
+        f2::pass2_tile<RPT, 1, true>(v, X, X, v.xr, v.xo, p.dpart, p.per2[w], status, tt.a, tt.b, sm);
+    else
+        f2::pass2_tile<RPT, 2, false>(v, p.Xmu, p.Xdna, v.O, 1, p.dpart, p.per2[w], status, tt.a, tt.b, sm);
+}
+
+template <bool FULL>
+__global__ void __launch_bounds__(f2::NT, 2)
+    k_g_pass2(const GProb* __restrict__ P, const GTile* __restrict__ tl, int w,
               int* __restrict__ status) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    for (int t = blockIdx.x; t < n; t += gridDim.x) {
-        const GTile tt = tl[t];
-        const GProb& p = P[tt.prob];
-        const View v = p.v[w];
-        if constexpr (FULL)
-            simt::pass2_tile<float, RB, 1, true>(v, static_cast<const float*>(v.X),
-                                                 static_cast<const float*>(v.X), v.xr, v.xo,
-                                                 p.dpart, p.per2[w], status, tt.a, tt.b, smem);
-        else
-            simt::pass2_tile<float, RB, NC, false>(v, p.Xmu, p.Xdna, v.O, 1, p.dpart, p.per2[w],
-                                                   status, tt.a, tt.b, smem);
-        __syncthreads();
+    extern __shared__ __align__(16) float smem_g2[];
+    const GTile tt = tl[blockIdx.x];
+    const GProb& p = P[tt.prob];
+    const View v = p.v[w];
+    switch ((v.R + 15) / 16) {
+        case 1: g_pass2<1, FULL>(p, v, w, tt, status, smem_g2); break;
+        case 2: g_pass2<2, FULL>(p, v, w, tt, status, smem_g2); break;
+        case 3: g_pass2<3, FULL>(p, v, w, tt, status, smem_g2); break;
+        default: g_pass2<4, FULL>(p, v, w, tt, status, smem_g2);
     }
 }
 
@@ -499,10 +509,9 @@ struct dna_group {
     GProb* dp = nullptr;
     double* kl_dev = nullptr;
     int* status = nullptr;
-    // tile lists [view][class] for the passes, [view] for the rest
-    TileList p1[2][dna::grp::NCLASS], p2[2][dna::grp::NCLASS], kl[dna::grp::NCLASS];
+    // tile lists [view]
+    TileList p1[2], p2[2], kl;
     TileList cand[2], sums_y[2], sums_x[2], resc[2];
-    int slots1[dna::grp::NCLASS] = {1, 1, 1}, slots2[dna::grp::NCLASS] = {1, 1, 1};
     int64_t split_rows = 1024;  // rows of s per split (autotuned)
     bool bound = false, use_graph = false;
     // BF16 form: the tensor-core passes
@@ -531,27 +540,16 @@ int set_smem(Kern k, size_t bytes) {
     return DNA_OK;
 }
 
-template <int RB>
-size_t p1_smem() { return simt::Pass1Cfg<float, RB>::smem; }
-template <int RB>
-size_t p2_smem() { return simt::Pass2Cfg<float, RB, 2>::smem; }
+constexpr size_t P1_SMEM = std::max(f2::Pass1<4, true, f2::s_groups(4)>::smem,
+                                    f2::Pass1<2, true, f2::s_groups(2)>::smem);
+constexpr size_t P2_SMEM = f2::Pass2<4, 2>::smem;
 
-template <int RB>
-int prep_class(dna_group* g, int cls) {
+int prep_passes() {
     using namespace dna::grp;
-    int e = set_smem(k_g_pass1<RB, true>, p1_smem<RB>());
-    e |= set_smem(k_g_pass1<RB, false>, p1_smem<RB>());
-    e |= set_smem(k_g_pass2<RB, 2, false>, p2_smem<RB>());
-    e |= set_smem(k_g_pass2<RB, 2, true>, p2_smem<RB>());
-    if (e) return DNA_ERR_CUDA;
-    int b1 = 1, b2 = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k_g_pass1<RB, true>, simt::NT, p1_smem<RB>());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, k_g_pass2<RB, 2, false>, simt::NT,
-                                                  p2_smem<RB>());
-    cudaGetLastError();
-    g->slots1[cls] = std::max(1, b1) * g->num_sms;
-    g->slots2[cls] = std::max(1, b2) * g->num_sms;
-    return DNA_OK;
+    int e = set_smem(k_g_pass1, P1_SMEM);
+    e |= set_smem(k_g_pass2<false>, P2_SMEM);
+    e |= set_smem(k_g_pass2<true>, P2_SMEM);
+    return e ? DNA_ERR_CUDA : DNA_OK;
 }
 
 void free_lists(dna_group* g) {
@@ -574,7 +572,7 @@ int upload(dna_group* g, const std::vector<GTile>& v, TileList* out) {
 // Split plan of every problem for rows-per-split `rows`, then all tile lists.
 int build_tiles(dna_group* g) {
     free_lists(g);
-    const int64_t ch = simt::SB, ob = simt::OB;
+    const int64_t ch = f2::SB, ob = f2::OB;
     for (int q = 0; q < g->count; ++q) {
         GProb& p = g->hp[q];
         for (int w = 0; w < 2; ++w) {
@@ -585,17 +583,18 @@ int build_tiles(dna_group* g) {
             p.sp1[w] = p.sp2[w] = (int)((S + per - 1) / per);
         }
     }
-    constexpr int NC = dna::grp::NCLASS;
-    std::vector<GTile> t1[2][NC], t2[2][NC], tk[NC], tc[2], ty[2], tx[2], tr[2];
+    std::vector<GTile> t1[2], t2[2], tk, tc[2], ty[2], tx[2], tr[2];
     for (int q = 0; q < g->count; ++q) {
         const GProb& p = g->hp[q];
         for (int w = 0; w < 2; ++w) {
             const View& v = p.v[w];
             const int64_t nob = (v.O + ob - 1) / ob;
-            for (int64_t b = 0; b < nob; ++b)
-                for (int s = 0; s < p.sp1[w]; ++s) t1[w][p.rclass].push_back({q, (int)b, s, 0});
-            for (int64_t b = 0; b < nob; ++b)
-                for (int s = 0; s < p.sp2[w]; ++s) t2[w][p.rclass].push_back({q, (int)b, s, 0});
+            if (!g->tc) {   // the passes on the CUDA cores
+                for (int64_t b = 0; b < nob; ++b)
+                    for (int s = 0; s < p.sp1[w]; ++s) t1[w].push_back({q, (int)b, s, 0});
+                for (int64_t b = 0; b < nob; ++b)
+                    for (int s = 0; s < p.sp2[w]; ++s) t2[w].push_back({q, (int)b, s, 0});
+            }
             for (int64_t b = 0; b < (v.O + 31) / 32; ++b) tc[w].push_back({q, (int)b, 0, 0});
             // factor sums: blocks of 8 rows where the matrix is contiguous along i (the
             // long sums over T), else one tile per problem
@@ -607,8 +606,24 @@ int build_tiles(dna_group* g) {
         }
         const View& v = p.v[0];
         for (int64_t b = 0; b < (v.O + ob - 1) / ob; ++b)
-            for (int s = 0; s < p.sp2[0]; ++s) tk[p.rclass].push_back({q, (int)b, s, 0});
+            for (int s = 0; s < p.sp2[0]; ++s) tk.push_back({q, (int)b, s, 0});
     }
+    // longest tiles first, by chunks x (16-rank groups + the element-wise part of a chunk)
+    auto longest_first = [&](std::vector<GTile>& t, int w, bool second) {
+        auto cost = [&](const GTile& x) {
+            const GProb& p = g->hp[x.prob];
+            const int64_t per = second ? p.per2[w] : p.per1[w];
+            const int64_t rows = std::min<int64_t>(per, p.v[w].S - (int64_t)x.b * per);
+            return (rows + ch - 1) / ch * ((p.v[w].R + 15) / 16 + 1);
+        };
+        std::stable_sort(t.begin(), t.end(),
+                         [&](const GTile& a, const GTile& b) { return cost(a) > cost(b); });
+    };
+    for (int w = 0; w < 2; ++w) {
+        longest_first(t1[w], w, false);
+        longest_first(t2[w], w, true);
+    }
+    longest_first(tk, 0, true);
     std::vector<GTile> ti[2], tcb[2], tq1[2], tq2[2];
     for (int q = 0; q < g->count; ++q)
         for (int w = 0; w < 2; ++w) {
@@ -681,16 +696,14 @@ int build_tiles(dna_group* g) {
             e = DNA_ERR_CUDA;
     }
     for (int w = 0; w < 2; ++w) {
-        for (int k = 0; k < NC; ++k) {
-            e |= upload(g, t1[w][k], &g->p1[w][k]);
-            e |= upload(g, t2[w][k], &g->p2[w][k]);
-        }
+        e |= upload(g, t1[w], &g->p1[w]);
+        e |= upload(g, t2[w], &g->p2[w]);
         e |= upload(g, tc[w], &g->cand[w]);
         e |= upload(g, ty[w], &g->sums_y[w]);
         e |= upload(g, tx[w], &g->sums_x[w]);
         e |= upload(g, tr[w], &g->resc[w]);
     }
-    for (int k = 0; k < NC; ++k) e |= upload(g, tk[k], &g->kl[k]);
+    e |= upload(g, tk, &g->kl);
     if (e) return e;
     if (cudaMemcpy(g->dp, g->hp.data(), sizeof(GProb) * g->count, cudaMemcpyHostToDevice) !=
         cudaSuccess)
@@ -704,24 +717,43 @@ int build_tiles(dna_group* g) {
 
 int grid_for(int n, int slots) { return std::max(1, std::min(n, slots)); }
 
-template <int RB>
-int launch_p1(dna_group* g, const TileList& t, int w, bool with_b) {
-    using namespace dna::grp;
+// The tile sizes a group starts with.  FP32, rows of s per split: the most of 2048, 1024,
+// 512, 256 that still gives each view three tiles per SM (8 problems of the batched workload
+// take 316 us an iteration with 256 rows instead of 431 with 1024, 48 problems 1200 with any
+// of 512 to 2048).  BF16: 1024 rows, and pass-2 units for about one CTA per SM, 4 to 16 (32
+// problems: 16 units instead of 4, 128 problems: 16 instead of 8 are 5 % of the iteration).
+void default_tiles(dna_group* g) {
+    const int64_t ob = g->tc ? 128 : f2::OB;
+    auto tiles = [&](const std::vector<int64_t>& S, const std::vector<int64_t>& O, int64_t rows) {
+        int64_t n = 0;
+        for (int q = 0; q < g->count; ++q)
+            n += (O[q] + ob - 1) / ob * ((S[q] + rows - 1) / rows);
+        return n;
+    };
+    if (g->tc) {
+        const int64_t units = std::max(tiles(g->N, g->T, 128), tiles(g->T, g->N, 128));
+        int64_t per = 4;
+        while (per < 16 && 3 * per * (int64_t)g->num_sms <= 2 * units) per *= 2;
+        g->p2_units = per;
+        return;
+    }
+    int64_t rows = 2048;
+    while (rows > dna::grp::MIN_SPLIT_ROWS &&
+           std::min(tiles(g->N, g->T, rows), tiles(g->T, g->N, rows)) < 3 * (int64_t)g->num_sms)
+        rows /= 2;
+    g->split_rows = rows;
+}
+
+int launch_p1(dna_group* g, const TileList& t, int w) {
     if (!t.n) return DNA_OK;
-    const int grid = grid_for(t.n, g->slots1[dna::grp::class_of_rb(RB)]);
-    if (with_b)
-        k_g_pass1<RB, true><<<grid, simt::NT, p1_smem<RB>(), g->gs>>>(g->dp, t.d, t.n, w, g->status);
-    else
-        k_g_pass1<RB, false><<<grid, simt::NT, p1_smem<RB>(), g->gs>>>(g->dp, t.d, t.n, w, g->status);
+    dna::grp::k_g_pass1<<<t.n, f2::NT, P1_SMEM, g->gs>>>(g->dp, t.d, w, g->status);
     return after_launch();
 }
 
-template <int RB, bool FULL>
+template <bool FULL>
 int launch_p2(dna_group* g, const TileList& t, int w) {
-    using namespace dna::grp;
     if (!t.n) return DNA_OK;
-    const int grid = grid_for(t.n, g->slots2[dna::grp::class_of_rb(RB)]);
-    k_g_pass2<RB, 2, FULL><<<grid, simt::NT, p2_smem<RB>(), g->gs>>>(g->dp, t.d, t.n, w, g->status);
+    dna::grp::k_g_pass2<FULL><<<t.n, f2::NT, P2_SMEM, g->gs>>>(g->dp, t.d, w, g->status);
     return after_launch();
 }
 
@@ -774,13 +806,9 @@ int g_half(dna_group* g, int w, bool mu_only, bool ops_ready = false, bool fuse_
         }
         if (!e) e = dna::TcBf16::group_pass2(g->gv, g->tp2[w].d, g->tp2[w].n, w, g->status, g->gs);
     } else {
-        if (!e) e = launch_p1<16>(g, g->p1[w][0], w, true);
-        if (!e) e = launch_p1<32>(g, g->p1[w][1], w, true);
-        if (!e) e = launch_p1<64>(g, g->p1[w][2], w, true);
+        if (!e) e = launch_p1(g, g->p1[w], w);
         if (!e) e = launch_small(g, 3, g->cand[w], w);
-        if (!e) e = launch_p2<16, false>(g, g->p2[w][0], w);
-        if (!e) e = launch_p2<32, false>(g, g->p2[w][1], w);
-        if (!e) e = launch_p2<64, false>(g, g->p2[w][2], w);
+        if (!e) e = launch_p2<false>(g, g->p2[w], w);
     }
     if (!e) e = launch_small(g, 4, g->cand[w], w, w ? g->o.rho : g->o.lambda);
     if (e) return e;
@@ -883,9 +911,7 @@ int dna_group_create(int count, const int64_t* N, const int64_t* T, const int64_
         cudaEventCreateWithFlags(&g->ev_in, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&g->ev_out, cudaEventDisableTiming) != cudaSuccess)
         e = DNA_ERR_CUDA;
-    if (!e) e = prep_class<16>(g, 0);
-    if (!e) e = prep_class<32>(g, 1);
-    if (!e) e = prep_class<64>(g, 2);
+    if (!e) e = prep_passes();
     if (!e && tc) e = dna::TcBf16::group_prepare();
     // arena: per problem Vt, V sums, factor sums, A/B partials (worst split count), candidates,
     // cost partials, final costs, choices; in the BF16 form also an aligned copy of V and
@@ -980,7 +1006,6 @@ int dna_group_create(int count, const int64_t* N, const int64_t* T, const int64_
             }
             g->tcb.push_back(tb);
         }
-        p.rclass = r <= 16 ? 0 : r <= 32 ? 1 : 2;
         // views without the caller's buffers yet
         View& vh = p.v[0];
         vh.S = n; vh.O = t; vh.R = r; vh.vsum = colsum;
@@ -988,6 +1013,7 @@ int dna_group_create(int count, const int64_t* N, const int64_t* T, const int64_
         vw.S = t; vw.O = n; vw.R = r; vw.V = Vt; vw.vs = ldvt; vw.vsum = rowsum;
     }
     if (tc) g->hgv.resize(2 * (size_t)count);
+    default_tiles(g);
     *out = g;
     return DNA_OK;
 }
@@ -1196,9 +1222,7 @@ int dna_group_kl(dna_group* g, double* out) {
     {
         Handoff h(g);
         if (h.err) return h.err;
-        e = launch_p2<16, true>(g, g->kl[0], 0);
-        if (!e) e = launch_p2<32, true>(g, g->kl[1], 0);
-        if (!e) e = launch_p2<64, true>(g, g->kl[2], 0);
+        e = launch_p2<true>(g, g->kl, 0);
         if (!e) {
             k_g_kl_reduce<<<std::min(g->count, 1024), 256, 0, g->gs>>>(g->dp, g->count, g->kl_dev);
             e = dna::after_launch();
@@ -1240,8 +1264,7 @@ int64_t dna_group_launches_per_iteration(dna_group* g) {
                      // rescale; dna_group_iterate writes the first H operands once per call)
             n += (g->tp1[w].n > 0) + (g->tp2[w].n > 0);
         else
-            for (int k = 0; k < dna::grp::NCLASS; ++k)
-                n += (g->p1[w][k].n > 0) + (g->p2[w][k].n > 0);
+            n += (g->p1[w].n > 0) + (g->p2[w].n > 0);
     }
     return n;
 }

@@ -370,24 +370,32 @@ template <typename Tp>
 bool Simt<Tp>::cand_in_registers(int64_t R) { return R <= (sizeof(Tp) == 8 ? 128 : 256); }
 
 template <typename Tp>
-int Simt<Tp>::split_sum(Tp* A, Tp* B, int64_t R, int64_t O, int splits, cudaStream_t st) {
+int Simt<Tp>::split_sum(Tp* A, Tp* B, int64_t R, int64_t O, int splits, cudaStream_t st,
+                        bool ascending) {
     if (splits <= 1) return DNA_OK;
     const int64_t n = R * O;
+    const int vec = sizeof(Tp) == 4 && n % 4 == 0 ? 4 : 1;
+    const int64_t work = n / vec;
+    const unsigned ab = B ? 2 : 1;
     // above four splits the loads of one thread would be rounds of dependent latency
-    if (splits > 4) {
-        const bool vec = sizeof(Tp) == 4 && n % 4 == 0;
-        const dim3 grid((unsigned)((n / (vec ? 4 : 1) + 31) / 32), B ? 2 : 1);
+    if (splits > 4 && !ascending) {
+        const dim3 grid((unsigned)((work + 31) / 32), ab);
         if constexpr (sizeof(Tp) == 4)
-            if (vec) {
+            if (vec == 4) {
                 glue::k_split_sum_par<Tp, 4><<<grid, dim3(32, 8), 0, st>>>(A, B, n, splits);
                 return simt::launch_status();
             }
         glue::k_split_sum_par<Tp, 1><<<grid, dim3(32, 8), 0, st>>>(A, B, n, splits);
         return simt::launch_status();
     }
-    const int64_t work = (sizeof(Tp) == 4 && n % 4 == 0) ? n / 4 : n;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 8));
-    glue::k_split_sum<Tp><<<(unsigned)blocks, 256, 0, st>>>(A, B, n, splits);
+    const dim3 grid((unsigned)blocks, ab);
+    if constexpr (sizeof(Tp) == 4)
+        if (vec == 4) {
+            glue::k_split_sum<Tp, 4><<<grid, 256, 0, st>>>(A, B, n, splits);
+            return simt::launch_status();
+        }
+    glue::k_split_sum<Tp, 1><<<grid, 256, 0, st>>>(A, B, n, splits);
     return simt::launch_status();
 }
 
