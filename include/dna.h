@@ -204,7 +204,7 @@ int dna_step_H_adjoint(dna_ctx* ctx, const void* Hk, const uint8_t* choice,
  * derivative in W, e.g. dna_kl_backward's dW) this is the gradient of the loss with
  * respect to W.  Vbar and Wbar may each be NULL (the other outputs are still written).
  * The first call with Wbar allocates the context's W-gradient workspace (at most
- * 32 x R x N values of the element type and ceil(T / 32) x R float64); later calls
+ * 32 x R x N values of the element type and (ceil(T / 32) + 1) x R float64); later calls
  * allocate nothing.  Same limits on R as dna_step_H_adjoint. Returns DNA_ERR_ALLOC if the
  * workspace cannot be allocated.
  * Asynchronous. */

@@ -59,6 +59,9 @@ struct dna_ctx {
     // within a split)
     int dsp1[2] = {1, 1};
     int64_t dper1[2] = {0, 0};
+    // float32 adjoint: splits of s, and runs of o-blocks (groups) that share a W partial
+    int asp = 1, agroups = 1;
+    int64_t aper = 0, aob = 1;
     // tensor-core (BF16) path
     bool tc = false;
     bool split = false;              // FP32 form on the tensor cores (hi + lo bf16 operands)
@@ -227,6 +230,31 @@ void plan_f2(int64_t S, int64_t nob, int sms, double chunk_us, double part_us, i
     *splits = (int)((S + *per - 1) / *per);
 }
 
+// Splits of s and groups of o-blocks of the float32 adjoint (f32_adjoint.cu), `slots` CTAs
+// at a time: a 64 x 64 tile takes about 3.2 us per 16 ranks and 1.5 us for the rest, an
+// o-block of a CTA 2 us to start; each split writes and reads R values per column, each
+// group R values per row.  At most 32 groups (the documented size of the W partials).
+void plan_adjoint(int64_t S, int64_t O, int64_t R, int slots, int* splits, int64_t* per,
+                  int* groups, int64_t* ob_per) {
+    const int64_t nch = (S + 63) / 64, nob = (O + 63) / 64;
+    const double tile = 3.2 * (double)((R + 15) / 16) + 1.5;
+    double best = 1e300;
+    int64_t bc = nch, bo = nob;
+    for (int64_t g = 1; g <= std::min<int64_t>(nob, 32); ++g)
+        for (int64_t sp = 1; sp <= std::min<int64_t>(nch, 32); ++sp) {
+            const int64_t op = (nob + g - 1) / g, cp = (nch + sp - 1) / sp;
+            const int64_t ctas = ((nob + op - 1) / op) * ((nch + cp - 1) / cp);
+            const double us = (double)((ctas + slots - 1) / slots) * (double)op *
+                                  ((double)cp * tile + 2.0) +
+                              8e-6 / 4.0 * (double)R * (double)(sp * O + g * S);
+            if (us < best) { best = us; bc = cp; bo = op; }
+        }
+    *per = bc * 64;
+    *splits = (int)((nch + bc - 1) / bc);
+    *ob_per = bo;
+    *groups = (int)((nob + bo - 1) / bo);
+}
+
 // Chunks of 128 that one pass-1 CTA of the split FP32 form accumulates in tensor memory
 // (1024 values of s: the accumulation error stays near 1e-6 relative).
 constexpr int64_t SPLIT_CHUNK = 128;
@@ -245,6 +273,9 @@ void plan_all(dna_ctx* c) {
     const int64_t nrb = (c->R + rb - 1) / rb;
     const int b1 = S::pass1_blocks_per_sm(c->R);
     const bool f2 = sizeof(Tp) == 4 && c->R <= dna::f2::MAX_R;   // the passes of f32_pass.cuh
+    if (f2 && !c->tc)
+        plan_adjoint(c->N, c->T, c->R, c->num_sms * (c->R <= 32 ? 2 : 1), &c->asp, &c->aper,
+                     &c->agroups, &c->aob);
     for (int w = 0; w < 2; ++w) {
         const int64_t Sdim = w ? c->T : c->N, Odim = w ? c->N : c->T;
         const int64_t nob = (Odim + ob - 1) / ob;
@@ -325,7 +356,7 @@ int alloc_workspace(dna_ctx* c) {
     for (int w = 0; w < 2; ++w) {
         const int64_t O = w ? N : T;
         ap = std::max<int64_t>(
-            ap, (int64_t)std::max(std::max(c->sp1[w], c->dsp1[w]), c->tsp1[w]) * R * O);
+            ap, (int64_t)std::max({c->sp1[w], c->dsp1[w], c->tsp1[w], w ? 1 : c->asp}) * R * O);
         dp = std::max<int64_t>(dp, (int64_t)std::max(c->sp2[w], c->tsp2[w]) * 2 * O);
     }
     c->ldvt = (N + 3) / 4 * 4;
@@ -613,26 +644,45 @@ int step_h_adjoint(dna_ctx* c, const Tp* Hk, const uint8_t* choice, const Tp* Hb
     View v = make_view(c, false);
     v.X = const_cast<Tp*>(Hk);
     cudaStream_t st = c->stream;
+    const int64_t cblocks = (c->T + 31) / 32;
     if (Wbar && !c->wg_part) {
-        // o split so that the s-blocks x splits fill the SMs (one CTA per SM)
-        plan_split(c->T, (c->N + 63) / 64, c->num_sms, 64, &c->wsp, &c->wper);
+        // float64: o split so that the s-blocks x splits fill the SMs (one CTA per SM)
+        if (sizeof(Tp) == 8) plan_split(c->T, (c->N + 63) / 64, c->num_sms, 64, &c->wsp, &c->wper);
+        else c->wsp = c->agroups;
         if (dmalloc(&c->wg_part, sizeof(Tp) * (size_t)c->wsp * (size_t)c->R * (size_t)c->N) ||
-            dmalloc(&c->wg_cpart, sizeof(double) * (size_t)((c->T + 31) / 32) * (size_t)c->R))
+            dmalloc(&c->wg_cpart, sizeof(double) * (size_t)(cblocks + 1) * (size_t)c->R))
             return DNA_ERR_ALLOC;
     }
     Tp* A = static_cast<Tp*>(c->Apart);
     Tp* B = static_cast<Tp*>(c->Bpart);
     Tp* Abar = static_cast<Tp*>(c->Xmu);
     Tp* Bbar = static_cast<Tp*>(c->Xdna);
+    Tp* Wpart = static_cast<Tp*>(c->wg_part);
+    double* cpart = Wbar ? c->wg_cpart : nullptr;
     int e = S::factor_sums_y(v, c->o.lambda, c->c, c->fwork, st);
     if (!e) e = S::pass1(v, A, B, c->dsp1[0], c->dper1[0], true, c->status, st, nullptr, true);
+    if (!e) e = S::split_sum(A, B, c->R, c->T, c->dsp1[0], st, true);
     if (!e)
-        e = S::adjoint_h(v, c->c, A, B, c->dsp1[0], choice, Hbar_next, Hbar_out, Abar, Bbar,
-                         c->dpart, A, c->dsp1[0], c->dper1[0], Vbar, c->T, c->o.eps, c->o.alpha,
-                         c->status, st, Wbar ? c->wg_cpart : nullptr);
-    if (!e && Wbar)
-        e = S::adjoint_w(v, Abar, Bbar, c->wg_cpart, static_cast<Tp*>(c->wg_part), c->wsp,
-                         c->wper, Wbar, c->status, st);
+        e = S::adjoint_elem(v, c->c, A, B, choice, Hbar_next, Hbar_out, Abar, Bbar, c->dpart,
+                            c->o.eps, c->o.alpha, st, cpart);
+    if (e) return e;
+    // A and B are used: A holds the partial sums of Hbar from here
+    if constexpr (sizeof(Tp) == 4) {
+        e = dna::f2::adjoint(v, Abar, Bbar, c->dpart, A, c->asp, c->aper, Vbar, c->T,
+                             Wbar ? Wpart : nullptr, c->agroups, c->aob, c->status, st);
+        if (!e) e = S::adjoint_add(v, A, c->asp, Hbar_out, st);
+        if (!e && Wbar) {
+            double* csum = cpart + cblocks * c->R;
+            e = S::raw_sums(cpart, cblocks, c->R, csum, st);
+            if (!e) e = dna::f2::wgrad_add(Wpart, c->agroups, csum, c->N, c->R, Wbar, st);
+        }
+    } else {
+        e = S::adjoint_h(v, Abar, Bbar, c->dpart, A, c->dsp1[0], c->dper1[0], Vbar, c->T,
+                         c->status, st);
+        if (!e) e = S::adjoint_add(v, A, c->dsp1[0], Hbar_out, st);
+        if (!e && Wbar)
+            e = S::adjoint_w(v, Abar, Bbar, cpart, Wpart, c->wsp, c->wper, Wbar, c->status, st);
+    }
     return e;
 }
 

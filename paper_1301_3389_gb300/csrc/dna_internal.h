@@ -98,15 +98,20 @@ template <typename Tp> struct Simt {
     static int grad_v(const View& v, double scale, Tp* dV, int64_t ldd, int* status,
                       cudaStream_t st);
     // adjoint of one H step (see k_adj_elem / k_adj_gemm): Hbar0 = dL/dH_k given
-    // Hbar1 = dL/dH_{k+1}; Vbar += dL/dV (Vbar may be null).  Uses A, B (pass 1 of H_k) and
-    // the column choices.  With cpart ([ceil(O / 32)][R] float64) also the column-sum part
-    // of dL/dW, per block of 32 columns.
-    static int adjoint_h(const View& v, const double* c, const Tp* Apart, const Tp* Bpart,
-                         int splits1, const uint8_t* choice, const Tp* Hbar1, Tp* Hbar0,
-                         Tp* Abar, Tp* Bbar, double* vs, Tp* Hpart, int splits2, int64_t s_per2,
-                         Tp* Vbar, int64_t ldvb, double eps, double alpha, int* status,
-                         cudaStream_t st, double* cpart = nullptr);
-    // after adjoint_h (its Abar, Bbar, cpart): Wbar += dL/dW of the step (k_adj_wgrad),
+    // Hbar1 = dL/dH_{k+1}; Vbar += dL/dV (Vbar may be null).  adjoint_elem: from A, B (pass 1
+    // of H_k) and the column choices the direct part of Hbar0, Abar, Bbar and vs; with cpart
+    // ([ceil(O / 32)][R] float64) also the column-sum part of dL/dW, per block of 32 columns.
+    // adjoint_h (float64): the GEMM-shaped part; adjoint_add: Hbar0 += sum of Hpart.
+    static int adjoint_elem(const View& v, const double* c, const Tp* A, const Tp* B,
+                            const uint8_t* choice, const Tp* Hbar1, Tp* Hbar0, Tp* Abar,
+                            Tp* Bbar, double* vs, double eps, double alpha, cudaStream_t st,
+                            double* cpart);
+    static int adjoint_h(const View& v, const Tp* Abar, const Tp* Bbar, const double* vs,
+                         Tp* Hpart, int splits, int64_t s_per, Tp* Vbar, int64_t ldvb,
+                         int* status, cudaStream_t st);
+    static int adjoint_add(const View& v, const Tp* Hpart, int splits, Tp* Hbar0,
+                           cudaStream_t st);
+    // float64, after adjoint_h (its Abar, Bbar, cpart): Wbar += dL/dW of the step (k_adj_wgrad),
     // through Wpart [wsplits][R][S], o split in ranges of o_per (a multiple of 64)
     static int adjoint_w(const View& v, const Tp* Abar, const Tp* Bbar, const double* cpart,
                          Tp* Wpart, int wsplits, int64_t o_per, Tp* Wbar, int* status,
@@ -195,6 +200,14 @@ int pass2_one(const View& v, const float* X, double* dpart, int splits, int64_t 
               int* status, cudaStream_t st);
 int kl_columns(const View& v, double* dpart, int splits, int64_t s_per, int* status,
                cudaStream_t st);
+// the adjoint's GEMM-shaped part (f32_adjoint.cu): Hpart [splits][R][O], Vbar += (may be
+// null) and, with Wpart [groups][S][R], the o-blocks of 64 taken in `groups` runs of ob_per
+int adjoint(const View& v, const float* Abar, const float* Bbar, const double* vs, float* Hpart,
+            int splits, int64_t s_per, float* Vbar, int64_t ldvb, float* Wpart, int groups,
+            int64_t ob_per, int* status, cudaStream_t st);
+// Wbar (S x R) += the groups' Wpart and csum_r in every row
+int wgrad_add(const float* Wpart, int groups, const double* csum, int64_t S, int64_t R,
+              float* Wbar, cudaStream_t st);
 }  // namespace f2
 
 // Tensor-core (tcgen05) operands of one half-step, bf16, zero-padded:

@@ -210,9 +210,23 @@ __device__ __forceinline__ void z_tile(const float* __restrict__ Ys, const float
     }
 }
 
-// The four v(s, o + j) of a thread's row by cp.async: 16 bytes at once where V's rows allow.
+// Whether four neighbouring v(s, o .. o + 3), o a multiple of 4, are one aligned 16-byte word
+// inside a row of V.
 __device__ __forceinline__ bool v_wide(const View& v) {
     return ((v.vs | v.O) & 3) == 0 && (reinterpret_cast<uintptr_t>(v.V) & 15) == 0;
+}
+// v(s, o .. o + 3), zeros where s >= s_end or past the last column
+__device__ __forceinline__ void load_v(const View& v, const float* __restrict__ V, bool wide,
+                                       int64_t s, int64_t s_end, int64_t o, float (&x)[4]) {
+    const float* p = V + s * v.vs + o;
+    if (wide) {
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s < s_end && o < v.O) t = __ldg(reinterpret_cast<const float4*>(p));
+        x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = s < s_end && o + j < v.O ? __ldg(p + j) : 0.f;
+    }
 }
 
 // Rank 16 RPT as SG groups of s x rows: each thread owns NR = RPT SG rows r in NP pairs
@@ -495,19 +509,8 @@ __device__ __forceinline__ void pass2_tile(const View& v, const float* __restric
         }
         float vv[4][4];   // in flight behind the z FMAs
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int64_t s = s0 + zp.sl + 16 * i, o = o0 + 4 * zp.ol;
-            const float* vp = V + s * v.vs + o;
-            if (wide) {
-                float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (s < s_end && o < v.O) t = __ldg(reinterpret_cast<const float4*>(vp));
-                vv[i][0] = t.x; vv[i][1] = t.y; vv[i][2] = t.z; vv[i][3] = t.w;
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    vv[i][j] = s < s_end && o + j < v.O ? __ldg(vp + j) : 0.f;
-            }
-        }
+        for (int i = 0; i < 4; ++i)
+            load_v(v, V, wide, s0 + zp.sl + 16 * i, s_end, o0 + 4 * zp.ol, vv[i]);
         cp_wait<0>();
         __syncthreads();
         if (ST == 2 && c + 1 < nch) {

@@ -388,32 +388,52 @@ __device__ __forceinline__ void candidates_tile(const View& v, const double* __r
     const bool live = o < v.O;
     const Tp* __restrict__ X = static_cast<const Tp*>(v.X);
     Tp den = Tp(0);   // this thread's R / 8 terms of the eq. 10 denominator
+    constexpr int U = 8;   // values of r whose loads are issued together
     if (live) {
-        for (int64_t r = ty; r < v.R; r += 8) {
-            Tp ra = Tp(0), rb = Tp(0);
+        for (int64_t r0 = ty; r0 < v.R; r0 += 8 * U) {
+            Tp ra[U], rb[U], xv[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t r = r0 + 8 * u;
+                ra[u] = Tp(0);
+                rb[u] = Tp(0);
+                xv[u] = r < v.R ? X[r * v.xr + o * v.xo] : Tp(0);
+            }
             for (int sp = 0; sp < splits; ++sp) {
-                ra += Apart[((int64_t)sp * v.R + r) * v.O + o];
-                rb += Bpart[((int64_t)sp * v.R + r) * v.O + o];
+                Tp a0[U], b0[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t r = r0 + 8 * u, at = ((int64_t)sp * v.R + r) * v.O + o;
+                    a0[u] = r < v.R ? Apart[at] : Tp(0);
+                    b0[u] = r < v.R ? Bpart[at] : Tp(0);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) { ra[u] += a0[u]; rb[u] += b0[u]; }
             }
-            const Tp ic = ics[r];
-            const Tp a = ra * ic - Tp(1);         // eq. 7
-            const Tp b = rb * ic;                 // eq. 14
-            const Tp x = X[r * v.xr + o * v.xo];
-            // eq. 11 (step 6) as x (W^t q)_r / c_r: no cancellation where 1 + a is small
-            const Tp xmu = x * (ra * ic);
-            Tp xd;
-            if (a < Tp(0)) {                      // eq. 15 with the eps floor on the gain
-                const Tp xb = x * b;
-                const Tp g = dev_div(xb, xb - a);
-                xd = x * (g > eps ? g : eps);
-            } else {                              // eq. 17, gain capped at 1 + alpha
-                const Tp st = b > Tp(0) ? dev_div(a, b) : Tp(0);
-                const Tp cap = alpha * x;
-                xd = x + (st < cap ? st : cap);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t r = r0 + 8 * u;
+                if (r >= v.R) break;
+                const Tp ic = ics[r];
+                const Tp a = ra[u] * ic - Tp(1);      // eq. 7
+                const Tp b = rb[u] * ic;              // eq. 14
+                const Tp x = xv[u];
+                // eq. 11 (step 6) as x (W^t q)_r / c_r: no cancellation where 1 + a is small
+                const Tp xmu = x * (ra[u] * ic);
+                Tp xd;
+                if (a < Tp(0)) {                      // eq. 15 with the eps floor on the gain
+                    const Tp xb = x * b;
+                    const Tp g = dev_div(xb, xb - a);
+                    xd = x * (g > eps ? g : eps);
+                } else {                              // eq. 17, gain capped at 1 + alpha
+                    const Tp st = b > Tp(0) ? dev_div(a, b) : Tp(0);
+                    const Tp cap = alpha * x;
+                    xd = x + (st < cap ? st : cap);
+                }
+                Xmu[r * v.O + o] = xmu;
+                Xdna[r * v.O + o] = xd;
+                den += cs[r] * xd;
             }
-            Xmu[r * v.O + o] = xmu;
-            Xdna[r * v.O + o] = xd;
-            den += cs[r] * xd;
         }
     }
     red[ty][tx] = (double)den;
@@ -579,31 +599,44 @@ __global__ void __launch_bounds__(NT) k_grad_v(View v, double scale, Tp* __restr
 // (a = A / c - 1 and b = B / c, so da/dc = -(a + 1) / c and db/dc = -b / c; the eq. 10
 // denominator D = sum_l c_l g_l gives dD/dc_r = g_r, and dL/dD = -s hg / D^2 with
 // hg = sum_r hb'_r g_r), summed over the CTA's 32 columns into cpart[blockIdx.x][r].
-// CTA = 32 columns x 8 groups of r (one warp per group).
+// CTA = 32 columns x 8 groups of r (one warp per group); a thread's loads of up to 8 values
+// of r are issued together.
 template <typename Tp>
 __global__ void __launch_bounds__(256)
-    k_adj_elem(View v, const double* __restrict__ c, const Tp* __restrict__ Apart,
-               const Tp* __restrict__ Bpart, int splits, const uint8_t* __restrict__ choice,
+    k_adj_elem(View v, const double* __restrict__ c, const Tp* __restrict__ A,
+               const Tp* __restrict__ B, const uint8_t* __restrict__ choice,
                const Tp* __restrict__ Hbar1, Tp* __restrict__ Hbar0, Tp* __restrict__ Abar,
                Tp* __restrict__ Bbar, double* __restrict__ vs, Tp eps, Tp alpha,
                double* __restrict__ cpart) {
+    constexpr int U = 8;
     __shared__ double red[2][8][32];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int64_t o = (int64_t)blockIdx.x * 32 + tx;
     const bool live = o < v.O;
     const Tp* __restrict__ X = static_cast<const Tp*>(v.X);
     const bool newton = live && choice[o];
+    Tp ra[U], rb[U], xv[U], hv[U], cv[U];
+    auto fetch = [&](int64_t r0) {   // r = r0 + 8 u
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t r = r0 + 8 * u;
+            const bool in = live && r < v.R;
+            ra[u] = in ? A[r * v.O + o] : Tp(0);
+            rb[u] = in ? B[r * v.O + o] : Tp(0);
+            xv[u] = in ? X[r * v.xr + o * v.xo] : Tp(0);
+            hv[u] = in ? Hbar1[r * v.xr + o * v.xo] : Tp(0);
+            cv[u] = r < v.R ? (Tp)c[r] : Tp(1);
+        }
+    };
     // pass 1 over r: D = sum c g and sum hb' g (Newton columns)
     double dsum = 0.0, hg = 0.0;
-    if (newton) {
-        for (int64_t r = ty; r < v.R; r += 8) {
-            Tp ra = Tp(0), rb = Tp(0);
-            for (int sp = 0; sp < splits; ++sp) {
-                ra += Apart[((int64_t)sp * v.R + r) * v.O + o];
-                rb += Bpart[((int64_t)sp * v.R + r) * v.O + o];
-            }
-            const Tp cr = (Tp)c[r], x = X[r * v.xr + o * v.xo];
-            const Tp a = ra / cr - Tp(1), b = rb / cr;
+    for (int64_t r0 = ty; r0 < v.R; r0 += 8 * U) {
+        fetch(r0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (!newton || r0 + 8 * u >= v.R) continue;
+            const Tp cr = cv[u], x = xv[u];
+            const Tp a = ra[u] / cr - Tp(1), b = rb[u] / cr;
             Tp g;
             if (a < Tp(0)) {
                 const Tp xb = x * b, gain = xb / (xb - a);
@@ -613,7 +646,7 @@ __global__ void __launch_bounds__(256)
                 g = x + (st < cap ? st : cap);
             }
             dsum += (double)(cr * g);
-            hg += (double)(Hbar1[r * v.xr + o * v.xo] * g);
+            hg += (double)(hv[u] * g);
         }
     }
     red[0][ty][tx] = dsum;
@@ -626,59 +659,60 @@ __global__ void __launch_bounds__(256)
     const Tp f1 = (Tp)(renorm ? s_o / D : 1.0);            // d h' / d g (diagonal part)
     const Tp f2 = (Tp)(renorm ? s_o * HG / (D * D) : 0.0); // weight of the D coupling
     if (ty == 0 && live) vs[o] = (newton && renorm) ? HG / D : 0.0;
-    // the loop bound is uniform over the warp (one warp per ty), so every lane takes part
+    // the loop bounds are uniform over the warp (one warp per ty), so every lane takes part
     // in the cpart shuffle; lanes past the last column contribute 0
-    for (int64_t r = ty; r < v.R; r += 8) {
-        double cb = 0.0;
-        if (live) {
-            Tp ra = Tp(0), rb = Tp(0);
-            for (int sp = 0; sp < splits; ++sp) {
-                ra += Apart[((int64_t)sp * v.R + r) * v.O + o];
-                rb += Bpart[((int64_t)sp * v.R + r) * v.O + o];
-            }
-            const Tp cr = (Tp)c[r], x = X[r * v.xr + o * v.xo];
-            const Tp hb1 = Hbar1[r * v.xr + o * v.xo];
-            const Tp a = ra / cr - Tp(1), b = rb / cr;
-            Tp hx, ab = Tp(0), bb = Tp(0);   // dL/dh (direct), dL/da, dL/db
-            Tp g = Tp(0);                    // the Newton column's g_r (for dL/dc)
-            if (!newton) {                   // h' = h (1 + a)
-                hx = hb1 * (Tp(1) + a);
-                ab = hb1 * x;
-            } else {
-                const Tp gb = f1 * hb1 - cr * f2;   // dL/dg_r
-                if (a < Tp(0)) {
-                    const Tp xb = x * b, den = xb - a, gain = xb / den;
-                    if (gain > eps) {                // g = x^2 b / (x b - a)
-                        const Tp d2 = den * den;
-                        hx = gb * xb * (xb - Tp(2) * a) / d2;
-                        ab = gb * x * xb / d2;
-                        bb = -gb * a * x * x / d2;
-                        g = x * gain;
-                    } else {                         // floor: g = eps x
-                        hx = gb * eps;
-                        g = eps * x;
-                    }
+    for (int64_t r0 = ty; r0 < v.R; r0 += 8 * U) {
+        if (v.R > 8 * U) fetch(r0);   // else the values of pass 1 are still here
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t r = r0 + 8 * u;
+            if (r >= v.R) continue;
+            double cb = 0.0;
+            if (live) {
+                const Tp cr = cv[u], x = xv[u], hb1 = hv[u];
+                const Tp a = ra[u] / cr - Tp(1), b = rb[u] / cr;
+                Tp hx, ab = Tp(0), bb = Tp(0);   // dL/dh (direct), dL/da, dL/db
+                Tp g = Tp(0);                    // the Newton column's g_r (for dL/dc)
+                if (!newton) {                   // h' = h (1 + a)
+                    hx = hb1 * (Tp(1) + a);
+                    ab = hb1 * x;
                 } else {
-                    const Tp st = b > Tp(0) ? a / b : Tp(0), cap = alpha * x;
-                    if (st < cap) {                  // g = x + a / b
-                        hx = gb;
-                        if (b > Tp(0)) { ab = gb / b; bb = -gb * a / (b * b); }
-                        g = x + st;
-                    } else {                         // cap: g = (1 + alpha) x
-                        hx = gb * (Tp(1) + alpha);
-                        g = x + cap;
+                    const Tp gb = f1 * hb1 - cr * f2;   // dL/dg_r
+                    if (a < Tp(0)) {
+                        const Tp xb = x * b, den = xb - a, gain = xb / den;
+                        if (gain > eps) {                // g = x^2 b / (x b - a)
+                            const Tp d2 = den * den;
+                            hx = gb * xb * (xb - Tp(2) * a) / d2;
+                            ab = gb * x * xb / d2;
+                            bb = -gb * a * x * x / d2;
+                            g = x * gain;
+                        } else {                         // floor: g = eps x
+                            hx = gb * eps;
+                            g = eps * x;
+                        }
+                    } else {
+                        const Tp st = b > Tp(0) ? a / b : Tp(0), cap = alpha * x;
+                        if (st < cap) {                  // g = x + a / b
+                            hx = gb;
+                            if (b > Tp(0)) { ab = gb / b; bb = -gb * a / (b * b); }
+                            g = x + st;
+                        } else {                         // cap: g = (1 + alpha) x
+                            hx = gb * (Tp(1) + alpha);
+                            g = x + cap;
+                        }
                     }
                 }
+                Hbar0[r * v.xr + o * v.xo] = hx;
+                Abar[r * v.O + o] = ab / cr;     // a = A / c - 1
+                Bbar[r * v.O + o] = bb / cr;     // b = B / c
+                cb = -(double)(ab * (a + Tp(1)) + bb * b) / (double)cr - (double)(f2 * g);
             }
-            Hbar0[r * v.xr + o * v.xo] = hx;
-            Abar[r * v.O + o] = ab / cr;     // a = A / c - 1
-            Bbar[r * v.O + o] = bb / cr;     // b = B / c
-            cb = -(double)(ab * (a + Tp(1)) + bb * b) / (double)cr - (double)(f2 * g);
-        }
-        if (cpart) {
+            if (cpart) {
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) cb += __shfl_xor_sync(0xffffffffu, cb, off);
-            if (tx == 0) cpart[(int64_t)blockIdx.x * v.R + r] = cb;
+                for (int off = 16; off > 0; off >>= 1)
+                    cb += __shfl_xor_sync(0xffffffffu, cb, off);
+                if (tx == 0) cpart[(int64_t)blockIdx.x * v.R + r] = cb;
+            }
         }
     }
 }

@@ -248,30 +248,33 @@ int adj_gemm_rb(const View& v, const Tp* Abar, const Tp* Bbar, const double* vs,
 }  // namespace simt
 
 template <typename Tp>
-int Simt<Tp>::adjoint_h(const View& v, const double* c, const Tp* Apart, const Tp* Bpart,
-                        int splits1, const uint8_t* choice, const Tp* Hbar1, Tp* Hbar0, Tp* Abar,
-                        Tp* Bbar, double* vs, Tp* Hpart, int splits2, int64_t s_per2, Tp* Vbar,
-                        int64_t ldvb, double eps, double alpha, int* status, cudaStream_t st,
-                        double* cpart) {
+int Simt<Tp>::adjoint_elem(const View& v, const double* c, const Tp* A, const Tp* B,
+                           const uint8_t* choice, const Tp* Hbar1, Tp* Hbar0, Tp* Abar, Tp* Bbar,
+                           double* vs, double eps, double alpha, cudaStream_t st, double* cpart) {
     simt::k_adj_elem<Tp><<<(unsigned)((v.O + 31) / 32), dim3(32, 8), 0, st>>>(
-        v, c, Apart, Bpart, splits1, choice, Hbar1, Hbar0, Abar, Bbar, vs, (Tp)eps, (Tp)alpha,
-        cpart);
-    if (simt::launch_status()) return DNA_ERR_CUDA;
-    int e;
-    switch (simt::rblock_for<Tp>(v.R)) {
-        case 32: e = simt::adj_gemm_rb<Tp, 32>(v, Abar, Bbar, vs, Hpart, splits2, s_per2, Vbar, ldvb, status, st); break;
-        case 64: e = simt::adj_gemm_rb<Tp, 64>(v, Abar, Bbar, vs, Hpart, splits2, s_per2, Vbar, ldvb, status, st); break;
-        default:
-            if constexpr (sizeof(Tp) == 4) {
-                if (v.R <= 128) {
-                    e = simt::adj_gemm_rb<Tp, 128>(v, Abar, Bbar, vs, Hpart, splits2, s_per2, Vbar, ldvb, status, st);
-                    break;
-                }
-            }
-            return DNA_ERR_UNSUPPORTED;
-    }
-    if (e) return e;
-    simt::k_adj_combine<Tp><<<(unsigned)((v.O + 31) / 32), dim3(32, 8), 0, st>>>(v, Hpart, splits2,
+        v, c, A, B, choice, Hbar1, Hbar0, Abar, Bbar, vs, (Tp)eps, (Tp)alpha, cpart);
+    return simt::launch_status();
+}
+
+template <typename Tp>
+int Simt<Tp>::adjoint_h(const View& v, const Tp* Abar, const Tp* Bbar, const double* vs,
+                        Tp* Hpart, int splits, int64_t s_per, Tp* Vbar, int64_t ldvb, int* status,
+                        cudaStream_t st) {
+    if constexpr (sizeof(Tp) == 4)
+        return DNA_ERR_UNSUPPORTED;   // f32_adjoint.cu
+    else if (simt::rblock_for<Tp>(v.R) == 32)
+        return simt::adj_gemm_rb<Tp, 32>(v, Abar, Bbar, vs, Hpart, splits, s_per, Vbar, ldvb,
+                                         status, st);
+    else if (v.R <= 64)
+        return simt::adj_gemm_rb<Tp, 64>(v, Abar, Bbar, vs, Hpart, splits, s_per, Vbar, ldvb,
+                                         status, st);
+    return DNA_ERR_UNSUPPORTED;
+}
+
+template <typename Tp>
+int Simt<Tp>::adjoint_add(const View& v, const Tp* Hpart, int splits, Tp* Hbar0,
+                          cudaStream_t st) {
+    simt::k_adj_combine<Tp><<<(unsigned)((v.O + 31) / 32), dim3(32, 8), 0, st>>>(v, Hpart, splits,
                                                                                  Hbar0);
     return simt::launch_status();
 }
@@ -293,22 +296,19 @@ template <typename Tp>
 int Simt<Tp>::adjoint_w(const View& v, const Tp* Abar, const Tp* Bbar, const double* cpart,
                         Tp* Wpart, int wsplits, int64_t o_per, Tp* Wbar, int* status,
                         cudaStream_t st) {
-    if (v.R > 128 || o_per % simt::OB) return DNA_ERR_UNSUPPORTED;
-    int e;
-    switch (simt::rblock_for<Tp>(v.R)) {
-        case 32: e = simt::adj_wgrad_rb<Tp, 32>(v, Abar, Bbar, Wpart, wsplits, o_per, status, st); break;
-        case 64: e = simt::adj_wgrad_rb<Tp, 64>(v, Abar, Bbar, Wpart, wsplits, o_per, status, st); break;
-        default:
-            if constexpr (sizeof(Tp) == 4) {
-                e = simt::adj_wgrad_rb<Tp, 128>(v, Abar, Bbar, Wpart, wsplits, o_per, status, st);
-                break;
-            }
-            return DNA_ERR_UNSUPPORTED;
+    if constexpr (sizeof(Tp) == 4) {
+        return DNA_ERR_UNSUPPORTED;   // f32_adjoint.cu
+    } else {
+        if (v.R > 64 || o_per % simt::OB) return DNA_ERR_UNSUPPORTED;
+        const int e = v.R <= 32 ? simt::adj_wgrad_rb<Tp, 32>(v, Abar, Bbar, Wpart, wsplits, o_per,
+                                                             status, st)
+                                : simt::adj_wgrad_rb<Tp, 64>(v, Abar, Bbar, Wpart, wsplits, o_per,
+                                                             status, st);
+        if (e) return e;
+        simt::k_adj_wcombine<Tp><<<(unsigned)((v.S + 31) / 32), dim3(32, 8), 0, st>>>(
+            v, Wpart, wsplits, cpart, (v.O + 31) / 32, Wbar);
+        return simt::launch_status();
     }
-    if (e) return e;
-    simt::k_adj_wcombine<Tp><<<(unsigned)((v.S + 31) / 32), dim3(32, 8), 0, st>>>(
-        v, Wpart, wsplits, cpart, (v.O + 31) / 32, Wbar);
-    return simt::launch_status();
 }
 
 template <typename Tp>
