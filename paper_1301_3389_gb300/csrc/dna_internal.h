@@ -200,6 +200,8 @@ int pass2_one(const View& v, const float* X, double* dpart, int splits, int64_t 
               int* status, cudaStream_t st);
 int kl_columns(const View& v, double* dpart, int splits, int64_t s_per, int* status,
                cudaStream_t st);
+// dV(s, o) = scale log(v / z) where v > 0, else 0, leading dimension ldd
+int grad_v(const View& v, float scale, float* dV, int64_t ldd, int* status, cudaStream_t st);
 // the adjoint's GEMM-shaped part (f32_adjoint.cu): Hpart [splits][R][O], Vbar += (may be
 // null) and, with Wpart [groups][S][R], the o-blocks of 64 taken in `groups` runs of ob_per
 int adjoint(const View& v, const float* Abar, const float* Bbar, const double* vs, float* Hpart,

@@ -520,19 +520,35 @@ __global__ void __launch_bounds__(256) k_select(View v, const Tp* __restrict__ X
 
 // Gradient of eq. 1 with respect to the view's X from the raw pass-1 sums:
 // G(r, o) = scale * (c_r - sum over splits of Apart(r, o)) = scale * sum_s y(s, r)(1 - q(s, o)),
-// written to G[r * gr + o * go].  CTA = 32 values of o x 8 groups of r.
+// written to G[r * gr + o * go].  CTA = 32 values of o x 8 groups of r, 64 values of r.
 template <typename Tp>
 __global__ void __launch_bounds__(256) k_grad_x(View v, const double* __restrict__ c,
                                                 const Tp* __restrict__ Apart, int splits,
                                                 double scale, Tp* __restrict__ G, int64_t gr,
                                                 int64_t go) {
+    constexpr int U = 8;   // values of r whose loads are issued together
     const int64_t o = (int64_t)blockIdx.x * 32 + threadIdx.x;
     if (o >= v.O) return;
     const Tp sc = (Tp)scale;
-    for (int64_t r = threadIdx.y; r < v.R; r += 8) {
-        Tp a = Tp(0);
-        for (int sp = 0; sp < splits; ++sp) a += Apart[((int64_t)sp * v.R + r) * v.O + o];
-        G[r * gr + o * go] = sc * ((Tp)c[r] - a);
+    // r = 8 U blockIdx.y + threadIdx.y + 8 u
+    const int64_t r0 = (int64_t)blockIdx.y * 8 * U + threadIdx.y;
+    Tp a[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) a[u] = Tp(0);
+    for (int sp = 0; sp < splits; ++sp) {
+        Tp t[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t r = r0 + 8 * u;
+            t[u] = r < v.R ? Apart[((int64_t)sp * v.R + r) * v.O + o] : Tp(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u] += t[u];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int64_t r = r0 + 8 * u;
+        if (r < v.R) G[r * gr + o * go] = sc * ((Tp)c[r] - a[u]);
     }
 }
 

@@ -205,8 +205,8 @@ int Simt<Tp>::kl_columns(const View& v, double* dpart, int splits, int64_t s_per
 template <typename Tp>
 int Simt<Tp>::grad_x(const View& v, const double* c, const Tp* A, int splits, double scale,
                      Tp* G, int64_t gr, int64_t go, cudaStream_t st) {
-    simt::k_grad_x<Tp><<<(unsigned)((v.O + 31) / 32), dim3(32, 8), 0, st>>>(v, c, A, splits, scale,
-                                                                           G, gr, go);
+    const dim3 grid((unsigned)((v.O + 31) / 32), (unsigned)((v.R + 63) / 64));
+    simt::k_grad_x<Tp><<<grid, dim3(32, 8), 0, st>>>(v, c, A, splits, scale, G, gr, go);
     return simt::launch_status();
 }
 
@@ -225,12 +225,12 @@ int grad_v_rb(const View& v, double scale, Tp* dV, int64_t ldd, int* status, cud
 template <typename Tp>
 int Simt<Tp>::grad_v(const View& v, double scale, Tp* dV, int64_t ldd, int* status,
                      cudaStream_t st) {
-    switch (simt::rblock_for<Tp>(v.R)) {
-        case 32: return simt::grad_v_rb<Tp, 32>(v, scale, dV, ldd, status, st);
-        case 64: return simt::grad_v_rb<Tp, 64>(v, scale, dV, ldd, status, st);
-        default:
-            if constexpr (sizeof(Tp) == 4) return simt::grad_v_rb<Tp, 128>(v, scale, dV, ldd, status, st);
-            return DNA_ERR_UNSUPPORTED;
+    if constexpr (sizeof(Tp) == 4) {
+        if (v.R <= f2::MAX_R) return f2::grad_v(v, (float)scale, dV, ldd, status, st);
+        return simt::grad_v_rb<Tp, 128>(v, scale, dV, ldd, status, st);
+    } else {
+        return v.R <= 32 ? simt::grad_v_rb<Tp, 32>(v, scale, dV, ldd, status, st)
+                         : simt::grad_v_rb<Tp, 64>(v, scale, dV, ldd, status, st);
     }
 }
 
