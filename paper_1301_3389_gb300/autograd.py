@@ -15,6 +15,13 @@ Library contexts (their device workspace) are kept per thread and per (N, T, R, 
 device) and bound afresh to the call's tensors each time (``dna_bind`` prepares
 everything from them), so repeated calls allocate nothing; a call that fails destroys its
 context.  ``release_contexts()`` frees the calling thread's contexts.
+
+Work is queued on the current stream and not waited for (``KLDiv``'s forward waits for its
+number): a kept context carries an event after its last call, which a call on another
+stream waits for, and every tensor that the queued kernels use is recorded on their stream.
+Waiting at the end of each call left the GPU idle while Python prepared the next one
+(N=1024 T=4096 R=64: d_KL forward and backward 590 us -> 442, two unrolled steps forward
+and backward 1300 -> 925).
 """
 from __future__ import annotations
 
@@ -37,26 +44,36 @@ def _pool() -> dict:
 def release_contexts() -> None:
     """Destroy the library contexts this thread keeps for the autograd wrappers."""
     pool = _pool()
-    for ctx in pool.values():
+    for ctx, _, _ in pool.values():
         L.dna_destroy(ctx)
     pool.clear()
 
 
 class _Ctx:
-    """A pooled context bound to (V, W, H) for the duration of a ``with`` block."""
+    """A pooled context bound to (V, W, H) for the duration of a ``with`` block, on the
+    current stream; ``others`` are further tensors that the block's calls use."""
 
-    def __init__(self, V, W, H):
+    def __init__(self, V, W, H, *others):
         N, T = V.shape
         R = W.shape[1]
         dtype = L.DNA_F64 if V.dtype == torch.float64 else L.DNA_F32
         self.key = (N, T, R, dtype, V.device.index)
-        pool = _pool()
-        ctx = pool.pop(self.key, None)   # taken out while in use (re-entrant calls get their own)
+        if torch.cuda.is_current_stream_capturing():
+            # a captured call would replay on a workspace that later calls use too
+            raise RuntimeError("the autograd wrappers cannot be captured in a CUDA graph")
+        stream = self.stream = torch.cuda.current_stream()
+        # taken out while in use (re-entrant calls get their own)
+        ctx, last, self.event = _pool().pop(self.key, (None, None, None))
         if ctx is None:
             ctx = L.dna_create(N, T, R, L.make_opts(dtype=dtype))
+            self.event = torch.cuda.Event()
         self.ctx = ctx
         try:
-            L.dna_set_stream(ctx)
+            if last is not None and last != stream:
+                stream.wait_event(self.event)   # the context's workspace is still in use there
+            for t in (V, W, H, *others):
+                t.record_stream(stream)
+            L.dna_set_stream(ctx, stream)
             L.dna_bind(ctx, V, W, H)
         except BaseException:
             L.dna_destroy(ctx)
@@ -68,7 +85,8 @@ class _Ctx:
     def __exit__(self, exc_type, exc, tb):
         pool = _pool()
         if exc_type is None and self.key not in pool:
-            pool[self.key] = self.ctx
+            self.event.record(self.stream)
+            pool[self.key] = (self.ctx, self.stream, self.event)
         else:
             L.dna_destroy(self.ctx)
         return False
@@ -81,7 +99,7 @@ class KLDiv(torch.autograd.Function):
         with _Ctx(V, W, H) as ctx:
             kl = L.dna_kl(ctx)
         fctx.save_for_backward(V, W, H)
-        return torch.tensor(kl, dtype=torch.float64, device=V.device)
+        return torch.full((), kl, dtype=torch.float64, device=V.device)
 
     @staticmethod
     def backward(fctx, grad):
@@ -92,7 +110,6 @@ class KLDiv(torch.autograd.Function):
         dH = torch.empty_like(H) if need_h else None
         with _Ctx(V, W, H) as ctx:
             L.dna_kl_backward(ctx, float(grad), dW, dH, dV)
-            torch.cuda.current_stream().synchronize()
         return dV, dW, dH
 
 
@@ -109,7 +126,6 @@ class UnrolledDNAH(torch.autograd.Function):
                 if k % every == 0:
                     ckpts.append(H.clone())
                 L.dna_step_H_fixed(ctx, choices[k])
-            torch.cuda.current_stream().synchronize()
         fctx.K, fctx.every = K, every
         fctx.save_for_backward(V, W, choices, *ckpts)
         return H
@@ -123,7 +139,7 @@ class UnrolledDNAH(torch.autograd.Function):
         Vbar = torch.zeros_like(V) if need_v else None
         Wbar = torch.zeros_like(W) if need_w else None
         Hrun = ckpts[0].clone()
-        with _Ctx(V, W, Hrun) as ctx:
+        with _Ctx(V, W, Hrun, choices, *ckpts) as ctx:
             for seg in reversed(range(len(ckpts))):
                 k0, k1 = seg * every, min(seg * every + every, K)
                 Hrun.copy_(ckpts[seg])
@@ -136,5 +152,4 @@ class UnrolledDNAH(torch.autograd.Function):
                     L.dna_step_H_adjoint_w(ctx, states[k - k0], choices[k], Hbar, out, Vbar,
                                            Wbar)
                     Hbar = out
-            torch.cuda.current_stream().synchronize()
         return Vbar, Wbar, Hbar, None, None
