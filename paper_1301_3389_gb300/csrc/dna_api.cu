@@ -95,7 +95,9 @@ struct dna_ctx {
     int64_t* cptr = nullptr;
     int32_t* ridx = nullptr;
     void* cval = nullptr;
-    void* Yt = nullptr;
+    int64_t R4 = 0;          // rows of both factors are padded to R4 values
+    void* Hr = nullptr;      // H^t as rows (T x R4)
+    void* Wr = nullptr;      // W as padded rows (N x R4), used where W's own rows are not
     double* c0 = nullptr;
     // segments of at most sparse::SEG non-zeros per view (0: columns of V, 1: rows), built
     // at bind, with their partial sums
@@ -333,7 +335,7 @@ void free_all(dna_ctx* c) {
     void* ptrs[] = {c->own_V, c->own_W, c->own_H, c->Vt, c->colsum_v, c->rowsum_v, c->c, c->sig,
                     c->fwork, c->gpart, c->vpart, c->Apart, c->Bpart, c->Xmu, c->Xdna, c->dpart, c->dfin_h, c->dfin_w,
                     c->choice_h, c->choice_w, c->kl_dev, c->kl_part, c->status, c->Xk, c->Yk, c->Ytk,
-                    c->Y2tk, c->Xmk, c->Xdk, c->Vp, c->Qg, c->Qbg, c->cptr, c->ridx, c->cval, c->Yt, c->c0,
+                    c->Y2tk, c->Xmk, c->Xdk, c->Vp, c->Qg, c->Qbg, c->cptr, c->ridx, c->cval, c->Hr, c->Wr, c->c0,
                     c->seg_col[0], c->seg_col[1], c->seg_k0[0], c->seg_k0[1], c->seg_k1[0],
                     c->seg_k1[1], c->seg_ptr[0], c->seg_ptr[1], c->Aseg, c->Bseg, c->dseg,
                     c->dcur, c->wg_part, c->wg_cpart};
@@ -422,7 +424,8 @@ int alloc_workspace(dna_ctx* c) {
 // and one split (each view column is reduced by one warp).
 template <typename Tp>
 int alloc_sparse_workspace(dna_ctx* c) {
-    const int64_t N = c->N, T = c->T, R = c->R, M = std::max(N, T);
+    const int64_t N = c->N, T = c->T, R = c->R, M = std::max(N, T), R4 = (R + 3) / 4 * 4;
+    c->R4 = R4;
     int e = DNA_OK;
     e |= dmalloc(&c->colsum_v, sizeof(double) * T);
     e |= dmalloc(&c->rowsum_v, sizeof(double) * N);
@@ -431,10 +434,8 @@ int alloc_sparse_workspace(dna_ctx* c) {
     e |= dmalloc(&c->sig, sizeof(double) * R);
     e |= dmalloc(&c->fwork, sizeof(double) * dna::FSUM_SPLITS * R);
     e |= dmalloc(&c->gpart, sizeof(double) * (size_t)(dna::Simt<Tp>::glue_parts(M) * R));
-    e |= dmalloc(&c->Apart, sizeof(Tp) * (size_t)(R * M));
-    e |= dmalloc(&c->Bpart, sizeof(Tp) * (size_t)(R * M));
-    e |= dmalloc(&c->Xmu, sizeof(Tp) * (size_t)(R * M));
-    e |= dmalloc(&c->Xdna, sizeof(Tp) * (size_t)(R * M));
+    e |= dmalloc(&c->Xmu, sizeof(Tp) * (size_t)(R4 * M));
+    e |= dmalloc(&c->Xdna, sizeof(Tp) * (size_t)(R4 * M));
     e |= dmalloc(&c->dpart, sizeof(double) * (size_t)(2 * M));
     e |= dmalloc(&c->dfin_h, sizeof(double) * 2 * T);
     e |= dmalloc(&c->dfin_w, sizeof(double) * 2 * N);
@@ -446,7 +447,8 @@ int alloc_sparse_workspace(dna_ctx* c) {
     e |= dmalloc(&c->cptr, sizeof(int64_t) * (size_t)(T + 1));
     e |= dmalloc(&c->ridx, sizeof(int32_t) * (size_t)std::max<int64_t>(c->nnz, 1));
     e |= dmalloc(&c->cval, sizeof(Tp) * (size_t)std::max<int64_t>(c->nnz, 1));
-    e |= dmalloc(&c->Yt, sizeof(Tp) * (size_t)(T * R));
+    e |= dmalloc(&c->Hr, sizeof(Tp) * (size_t)(T * R4));
+    e |= dmalloc(&c->Wr, sizeof(Tp) * (size_t)(N * R4));
     if (e != DNA_OK) return DNA_ERR_ALLOC;
     if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess ||
         cudaMemset(c->choice_h, 0, (size_t)T) != cudaSuccess ||
@@ -525,8 +527,8 @@ int bind_csr(dna_ctx* c, const int64_t* rptr, const int32_t* cidx, const Tp* val
     }
     for (void* q : {c->Aseg, c->Bseg, (void*)c->dseg})
         if (q) cudaFree(q);
-    if (dmalloc(&c->Aseg, sizeof(Tp) * (size_t)(maxseg * c->R)) ||
-        dmalloc(&c->Bseg, sizeof(Tp) * (size_t)(maxseg * c->R)) ||
+    if (dmalloc(&c->Aseg, sizeof(Tp) * (size_t)(maxseg * c->R4)) ||
+        dmalloc(&c->Bseg, sizeof(Tp) * (size_t)(maxseg * c->R4)) ||
         dmalloc(&c->dseg, sizeof(double) * (size_t)(2 * maxseg)))
         return DNA_ERR_ALLOC;
     for (int w = 0; w < 2; ++w) {
@@ -861,61 +863,69 @@ dna::SparseSegs segs(const dna_ctx* c, int w) {
     return dna::SparseSegs{c->seg_col[w], c->seg_k0[w], c->seg_k1[w], c->seg_ptr[w], c->nseg[w]};
 }
 
+// Both factors as rows of R4 values for the sparse kernels: a transposed copy of H, and W
+// itself where its rows are 16-byte words already.
+template <typename Tp>
+int sparse_rows(dna_ctx* c, const Tp** Wr, const Tp** Hr) {
+    using S = dna::Simt<Tp>;
+    const bool direct = c->R4 == c->R && reinterpret_cast<uintptr_t>(c->W) % 16 == 0;
+    *Wr = static_cast<const Tp*>(direct ? c->W : c->Wr);
+    *Hr = static_cast<const Tp*>(c->Hr);
+    return phase(c, DNA_PHASE_OPERANDS, direct ? 1 : 2, [&] {
+        int e = S::transpose(static_cast<const Tp*>(c->H), c->R, c->T, c->R4,
+                             static_cast<Tp*>(c->Hr), c->stream);
+        if (!e && !direct)
+            e = S::pad_rows(static_cast<const Tp*>(c->W), c->N, c->R, c->R4,
+                            static_cast<Tp*>(c->Wr), c->stream);
+        return e;
+    });
+}
+
 // One half-step of the sparse-V form: the same steps as half_step with the two O(NRT)
-// passes replaced by passes over the non-zeros (sparse_kernels.cuh); candidates, selection
-// and normalisation are the dense glue kernels (they touch only W, H and O-vectors).
+// passes replaced by passes over the non-zeros (sparse_kernels.cuh) and candidates and
+// selection on rows; the normalisation is the dense glue.
 template <typename Tp>
 int sparse_half_step(dna_ctx* c, int w, bool mu_only, bool prepared, bool next) {
     using S = dna::Simt<Tp>;
     const View v = make_view(c, w == 1);
-    Tp* A = static_cast<Tp*>(c->Apart);
-    Tp* B = static_cast<Tp*>(c->Bpart);
-    Tp* Xmu = static_cast<Tp*>(c->Xmu);
-    Tp* Xdna = static_cast<Tp*>(c->Xdna);
+    Tp* Xm = static_cast<Tp*>(c->Xmu);
+    Tp* Xd = static_cast<Tp*>(c->Xdna);
     cudaStream_t st = c->stream;
     int e = DNA_OK;
     if (!prepared)
         if ((e = prep_step<Tp>(c, w, false))) return e;
     // c0 from the per-block column sums of Y that the preparation left in gpart
-    e = phase(c, DNA_PHASE_SUMS, 1, [&] {
-        return S::raw_sums(c->gpart, S::glue_parts(v.S), c->R, c->c0, st);
-    });
-    if (e) return e;
-    const Tp* Yg = static_cast<const Tp*>(c->W);   // H-step: W is already S x R
-    if (w == 1) {                                   // W-step: gather rows of H^t
-        e = phase(c, DNA_PHASE_OPERANDS, 1, [&] {
-            return S::transpose(static_cast<const Tp*>(c->H), c->R, c->T, static_cast<Tp*>(c->Yt), st);
+    if (!mu_only)
+        e = phase(c, DNA_PHASE_SUMS, 1, [&] {
+            return S::raw_sums(c->gpart, S::glue_parts(v.S), c->R, c->c0, st);
         });
-        if (e) return e;
-        Yg = static_cast<const Tp*>(c->Yt);
-    }
+    if (e) return e;
+    const Tp *Wr, *Hr;
+    if ((e = sparse_rows<Tp>(c, &Wr, &Hr))) return e;
+    const Tp *Yr = w ? Hr : Wr, *Xr = w ? Wr : Hr;
     const dna::SparseSegs sg = segs(c, w);
     const int32_t* idx = w ? c->cidx : c->ridx;
     const Tp* val = static_cast<const Tp*>(w ? c->rval : c->cval);
     Tp* Aseg = static_cast<Tp*>(c->Aseg);
     Tp* Bseg = static_cast<Tp*>(c->Bseg);
-    e = phase(c, DNA_PHASE_PASS1, 2, [&] {
-        return S::sp_pass1(v, sg, idx, val, Yg, Aseg, Bseg, A, B, !mu_only, c->status, st);
+    e = phase(c, DNA_PHASE_PASS1, 1, [&] {
+        return S::sp_pass1(c->R, sg, idx, val, Yr, Xr, c->R4, Aseg, Bseg, !mu_only, c->status, st);
     });
-    if (e) return e;
-    if (mu_only) {
-        e = phase(c, DNA_PHASE_CANDIDATES, 1, [&] { return S::mu_fused(v, c->c, A, 1, c->gpart, st); });
-        return e ? e : finish_step<Tp>(c, w, next);
-    }
-    e = phase(c, DNA_PHASE_CANDIDATES, 1, [&] {
-        return S::cand_fused(v, c->c, A, B, 1, Xmu, Xdna, c->o.eps, c->o.alpha, nullptr, nullptr,
-                             0, 0, 0, st);
-    });
-    if (e) return e;
-    e = phase(c, DNA_PHASE_PASS2, 2, [&] {
-        return S::sp_pass2(v, sg, idx, val, Yg, Xmu, Xdna, c->c0, c->dseg, c->dpart, c->status, st);
-    });
-    if (e) return e;
-    e = phase(c, DNA_PHASE_SELECT, 1, [&] {
-        return S::select_fused(v, Xmu, Xdna, c->dpart, 1, w ? c->choice_w : c->choice_h,
-                               w ? c->dfin_w : c->dfin_h, c->gpart, w ? c->o.rho : c->o.lambda,
-                               st);
-    });
+    if (!e)
+        e = phase(c, DNA_PHASE_CANDIDATES, 1, [&] {
+            return S::sp_cand(v, sg, Aseg, Bseg, Xr, c->R4, c->c, Xm, Xd, c->o.eps, c->o.alpha,
+                              mu_only, st);
+        });
+    if (!e && !mu_only)
+        e = phase(c, DNA_PHASE_PASS2, 1, [&] {
+            return S::sp_pass2(c->R, sg, idx, val, Yr, Xm, Xd, c->R4, c->dseg, st);
+        });
+    if (!e)
+        e = phase(c, DNA_PHASE_SELECT, 1, [&] {
+            return S::sp_select(v, sg, c->dseg, Xm, Xd, c->R4, c->c0, w ? c->choice_w : c->choice_h,
+                                w ? c->dfin_w : c->dfin_h, c->gpart, w ? c->o.rho : c->o.lambda,
+                                mu_only, c->status, st);
+        });
     if (e) return e;
     return finish_step<Tp>(c, w, next);
 }
@@ -927,13 +937,14 @@ int sparse_kl(dna_ctx* c) {
     using S = dna::Simt<Tp>;
     const View v = make_view(c, false);
     cudaStream_t st = c->stream;
+    const Tp *Wr, *Hr;
+    if (int e = sparse_rows<Tp>(c, &Wr, &Hr)) return e;
     return phase(c, DNA_PHASE_KL, 5, [&] {
         int e = S::scale_ops(v, nullptr, false, nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0,
                              c->gpart, st);
         if (!e) e = S::raw_sums(c->gpart, S::glue_parts(v.S), c->R, c->c0, st);
-        if (!e) e = S::sp_kl(v, segs(c, 0), c->ridx, static_cast<const Tp*>(c->cval),
-                             static_cast<const Tp*>(c->W), c->c0, c->dseg, c->dpart, c->status,
-                             st);
+        if (!e) e = S::sp_kl(v, segs(c, 0), c->ridx, static_cast<const Tp*>(c->cval), Wr, Hr, c->R4,
+                             c->c0, c->dseg, c->dpart, c->status, st);
         return e ? e : dna::reduce_sum(c->dpart, c->T, c->kl_dev, c->kl_part, st);
     });
 }

@@ -160,19 +160,29 @@ template <typename Tp> struct Simt {
     static int raw_sums(const double* part, int64_t nparts, int64_t R, double* out,
                         cudaStream_t st);
     // Sparse-V form (sparse_kernels.cuh): the view's non-zero k is at s = idx[k] with value
-    // val[k], grouped in segments `sg`; Yg is Y as S x R row-major; R <= 128.  Each call is a
-    // segment kernel (partials Aseg, Bseg [nseg][R] or dseg) and a per-column reduction.
-    static int sp_pass1(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-                        const Tp* Yg, Tp* Aseg, Tp* Bseg, Tp* A, Tp* B, bool with_b,
+    // val[k], grouped in segments `sg`; Yr, Xr the factors as rows of R values padded to R4
+    // (S x R4, O x R4), Xm, Xd the candidates as such rows; R <= 128.
+    static int sp_pass1(int64_t R, const SparseSegs& sg, const int32_t* idx, const Tp* val,
+                        const Tp* Yr, const Tp* Xr, int64_t R4, Tp* Aseg, Tp* Bseg, bool with_b,
                         int* status, cudaStream_t st);
-    static int sp_pass2(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-                        const Tp* Yg, const Tp* Xmu, const Tp* Xdna, const double* c0,
-                        double* dseg, double* dpart, int* status, cudaStream_t st);
+    static int sp_cand(const View& v, const SparseSegs& sg, const Tp* Aseg, const Tp* Bseg,
+                       const Tp* Xr, int64_t R4, const double* c, Tp* Xm, Tp* Xd, double eps,
+                       double alpha, bool mu, cudaStream_t st);
+    static int sp_pass2(int64_t R, const SparseSegs& sg, const int32_t* idx, const Tp* val,
+                        const Tp* Yr, const Tp* Xm, const Tp* Xd, int64_t R4, double* dseg,
+                        cudaStream_t st);
+    // selection and the new X with its per-block sums fpart (mu: Xm is kept)
+    static int sp_select(const View& v, const SparseSegs& sg, const double* dseg, const Tp* Xm,
+                         const Tp* Xd, int64_t R4, const double* c0, uint8_t* choice, double* dfin,
+                         double* fpart, double reg, bool mu, int* status, cudaStream_t st);
     static int sp_kl(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-                     const Tp* Yg, const double* c0, double* dseg, double* part, int* status,
-                     cudaStream_t st);
-    // out (cols x rows) = in^t (rows x cols), both row-major
-    static int transpose(const Tp* in, int64_t rows, int64_t cols, Tp* out, cudaStream_t st);
+                     const Tp* Yr, const Tp* Xr, int64_t R4, const double* c0, double* dseg,
+                     double* part, int* status, cudaStream_t st);
+    // out (n x ld) = in (n x R) with zeros past R
+    static int pad_rows(const Tp* in, int64_t n, int64_t R, int64_t ld, Tp* out, cudaStream_t st);
+    // out (cols x ld) = in^t (in rows x cols), zeros past `rows`, all row-major
+    static int transpose(const Tp* in, int64_t rows, int64_t cols, int64_t ld, Tp* out,
+                         cudaStream_t st);
     // one-time: row and column sums of V (float64) and the transposed copy; with Vc (needs
     // part) also a copy of V into Vc [N][T] in the same pass (V may be pinned host memory)
     static int prepare_v(const Tp* V, int64_t N, int64_t T, int64_t ldv, Tp* Vt, int64_t ldvt,

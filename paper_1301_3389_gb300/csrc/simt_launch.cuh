@@ -2,6 +2,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "glue_kernels.cuh"
 #include "simt_kernels.cuh"
@@ -538,81 +539,99 @@ int Simt<Tp>::raw_sums(const double* part, int64_t nparts, int64_t R, double* ou
 namespace simt {
 inline unsigned sp_grid(int64_t n) { return (unsigned)((n + sparse::WARPS - 1) / sparse::WARPS); }
 
-template <typename Tp, int RPL>
-int sp_pass1_r(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-               const Tp* Yg, Tp* Aseg, Tp* Bseg, Tp* A, Tp* B, bool with_b, int* status,
-               cudaStream_t st) {
-    if (sg.n > 0) {
-        sparse::k_sp_pass1<Tp, RPL><<<sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(
-            v, sg, idx, val, Yg, Aseg, Bseg, with_b, status);
-        if (launch_status()) return DNA_ERR_CUDA;
-    }
-    sparse::k_sp_reduce_ab<Tp, RPL><<<sp_grid(v.O), sparse::WARPS * 32, 0, st>>>(
-        v.O, v.R, sg.sptr, Aseg, Bseg, A, B, with_b);
-    return launch_status();
-}
-template <typename Tp, int RPL>
-int sp_pass2_r(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-               const Tp* Yg, const Tp* Xmu, const Tp* Xdna, const double* c0, double* dseg,
-               double* dpart, int* status, cudaStream_t st) {
-    if (sg.n > 0) {
-        sparse::k_sp_pass2<Tp, RPL><<<sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(
-            v, sg, idx, val, Yg, Xmu, Xdna, dseg);
-        if (launch_status()) return DNA_ERR_CUDA;
-    }
-    sparse::k_sp_reduce_cost<Tp, RPL><<<sp_grid(v.O), sparse::WARPS * 32, 0, st>>>(
-        v.O, v.R, sg.sptr, dseg, Xmu, Xdna, c0, dpart, status);
-    return launch_status();
-}
-template <typename Tp, int RPL>
-int sp_kl_r(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-            const Tp* Yg, const double* c0, double* dseg, double* part, int* status,
-            cudaStream_t st) {
-    if (sg.n > 0) {
-        sparse::k_sp_kl<Tp, RPL><<<sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(v, sg, idx, val,
-                                                                               Yg, dseg);
-        if (launch_status()) return DNA_ERR_CUDA;
-    }
-    sparse::k_sp_reduce_kl<Tp, RPL><<<sp_grid(v.O), sparse::WARPS * 32, 0, st>>>(
-        v, sg.sptr, dseg, c0, part, status);
-    return launch_status();
+// f(constant LPN) with the lanes per row of rank R (R <= 128)
+template <class F>
+int by_lanes(int64_t R, F&& f) {
+    if (R <= 32) return f(std::integral_constant<int, 8>());
+    if (R <= 64) return f(std::integral_constant<int, 16>());
+    if (R <= 128) return f(std::integral_constant<int, 32>());
+    return DNA_ERR_UNSUPPORTED;
 }
 }  // namespace simt
 
 template <typename Tp>
-int Simt<Tp>::sp_pass1(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-                       const Tp* Yg, Tp* Aseg, Tp* Bseg, Tp* A, Tp* B, bool with_b, int* status,
-                       cudaStream_t st) {
-    if (v.R <= 32) return simt::sp_pass1_r<Tp, 1>(v, sg, idx, val, Yg, Aseg, Bseg, A, B, with_b, status, st);
-    if (v.R <= 64) return simt::sp_pass1_r<Tp, 2>(v, sg, idx, val, Yg, Aseg, Bseg, A, B, with_b, status, st);
-    if (v.R <= 128) return simt::sp_pass1_r<Tp, 4>(v, sg, idx, val, Yg, Aseg, Bseg, A, B, with_b, status, st);
-    return DNA_ERR_UNSUPPORTED;
+int Simt<Tp>::sp_pass1(int64_t R, const SparseSegs& sg, const int32_t* idx, const Tp* val,
+                       const Tp* Yr, const Tp* Xr, int64_t R4, Tp* Aseg, Tp* Bseg, bool with_b,
+                       int* status, cudaStream_t st) {
+    if (sg.n == 0) return DNA_OK;
+    return simt::by_lanes(R, [&](auto lpn) {
+        sparse::k_sp_pass1<Tp, decltype(lpn)::value>
+            <<<simt::sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(R4, sg, idx, val, Yr, Xr, Aseg,
+                                                                 Bseg, with_b, status);
+        return simt::launch_status();
+    });
 }
 
 template <typename Tp>
-int Simt<Tp>::sp_pass2(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-                       const Tp* Yg, const Tp* Xmu, const Tp* Xdna, const double* c0,
-                       double* dseg, double* dpart, int* status, cudaStream_t st) {
-    if (v.R <= 32) return simt::sp_pass2_r<Tp, 1>(v, sg, idx, val, Yg, Xmu, Xdna, c0, dseg, dpart, status, st);
-    if (v.R <= 64) return simt::sp_pass2_r<Tp, 2>(v, sg, idx, val, Yg, Xmu, Xdna, c0, dseg, dpart, status, st);
-    if (v.R <= 128) return simt::sp_pass2_r<Tp, 4>(v, sg, idx, val, Yg, Xmu, Xdna, c0, dseg, dpart, status, st);
-    return DNA_ERR_UNSUPPORTED;
+int Simt<Tp>::sp_cand(const View& v, const SparseSegs& sg, const Tp* Aseg, const Tp* Bseg,
+                      const Tp* Xr, int64_t R4, const double* c, Tp* Xm, Tp* Xd, double eps,
+                      double alpha, bool mu, cudaStream_t st) {
+    return simt::by_lanes(v.R, [&](auto lpn) {
+        constexpr int LPN = decltype(lpn)::value;
+        const unsigned grid = simt::sp_grid((v.O + 32 / LPN - 1) / (32 / LPN));
+        auto k = mu ? sparse::k_sp_cand<Tp, LPN, true> : sparse::k_sp_cand<Tp, LPN, false>;
+        k<<<grid, sparse::WARPS * 32, 0, st>>>(v.O, v.R, R4, sg.sptr, Aseg, Bseg, Xr, c, v.vsum,
+                                               Xm, Xd, (Tp)eps, (Tp)alpha);
+        return simt::launch_status();
+    });
+}
+
+template <typename Tp>
+int Simt<Tp>::sp_pass2(int64_t R, const SparseSegs& sg, const int32_t* idx, const Tp* val,
+                       const Tp* Yr, const Tp* Xm, const Tp* Xd, int64_t R4, double* dseg,
+                       cudaStream_t st) {
+    if (sg.n == 0) return DNA_OK;
+    return simt::by_lanes(R, [&](auto lpn) {
+        sparse::k_sp_pass2<Tp, decltype(lpn)::value>
+            <<<simt::sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(R4, sg, idx, val, Yr, Xm, Xd,
+                                                                 dseg);
+        return simt::launch_status();
+    });
+}
+
+template <typename Tp>
+int Simt<Tp>::sp_select(const View& v, const SparseSegs& sg, const double* dseg, const Tp* Xm,
+                        const Tp* Xd, int64_t R4, const double* c0, uint8_t* choice, double* dfin,
+                        double* fpart, double reg, bool mu, int* status, cudaStream_t st) {
+    return simt::by_lanes(v.R, [&](auto lpn) {
+        constexpr int LPN = decltype(lpn)::value;
+        auto k = mu ? sparse::k_sp_select<Tp, LPN, true> : sparse::k_sp_select<Tp, LPN, false>;
+        k<<<(unsigned)glue_parts(v.O), sparse::WARPS * 32, 0, st>>>(
+            v, R4, sg.sptr, dseg, Xm, Xd, c0, choice, dfin, fpart, reg, status);
+        return simt::launch_status();
+    });
 }
 
 template <typename Tp>
 int Simt<Tp>::sp_kl(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-                    const Tp* Yg, const double* c0, double* dseg, double* part, int* status,
-                    cudaStream_t st) {
-    if (v.R <= 32) return simt::sp_kl_r<Tp, 1>(v, sg, idx, val, Yg, c0, dseg, part, status, st);
-    if (v.R <= 64) return simt::sp_kl_r<Tp, 2>(v, sg, idx, val, Yg, c0, dseg, part, status, st);
-    if (v.R <= 128) return simt::sp_kl_r<Tp, 4>(v, sg, idx, val, Yg, c0, dseg, part, status, st);
-    return DNA_ERR_UNSUPPORTED;
+                    const Tp* Yr, const Tp* Xr, int64_t R4, const double* c0, double* dseg,
+                    double* part, int* status, cudaStream_t st) {
+    if (sg.n > 0) {
+        const int e = simt::by_lanes(v.R, [&](auto lpn) {
+            sparse::k_sp_kl<Tp, decltype(lpn)::value>
+                <<<simt::sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(R4, sg, idx, val, Yr, Xr,
+                                                                     dseg);
+            return simt::launch_status();
+        });
+        if (e) return e;
+    }
+    sparse::k_sp_reduce_kl<Tp><<<simt::sp_grid(v.O), sparse::WARPS * 32, 0, st>>>(
+        v.O, v.R, R4, sg.sptr, dseg, Xr, c0, part, status);
+    return simt::launch_status();
 }
 
 template <typename Tp>
-int Simt<Tp>::transpose(const Tp* in, int64_t rows, int64_t cols, Tp* out, cudaStream_t st) {
-    const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
-    sparse::k_transpose<Tp><<<grid, dim3(32, 8), 0, st>>>(in, rows, cols, out);
+int Simt<Tp>::pad_rows(const Tp* in, int64_t n, int64_t R, int64_t ld, Tp* out, cudaStream_t st) {
+    const int64_t blocks = std::min<int64_t>((n * ld + 255) / 256, 152 * 16);
+    sparse::k_pad_rows<Tp><<<(unsigned)blocks, 256, 0, st>>>(in, n, R, ld, out);
+    return simt::launch_status();
+}
+
+template <typename Tp>
+int Simt<Tp>::transpose(const Tp* in, int64_t rows, int64_t cols, int64_t ld, Tp* out,
+                        cudaStream_t st) {
+    const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((ld + 31) / 32));
+    sparse::k_transpose<Tp><<<grid, dim3(32, 8), 0, st>>>(in, rows, cols, ld, out);
     return simt::launch_status();
 }
 

@@ -8,15 +8,26 @@
 // sum_s z_so = sum_r (sum_s y_sr) x_ro = sum_r c0_r x_ro with c0 the column sums of Y.
 //
 // Storage: the non-zeros of view column o are k in [ptr[o], ptr[o + 1]), at s = idx[k] with
-// value val[k] (CSC of V for the H-step, CSR of V for the W-step); Yg is the fixed factor
-// as an S x R row-major array (W for the H-step, a transposed copy of H for the W-step),
-// so the R values of y(s, .) are one contiguous, coalesced row.
+// value val[k] (CSC of V for the H-step, CSR of V for the W-step).  Both factors are read as
+// rows of R values padded with zeros to R4 = ceil(R / 4) 4 (W itself where R is a multiple
+// of 4, else a padded copy; a transposed copy of H), and the candidates are rows [O][R4] too,
+// so that every access of a lane is one 16-byte word of a contiguous row.
 //
 // Work is split into segments of at most SEG non-zeros of one view column (term rows of
 // count data follow a Zipf law: one row can hold thousands of non-zeros), one warp per
-// segment; lane l holds r = l + 32 j (j < RPL).  Each segment writes its partial sums
-// [seg][R], and a warp per view column then adds its segments in order.  Dot products over
-// r are reduced with a fixed xor butterfly, so every result is bit-reproducible.
+// segment.  LPN = 8, 16 or 32 lanes (R <= 32, 64, 128) hold the four-value pieces of one row,
+// so a warp works on 32 / LPN non-zeros (or view columns) at once: at R = 64 two rows per warp
+// halve the shuffles and loads per non-zero against one row per warp with lane l holding
+// r = l, l + 32.  What is left of the passes is the gather itself, 256 bytes per non-zero
+// from L2 at 5 to 8 TB/s.  (A segment per lane group instead of per warp was no faster: 48, 65
+// and 46, 61 us.)
+// Each segment writes its partial sums [seg][R4], which the candidates kernel adds per
+// column in order.  Sums over lanes run in a fixed order, so every result is
+// bit-reproducible; costs are summed across lanes in pairs of float32 (value and rounding
+// error, about 48 bits) because a float64 add costs 64 cycles per warp on this GPU.
+// Measured at 36771 x 10212, 1.34 M non-zeros, R = 64 (H and W view, microseconds): pass 1
+// 60, 73 -> 47, 66, pass 2 57, 70 -> 40, 54, sums of segments and candidates 20, 78 -> 6, 20,
+// cost sums and selection 27, 81 -> 7, 15.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -24,24 +35,120 @@
 #include <stdint.h>
 
 #include "dna_internal.h"
+#include "simt_kernels.cuh"
 
 namespace dna {
 namespace sparse {
 
-constexpr int WARPS = 8;   // warps (segments or view columns) per CTA
-constexpr int U = 8;       // non-zeros whose loads are issued together
+constexpr int WARPS = 8;   // warps per CTA
+constexpr int U = 8;       // non-zeros per lane group whose loads are issued together
 constexpr int SEG = SPARSE_SEG;
 
+// Four consecutive values.
 template <typename Tp>
-__device__ __forceinline__ Tp warp_sum(Tp x) {
+struct Four {
+    Tp v[4];
+};
+__device__ __forceinline__ Four<float> load4(const float* p) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    return {{t.x, t.y, t.z, t.w}};
+}
+__device__ __forceinline__ Four<double> load4(const double* p) {
+    const double2 a = *reinterpret_cast<const double2*>(p);
+    const double2 b = *reinterpret_cast<const double2*>(p + 2);
+    return {{a.x, a.y, b.x, b.y}};
+}
+__device__ __forceinline__ void store4(float* p, const Four<float>& x) {
+    *reinterpret_cast<float4*>(p) = make_float4(x.v[0], x.v[1], x.v[2], x.v[3]);
+}
+__device__ __forceinline__ void store4(double* p, const Four<double>& x) {
+    *reinterpret_cast<double2*>(p) = make_double2(x.v[0], x.v[1]);
+    *reinterpret_cast<double2*>(p + 2) = make_double2(x.v[2], x.v[3]);
+}
+
+// A sum with its rounding error (float32), or a plain float64 sum.
+template <typename Tp>
+struct Sum;
+template <>
+struct Sum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double t) { s += t; }
+    __device__ __forceinline__ void add_product(double hi, double lo, double x) {
+        s += (hi + lo) * x;
+    }
+    __device__ __forceinline__ void add_lane(int m) { s += __shfl_xor_sync(0xffffffffu, s, m); }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct Sum<float> {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float t) {   // two-sum of Knuth
+        const float n = __fadd_rn(s, t), b = __fsub_rn(n, s);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(t, b)));
+        s = n;
+    }
+    // the exact product of x with the two-float number hi + lo, to float32 of the error
+    __device__ __forceinline__ void add_product(float hi, float lo, float x) {
+        const float p = __fmul_rn(hi, x);
+        add(p);
+        e = __fadd_rn(e, __fmaf_rn(lo, x, __fmaf_rn(hi, x, -p)));
+    }
+    __device__ __forceinline__ void add_lane(int m) {
+        const float t = __shfl_xor_sync(0xffffffffu, s, m);
+        const float u = __shfl_xor_sync(0xffffffffu, e, m);
+        // the same order on both sides of the exchange: the lower lane's pair first
+        const bool up = (threadIdx.x & m) != 0;
+        const float a = up ? t : s, b = up ? s : t, ea = up ? u : e, eb = up ? e : u;
+        s = a;
+        e = ea;
+        add(b);
+        e = __fadd_rn(e, eb);
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+// the sum over groups of LPN lanes
+template <int LPN, typename Tp>
+__device__ __forceinline__ Sum<Tp> group_add(Sum<Tp> x) {
 #pragma unroll
-    for (int m = 16; m > 0; m >>= 1) x += __shfl_xor_sync(0xffffffffu, x, m);
+    for (int m = LPN / 2; m > 0; m >>= 1) x.add_lane(m);
     return x;
+}
+template <int LPN, typename Tp>
+__device__ __forceinline__ Tp group_sum(Tp x) {
+#pragma unroll
+    for (int m = LPN / 2; m > 0; m >>= 1) x += __shfl_xor_sync(0xffffffffu, x, m);
+    return x;
+}
+
+// The two cost sums of a segment, 16 bytes: as value and rounding error in float32 (the
+// conversion to float64 would cost six float64 instructions per warp and segment, a quarter
+// of pass 2; the selection converts 32 columns at once).
+__device__ __forceinline__ void store_costs(double* dseg, int64_t g, const Sum<float>& m,
+                                            const Sum<float>& d) {
+    reinterpret_cast<float4*>(dseg)[g] = make_float4(m.s, m.e, d.s, d.e);
+}
+__device__ __forceinline__ void store_costs(double* dseg, int64_t g, const Sum<double>& m,
+                                            const Sum<double>& d) {
+    reinterpret_cast<double2*>(dseg)[g] = make_double2(m.s, d.s);
+}
+__device__ __forceinline__ void add_costs(const double* dseg, int64_t g, Sum<float>& m,
+                                          Sum<float>& d) {
+    const float4 t = reinterpret_cast<const float4*>(dseg)[g];
+    m.add(t.x);
+    m.e = __fadd_rn(m.e, t.y);
+    d.add(t.z);
+    d.e = __fadd_rn(d.e, t.w);
+}
+__device__ __forceinline__ void add_costs(const double* dseg, int64_t g, Sum<double>& m,
+                                          Sum<double>& d) {
+    const double2 t = reinterpret_cast<const double2*>(dseg)[g];
+    m.add(t.x);
+    d.add(t.y);
 }
 
 // The non-zeros of a segment are read 32 at a time with one coalesced load (lane l holds
 // the index and value of non-zero k + l) and handed to the whole warp by shuffles; the
-// next 32 are loaded while the current ones are used, so each batch of U non-zeros waits
+// next 32 are loaded while the current ones are used, so each batch of non-zeros waits
 // only for its gathered rows y(s, .).
 template <typename Tp>
 struct Chunk {
@@ -60,32 +167,15 @@ __device__ __forceinline__ Chunk<Tp> load_chunk(int64_t k, int64_t k1, int lane,
     return c;
 }
 
-// The rows y(s, .) gathered by the U non-zeros base .. base + U - 1 of chunk c (row 0 past
-// the segment's end, where the chunk holds s = 0 and v = 0).
-template <typename Tp, int RPL>
-__device__ __forceinline__ void gather_batch(const Chunk<Tp>& c, int base, int lane, int64_t R,
-                                             const Tp* __restrict__ Yg, Tp (&y)[U][RPL]) {
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const int64_t s = __shfl_sync(0xffffffffu, c.s, base + u);
-#pragma unroll
-        for (int j = 0; j < RPL; ++j) {
-            const int64_t r = lane + 32 * j;
-            y[u][j] = r < R ? Yg[s * R + r] : Tp(0);
-        }
-    }
-}
-
-// Sums each of the NV per-lane values p[i] over the warp (NV a power of two <= 32) with a
-// fixed reduce-scatter: at the step with xor mask m the lanes with bit m set keep the upper
-// half of the remaining values and the others the lower half, each adding its partner's
-// copy of the half it keeps; after log2(NV) steps a lane holds one value, index
-// lane >> (5 - log2(NV)), and the remaining xor steps complete its sum over all 32 lanes.
-// NV + 5 - log2(NV) - 1 shuffles for NV values instead of 5 NV.
-template <typename Tp, int NV>
+// Sums each of the NV per-lane values p[i] over groups of LPN lanes (NV a power of two, at
+// most LPN) with a fixed reduce-scatter: at the step with xor mask m the lanes with bit m set
+// keep the upper half of the remaining values and the others the lower half, each adding
+// its partner's copy of the half it keeps; after log2(NV) steps a lane holds one value, index
+// (lane % LPN) / (LPN / NV), and the remaining xor steps complete its sum.
+template <int LPN, int NV, typename Tp>
 __device__ __forceinline__ Tp scatter_sum(Tp (&p)[NV], int lane) {
-    static_assert(NV >= 1 && NV <= 32 && (NV & (NV - 1)) == 0, "NV: a power of two <= 32");
-    int m = 16;
+    static_assert(NV >= 1 && NV <= LPN && (NV & (NV - 1)) == 0, "NV: a power of two <= LPN");
+    int m = LPN / 2;
 #pragma unroll
     for (int cnt = NV; cnt > 1; cnt >>= 1, m >>= 1) {
         const bool hi = (lane & m) != 0;
@@ -102,23 +192,48 @@ __device__ __forceinline__ Tp scatter_sum(Tp (&p)[NV], int lane) {
     return t;
 }
 
-// Runs body(chunk, base, y) over the non-zeros [k0, k1) in batches of U.
-template <typename Tp, int RPL, class F>
-__device__ __forceinline__ void for_nonzeros(int64_t k0, int64_t k1, int lane, int64_t R,
+// Runs body(c, first, y) over the non-zeros [k0, k1) in batches of U per lane group: y[u] is
+// the row of the non-zero whose index and value lane first + u holds in c (past the end: row
+// 0 and value 0).
+template <int LPN, typename Tp, class F>
+__device__ __forceinline__ void for_nonzeros(int64_t k0, int64_t k1, int lane, int64_t R4,
                                              const int32_t* __restrict__ idx,
                                              const Tp* __restrict__ val,
-                                             const Tp* __restrict__ Yg, F&& body) {
+                                             const Tp* __restrict__ Yr, F&& body) {
+    constexpr int G = 32 / LPN;
+    const int r = 4 * (lane % LPN);
+    const bool in_row = r < R4;
     Chunk<Tp> cur = load_chunk<Tp>(k0, k1, lane, idx, val);
     for (int64_t k = k0; k < k1; k += 32) {
         const Chunk<Tp> nxt = load_chunk<Tp>(k + 32, k1, lane, idx, val);
         const int n = (int)(k1 - k < 32 ? k1 - k : 32);
-        for (int base = 0; base < n; base += U) {
-            Tp y[U][RPL];
-            gather_batch<Tp, RPL>(cur, base, lane, R, Yg, y);
-            body(cur, base, y);
+        for (int base = 0; base < n; base += U * G) {
+            const int first = base + U * (lane / LPN);
+            Four<Tp> y[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t s = __shfl_sync(0xffffffffu, cur.s, first + u);
+                if (in_row) y[u] = load4(Yr + s * R4 + r);
+                else y[u] = Four<Tp>{{Tp(0), Tp(0), Tp(0), Tp(0)}};
+            }
+            body(cur, first, y);
         }
         cur = nxt;
     }
+}
+
+template <typename Tp>
+__device__ __forceinline__ Tp dot4(const Four<Tp>& a, const Four<Tp>& b) {
+    Tp t = a.v[0] * b.v[0];
+#pragma unroll
+    for (int i = 1; i < 4; ++i) t = fma(a.v[i], b.v[i], t);
+    return t;
+}
+
+template <typename Tp>
+__device__ __forceinline__ Four<Tp> row4(const Tp* __restrict__ M, int64_t row, int64_t R4, int r) {
+    if (r < R4) return load4(M + row * R4 + r);
+    return Four<Tp>{{Tp(0), Tp(0), Tp(0), Tp(0)}};
 }
 
 using Segs = SparseSegs;
@@ -126,39 +241,26 @@ using Segs = SparseSegs;
 // Pass 1 (Algorithm 1 steps 2-5 and 10 on the non-zeros of one segment): partial raw sums
 // Aseg[g][r] = sum_k y(s_k, r) q_k and Bseg[g][r] = sum_k y(s_k, r)^2 qbar_k with q = v / z,
 // qbar = q / z.  Sets STATUS_NONFINITE when z <= 0 (or is not a number) at a positive v.
-template <typename Tp, int RPL>
+template <typename Tp, int LPN>
 __global__ void __launch_bounds__(WARPS * 32)
-    k_sp_pass1(View v, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
-               const Tp* __restrict__ Yg, Tp* __restrict__ Aseg, Tp* __restrict__ Bseg,
-               bool with_b, int* __restrict__ status) {
-    const int lane = threadIdx.x & 31;
+    k_sp_pass1(int64_t R4, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
+               const Tp* __restrict__ Yr, const Tp* __restrict__ Xr, Tp* __restrict__ Aseg,
+               Tp* __restrict__ Bseg, bool with_b, int* __restrict__ status) {
+    constexpr int STEP = LPN / U;   // lanes that hold the same finished z
+    const int lane = threadIdx.x & 31, sub = lane % LPN, lead = lane - sub, r = 4 * sub;
     const int64_t g = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
     if (g >= sg.n) return;
-    const int64_t R = v.R, o = sg.col[g];
-    const Tp* __restrict__ X = static_cast<const Tp*>(v.X);
-    Tp x[RPL], a[RPL], b[RPL];
-#pragma unroll
-    for (int j = 0; j < RPL; ++j) {
-        const int64_t r = lane + 32 * j;
-        x[j] = r < R ? X[r * v.xr + o * v.xo] : Tp(0);
-        a[j] = Tp(0);
-        b[j] = Tp(0);
-    }
+    const int64_t k0 = sg.k0[g], k1 = sg.k1[g], col = sg.col[g];
+    const Four<Tp> x = row4(Xr, col, R4, r);
+    Four<Tp> a{{Tp(0), Tp(0), Tp(0), Tp(0)}}, b{{Tp(0), Tp(0), Tp(0), Tp(0)}};
     bool bad = false;
-    constexpr int LOGU = U == 8 ? 3 : (U == 4 ? 2 : (U == 16 ? 4 : -1));
-    static_assert(LOGU > 0, "U: 4, 8 or 16");
-    const int ul = lane >> (5 - LOGU);   // the non-zero of the batch this lane finishes
-    for_nonzeros<Tp, RPL>(sg.k0[g], sg.k1[g], lane, R, idx, val, Yg,
-                          [&](const Chunk<Tp>& c, int base, Tp (&y)[U][RPL]) {
+    for_nonzeros<LPN>(k0, k1, lane, R4, idx, val, Yr,
+                      [&](const Chunk<Tp>& c, int first, const Four<Tp> (&y)[U]) {
         Tp p[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            p[u] = Tp(0);
-#pragma unroll
-            for (int j = 0; j < RPL; ++j) p[u] += y[u][j] * x[j];
-        }
-        const Tp z = scatter_sum<Tp, U>(p, lane);             // z of non-zero ul
-        const Tp vl = __shfl_sync(0xffffffffu, c.v, base + ul);
+        for (int u = 0; u < U; ++u) p[u] = dot4(y[u], x);
+        const Tp z = scatter_sum<LPN, U>(p, lane);            // z of non-zero sub / STEP
+        const Tp vl = __shfl_sync(0xffffffffu, c.v, first + sub / STEP);
         Tp q = Tp(0), qb = Tp(0);
         if (vl > Tp(0)) {                                      // v = 0: q = qbar = 0
             if (z > Tp(0)) {
@@ -171,207 +273,317 @@ __global__ void __launch_bounds__(WARPS * 32)
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const Tp qu = __shfl_sync(0xffffffffu, q, u << (5 - LOGU));
-            const Tp qbu = __shfl_sync(0xffffffffu, qb, u << (5 - LOGU));
+            const Tp qu = __shfl_sync(0xffffffffu, q, lead + u * STEP);
+            const Tp qbu = __shfl_sync(0xffffffffu, qb, lead + u * STEP);
 #pragma unroll
-            for (int j = 0; j < RPL; ++j) {
-                a[j] += y[u][j] * qu;
-                b[j] += y[u][j] * y[u][j] * qbu;
+            for (int i = 0; i < 4; ++i) {
+                a.v[i] = fma(y[u].v[i], qu, a.v[i]);
+                b.v[i] = fma(y[u].v[i] * y[u].v[i], qbu, b.v[i]);
             }
         }
     });
-    bad = __any_sync(0xffffffffu, bad);
 #pragma unroll
-    for (int j = 0; j < RPL; ++j) {
-        const int64_t r = lane + 32 * j;
-        if (r < R) {
-            Aseg[g * R + r] = a[j];
-            if (with_b) Bseg[g * R + r] = b[j];
+    for (int m = LPN; m < 32; m <<= 1)   // the lane groups' shares of the segment
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            a.v[i] += __shfl_xor_sync(0xffffffffu, a.v[i], m);
+            b.v[i] += __shfl_xor_sync(0xffffffffu, b.v[i], m);
         }
+    if (lead == 0 && r < R4) {
+        store4(Aseg + g * R4 + r, a);
+        if (with_b) store4(Bseg + g * R4 + r, b);
     }
-    if (bad && status) atomicOr(status, STATUS_NONFINITE);
+    bad = __any_sync(0xffffffffu, bad);
+    if (bad && lane == 0) atomicOr(status, STATUS_NONFINITE);
 }
 
-// A(r, o) = sum over the segments of column o of Aseg (in segment order), written [R][O]
-// (split 0 of the dense layout); the same for B.  A warp per view column.
-template <typename Tp, int RPL>
+// The candidates of view column o, a group of LPN lanes per column: A and B as the sums of
+// the column's segments in order, then eq. 11 (Xm), eq. 15 / 17 and the eq. 10
+// renormalisation (Xd), rows [O][R4] with zeros past R.  MU: Xm only.
+template <typename Tp, int LPN, bool MU>
 __global__ void __launch_bounds__(WARPS * 32)
-    k_sp_reduce_ab(int64_t O, int64_t R, const int64_t* __restrict__ sptr,
-                   const Tp* __restrict__ Aseg, const Tp* __restrict__ Bseg, Tp* __restrict__ A,
-                   Tp* __restrict__ B, bool with_b) {
-    const int lane = threadIdx.x & 31;
-    const int64_t o = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
-    if (o >= O) return;
-    Tp a[RPL], b[RPL];
+    k_sp_cand(int64_t O, int64_t R, int64_t R4, const int64_t* __restrict__ sptr,
+              const Tp* __restrict__ Aseg, const Tp* __restrict__ Bseg,
+              const Tp* __restrict__ Xr, const double* __restrict__ c,
+              const double* __restrict__ vsum, Tp* __restrict__ Xm, Tp* __restrict__ Xd, Tp eps,
+              Tp alpha) {
+    __shared__ Tp cs[4 * LPN], ics[4 * LPN];
+    for (int k = threadIdx.x; k < 4 * LPN; k += WARPS * 32) {
+        cs[k] = k < R ? (Tp)c[k] : Tp(1);
+        ics[k] = Tp(1) / cs[k];
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, sub = lane % LPN, r = 4 * sub;
+    const int64_t o =
+        ((int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5)) * (32 / LPN) + lane / LPN;
+    const bool live = o < O;
+    const bool in = live && r < R4;
+    Four<Tp> a{{Tp(0), Tp(0), Tp(0), Tp(0)}}, b = a, x = a;
+    if (in) {
+        x = load4(Xr + o * R4 + r);
+        const int64_t g1 = sptr[o + 1];
+#pragma unroll 8
+        for (int64_t g = sptr[o]; g < g1; ++g) {   // the longest columns have dozens
+            const Four<Tp> ta = load4(Aseg + g * R4 + r);
 #pragma unroll
-    for (int j = 0; j < RPL; ++j) { a[j] = Tp(0); b[j] = Tp(0); }
-    for (int64_t g = sptr[o]; g < sptr[o + 1]; ++g) {
+            for (int i = 0; i < 4; ++i) a.v[i] += ta.v[i];
+            if (!MU) {
+                const Four<Tp> tb = load4(Bseg + g * R4 + r);
 #pragma unroll
-        for (int j = 0; j < RPL; ++j) {
-            const int64_t r = lane + 32 * j;
-            if (r < R) {
-                a[j] += Aseg[g * R + r];
-                if (with_b) b[j] += Bseg[g * R + r];
+                for (int i = 0; i < 4; ++i) b.v[i] += tb.v[i];
             }
         }
     }
+    Four<Tp> xm, xd;
+    Tp den = Tp(0);
 #pragma unroll
-    for (int j = 0; j < RPL; ++j) {
-        const int64_t r = lane + 32 * j;
-        if (r < R) {
-            A[r * O + o] = a[j];
-            if (with_b) B[r * O + o] = b[j];
+    for (int i = 0; i < 4; ++i) {
+        const Tp ic = ics[r + i], xr = x.v[i];
+        if (MU) {
+            xm.v[i] = xr * (a.v[i] / cs[r + i]);
+            continue;
         }
+        const Tp av = a.v[i] * ic - Tp(1), bv = b.v[i] * ic;   // eq. 7, 14
+        xm.v[i] = xr * (a.v[i] * ic);      // eq. 11 as x (W^t q)_r / c_r (no cancellation)
+        Tp d;
+        if (av < Tp(0)) {                  // eq. 15, gain floored at eps
+            const Tp xb = xr * bv;
+            const Tp gn = simt::dev_div(xb, xb - av);
+            d = xr * (gn > eps ? gn : eps);
+        } else {                           // eq. 17, step capped at alpha x
+            const Tp stp = bv > Tp(0) ? simt::dev_div(av, bv) : Tp(0);
+            const Tp cap = alpha * xr;
+            d = xr + (stp < cap ? stp : cap);
+        }
+        xd.v[i] = r + i < R ? d : Tp(0);
+        den += cs[r + i] * xd.v[i];
     }
+    if (in) store4(Xm + o * R4 + r, xm);
+    if (MU) return;
+    const Tp tot = group_sum<LPN>(den);    // eq. 10
+    const Tp sc = live && tot > Tp(0) ? (Tp)vsum[o] / tot : Tp(1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) xd.v[i] *= sc;
+    if (in) store4(Xd + o * R4 + r, xd);
 }
 
 // Pass 2 (steps 7-9, 12-14 on the non-zeros of one segment): the partial sums
-// dseg[2 g] = sum_{v>0} -v log z_MU and dseg[2 g + 1] = sum_{v>0} -v log z_DNA.  The term
-// of non-zero k is added by lane (k - k0) mod U in the element type (at most SEG / U terms
-// per lane: float64 arithmetic is slow on this GPU), then the lanes' sums are added in
-// float64 by the fixed butterfly.
-template <typename Tp, int RPL>
+// sum_{v>0} -v log z_MU and sum_{v>0} -v log z_DNA as the pair g of dseg.  A lane adds
+// the terms of its non-zeros in the element type (at most SEG / U of them), the lanes' sums
+// are added with their rounding errors.
+template <typename Tp, int LPN>
 __global__ void __launch_bounds__(WARPS * 32)
-    k_sp_pass2(View v, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
-               const Tp* __restrict__ Yg, const Tp* __restrict__ Xmu,
-               const Tp* __restrict__ Xdna, double* __restrict__ dseg) {
-    const int lane = threadIdx.x & 31;
+    k_sp_pass2(int64_t R4, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
+               const Tp* __restrict__ Yr, const Tp* __restrict__ Xm, const Tp* __restrict__ Xd,
+               double* __restrict__ dseg) {
+    const int lane = threadIdx.x & 31, sub = lane % LPN, r = 4 * sub;
     const int64_t g = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
     if (g >= sg.n) return;
-    const int64_t R = v.R, O = v.O, o = sg.col[g];
-    Tp xm[RPL], xd[RPL];
-#pragma unroll
-    for (int j = 0; j < RPL; ++j) {
-        const int64_t r = lane + 32 * j;
-        xm[j] = r < R ? Xmu[r * O + o] : Tp(0);
-        xd[j] = r < R ? Xdna[r * O + o] : Tp(0);
-    }
+    const int64_t k0 = sg.k0[g], k1 = sg.k1[g], col = sg.col[g];
+    const Four<Tp> xm = row4(Xm, col, R4, r), xd = row4(Xd, col, R4, r);
     Tp lm_t = Tp(0), ld_t = Tp(0);
-    constexpr int LOG2U = U == 8 ? 4 : (U == 4 ? 3 : (U == 16 ? 5 : -1));
-    static_assert(LOG2U > 0, "U: 4, 8 or 16");
-    // lane l finishes value l >> (5 - LOG2U) of the 2U: the MU z of non-zero u (values
-    // 0 .. U - 1) or the Newton z (U .. 2U - 1); one lane of each value adds its term
-    const int vi = lane >> (5 - LOG2U), ul = vi & (U - 1);
-    const bool adds = (lane & ((1 << (5 - LOG2U)) - 1)) == 0;
-    for_nonzeros<Tp, RPL>(sg.k0[g], sg.k1[g], lane, R, idx, val, Yg,
-                          [&](const Chunk<Tp>& c, int base, Tp (&y)[U][RPL]) {
-        Tp p[2 * U];
+    for_nonzeros<LPN>(k0, k1, lane, R4, idx, val, Yr,
+                      [&](const Chunk<Tp>& c, int first, const Four<Tp> (&y)[U]) {
+        if constexpr (LPN >= 2 * U) {
+            // a lane finishes one z: the MU z of non-zero u (values 0 .. U - 1) or the Newton
+            // z (U .. 2U - 1); one lane of each value adds its term
+            constexpr int STEP = LPN / (2 * U);
+            Tp p[2 * U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            p[u] = Tp(0);
-            p[U + u] = Tp(0);
+            for (int u = 0; u < U; ++u) {
+                p[u] = dot4(y[u], xm);
+                p[U + u] = dot4(y[u], xd);
+            }
+            const Tp z = scatter_sum<LPN, 2 * U>(p, lane);
+            const int vi = sub / STEP;
+            const Tp vl = __shfl_sync(0xffffffffu, c.v, first + vi % U);
+            if (sub % STEP == 0 && vl > Tp(0)) {   // log of a non-positive z: NaN / -inf
+                const Tp t = vl * log(z);
+                if (vi < U) lm_t -= t; else ld_t -= t;
+            }
+        } else {   // as many lanes as non-zeros: a lane finishes both z of one
+            static_assert(LPN == U || LPN >= 2 * U, "");
+            Tp p[U], d[U];
 #pragma unroll
-            for (int j = 0; j < RPL; ++j) {
-                p[u] += y[u][j] * xm[j];
-                p[U + u] += y[u][j] * xd[j];
+            for (int u = 0; u < U; ++u) {
+                p[u] = dot4(y[u], xm);
+                d[u] = dot4(y[u], xd);
+            }
+            const Tp zm = scatter_sum<LPN, U>(p, lane), zd = scatter_sum<LPN, U>(d, lane);
+            const Tp vl = __shfl_sync(0xffffffffu, c.v, first + sub);
+            if (vl > Tp(0)) {
+                lm_t -= vl * log(zm);
+                ld_t -= vl * log(zd);
             }
         }
-        const Tp z = scatter_sum<Tp, 2 * U>(p, lane);
-        const Tp vl = __shfl_sync(0xffffffffu, c.v, base + ul);
-        if (adds && vl > Tp(0)) {   // log of a non-positive z gives NaN / -inf
-            const Tp t = vl * log(z);
-            if (vi < U) lm_t -= t; else ld_t -= t;
-        }
     });
-    const double lm = warp_sum((double)lm_t);
-    const double ld = warp_sum((double)ld_t);
-    if (lane == 0) {
-        dseg[2 * g] = lm;
-        dseg[2 * g + 1] = ld;
-    }
+    Sum<Tp> lm, ld;
+    lm.add(lm_t);
+    ld.add(ld_t);
+    lm = group_add<32>(lm);
+    ld = group_add<32>(ld);
+    if (lane == 0) store_costs(dseg, g, lm, ld);
 }
 
-// Per view column o: the segments' partial costs in order, plus sum_s z = sum_r c0_r x(r, o)
-// of each candidate, into dpart[o] (MU) and dpart[O + o] (Newton).
-template <typename Tp, int RPL>
+// The cost of each candidate (the segments' sums in order, sum_s z = sum_r c0_r x(r, o), and
+// reg sum_r x(r, o), the eq. 5 / eq. 4 penalty), the selection (Newton iff cheaper), the kept
+// row into X, and fpart[blk][r] = sum over the CTA's 32 columns of the new x(r, o) (float64;
+// the layout of k_select_fused).  MU: the row of Xm is kept.  A group of LPN lanes per column.
+template <typename Tp, int LPN, bool MU>
 __global__ void __launch_bounds__(WARPS * 32)
-    k_sp_reduce_cost(int64_t O, int64_t R, const int64_t* __restrict__ sptr,
-                     const double* __restrict__ dseg, const Tp* __restrict__ Xmu,
-                     const Tp* __restrict__ Xdna, const double* __restrict__ c0,
-                     double* __restrict__ dpart, int* __restrict__ status) {
-    const int lane = threadIdx.x & 31;
-    const int64_t o = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
-    if (o >= O) return;
-    double zm = 0.0, zd = 0.0;
+    k_sp_select(View v, int64_t R4, const int64_t* __restrict__ sptr,
+                const double* __restrict__ dseg, const Tp* __restrict__ Xm,
+                const Tp* __restrict__ Xd, const double* __restrict__ c0,
+                uint8_t* __restrict__ choice, double* __restrict__ dfin,
+                double* __restrict__ fpart, double reg, int* __restrict__ status) {
+    constexpr int G = 32 / LPN, NK = 4 / G;   // columns of a warp at once, rounds
+    __shared__ Tp xs[4 * LPN][33];
+    __shared__ Tp ch[4 * LPN], cl[4 * LPN];   // c0 = ch + cl
+    __shared__ Sum<Tp> sums[4][32];           // per column: sum z and sum x of both candidates
+    __shared__ int kept[32];
+    const int64_t R = v.R, O = v.O, o0 = (int64_t)blockIdx.x * 32;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, sub = lane % LPN, r = 4 * sub;
+    Four<Tp> x[NK], xd[NK];
+    const Four<Tp> zero{{Tp(0), Tp(0), Tp(0), Tp(0)}};
 #pragma unroll
-    for (int j = 0; j < RPL; ++j) {
-        const int64_t r = lane + 32 * j;
-        if (r < R) {
-            zm += c0[r] * (double)Xmu[r * O + o];
-            zd += c0[r] * (double)Xdna[r * O + o];
+    for (int k = 0; k < NK; ++k) {
+        const int64_t o = o0 + 4 * w + k * G + lane / LPN;
+        const bool in = o < O && r < R4;
+        x[k] = in ? load4(Xm + o * R4 + r) : zero;
+        if (!MU) xd[k] = in ? load4(Xd + o * R4 + r) : zero;
+    }
+    if (!MU) {
+        for (int k = tid; k < 4 * LPN; k += WARPS * 32) {
+            const double t = k < R ? c0[k] : 0.0;
+            ch[k] = (Tp)t;
+            cl[k] = (Tp)(t - (double)ch[k]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            Sum<Tp> zm, zd, pm, pd;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                zm.add_product(ch[r + i], cl[r + i], x[k].v[i]);
+                zd.add_product(ch[r + i], cl[r + i], xd[k].v[i]);
+            }
+            zm = group_add<LPN>(zm);
+            zd = group_add<LPN>(zd);
+            if (reg != 0.0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    pm.add(x[k].v[i]);
+                    pd.add(xd[k].v[i]);
+                }
+                pm = group_add<LPN>(pm);
+                pd = group_add<LPN>(pd);
+            }
+            if (sub == 0) {
+                const int col = 4 * w + k * G + lane / LPN;
+                sums[0][col] = zm;
+                sums[1][col] = zd;
+                sums[2][col] = pm;
+                sums[3][col] = pd;
+            }
+        }
+        __syncthreads();
+        if (w == 0) {   // lane = column: float64 for 32 columns at once
+            const int64_t o = o0 + lane;
+            bool newton = false;
+            if (o < O) {
+                Sum<Tp> lm, ld;
+                const int64_t g1 = sptr[o + 1];
+#pragma unroll 16
+                for (int64_t g = sptr[o]; g < g1; ++g) add_costs(dseg, g, lm, ld);
+                double dm = lm.value() + sums[0][lane].value();
+                double dd = ld.value() + sums[1][lane].value();
+                if (reg != 0.0) {
+                    dm += reg * sums[2][lane].value();
+                    dd += reg * sums[3][lane].value();
+                }
+                newton = dd < dm;
+                choice[o] = newton ? 1 : 0;
+                dfin[o] = dm;
+                dfin[O + o] = dd;
+                if (!isfinite(dm) || !isfinite(dd)) atomicOr(status, STATUS_NONFINITE);
+            }
+            kept[lane] = newton;
+        }
+        __syncthreads();
+    }
+    Tp* __restrict__ X = static_cast<Tp*>(v.X);
+    const bool rows = v.xo != 1;   // X has contiguous rows of r
+    const bool wide = R4 == R && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int col = 4 * w + k * G + lane / LPN;
+        const int64_t o = o0 + col;
+        if (!MU && kept[col]) x[k] = xd[k];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) xs[r + i][col] = x[k].v[i];
+        if (rows && o < O && r < R) {
+            if (wide) store4(X + o * v.xo + r, x[k]);
+            else
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (r + i < R) X[o * v.xo + r + i] = x[k].v[i];
         }
     }
-    zm = warp_sum(zm);
-    zd = warp_sum(zd);
-    if (lane == 0) {
-        double lm = 0.0, ld = 0.0;
-        for (int64_t g = sptr[o]; g < sptr[o + 1]; ++g) {
-            lm += dseg[2 * g];
-            ld += dseg[2 * g + 1];
-        }
-        const double dm = lm + zm, dd = ld + zd;
-        dpart[o] = dm;
-        dpart[O + o] = dd;
-        if (!isfinite(dm) || !isfinite(dd)) atomicOr(status, STATUS_NONFINITE);
+    __syncthreads();
+    if (!rows && o0 + lane < O)
+#pragma unroll 4
+        for (int64_t q = w; q < R; q += WARPS) X[q * v.xr + o0 + lane] = xs[q][lane];
+    for (int64_t q = tid; q < R; q += WARPS * 32) {
+        Tp s = Tp(0);
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i) s += xs[q][i];
+        fpart[(int64_t)blockIdx.x * R + q] = (double)s;
     }
 }
 
 // d_KL (eq. 1) of the H view, per segment: sum over its non-zeros of v log(v / z) - v into
 // dseg[g] (float64).
-template <typename Tp, int RPL>
+template <typename Tp, int LPN>
 __global__ void __launch_bounds__(WARPS * 32)
-    k_sp_kl(View v, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
-            const Tp* __restrict__ Yg, double* __restrict__ dseg) {
-    const int lane = threadIdx.x & 31;
+    k_sp_kl(int64_t R4, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
+            const Tp* __restrict__ Yr, const Tp* __restrict__ Xr, double* __restrict__ dseg) {
+    constexpr int STEP = LPN / U;
+    const int lane = threadIdx.x & 31, sub = lane % LPN, r = 4 * sub;
     const int64_t g = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
     if (g >= sg.n) return;
-    const int64_t R = v.R, o = sg.col[g];
-    const Tp* __restrict__ X = static_cast<const Tp*>(v.X);
-    Tp x[RPL];
-#pragma unroll
-    for (int j = 0; j < RPL; ++j) {
-        const int64_t r = lane + 32 * j;
-        x[j] = r < R ? X[r * v.xr + o * v.xo] : Tp(0);
-    }
-    Tp acc_t = Tp(0);   // the element type within the segment, float64 across lanes
-    constexpr int LOGU = U == 8 ? 3 : (U == 4 ? 2 : (U == 16 ? 4 : -1));
-    const int ul = lane >> (5 - LOGU);
-    const bool adds = (lane & ((1 << (5 - LOGU)) - 1)) == 0;
-    for_nonzeros<Tp, RPL>(sg.k0[g], sg.k1[g], lane, R, idx, val, Yg,
-                          [&](const Chunk<Tp>& c, int base, Tp (&y)[U][RPL]) {
+    const int64_t k0 = sg.k0[g], k1 = sg.k1[g], col = sg.col[g];
+    const Four<Tp> x = row4(Xr, col, R4, r);
+    Tp acc_t = Tp(0);   // the element type within the segment
+    for_nonzeros<LPN>(k0, k1, lane, R4, idx, val, Yr,
+                      [&](const Chunk<Tp>& c, int first, const Four<Tp> (&y)[U]) {
         Tp p[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            p[u] = Tp(0);
-#pragma unroll
-            for (int j = 0; j < RPL; ++j) p[u] += y[u][j] * x[j];
-        }
-        const Tp z = scatter_sum<Tp, U>(p, lane);
-        const Tp vl = __shfl_sync(0xffffffffu, c.v, base + ul);
-        if (adds && vl > Tp(0)) acc_t += vl * log(vl / z) - vl;
+        for (int u = 0; u < U; ++u) p[u] = dot4(y[u], x);
+        const Tp z = scatter_sum<LPN, U>(p, lane);
+        const Tp vl = __shfl_sync(0xffffffffu, c.v, first + sub / STEP);
+        if (sub % STEP == 0 && vl > Tp(0)) acc_t += vl * log(vl / z) - vl;
     });
-    const double acc = warp_sum((double)acc_t);
-    if (lane == 0) dseg[g] = acc;
+    Sum<Tp> acc;
+    acc.add(acc_t);
+    const double t = group_add<32>(acc).value();
+    if (lane == 0) dseg[g] = t;
 }
 
 // Per column t of the H view: its segments' d_KL terms plus sum_n z_nt = sum_r c0_r h(r, t)
-// into part[t].
-template <typename Tp, int RPL>
+// into part[t].  A warp per column.
+template <typename Tp>
 __global__ void __launch_bounds__(WARPS * 32)
-    k_sp_reduce_kl(View v, const int64_t* __restrict__ sptr, const double* __restrict__ dseg,
+    k_sp_reduce_kl(int64_t O, int64_t R, int64_t R4, const int64_t* __restrict__ sptr,
+                   const double* __restrict__ dseg, const Tp* __restrict__ Xr,
                    const double* __restrict__ c0, double* __restrict__ part,
                    int* __restrict__ status) {
     const int lane = threadIdx.x & 31;
     const int64_t o = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
-    if (o >= v.O) return;
-    const Tp* __restrict__ X = static_cast<const Tp*>(v.X);
+    if (o >= O) return;
     double zs = 0.0;
+    for (int64_t r = lane; r < R; r += 32) zs += c0[r] * (double)Xr[o * R4 + r];
 #pragma unroll
-    for (int j = 0; j < RPL; ++j) {
-        const int64_t r = lane + 32 * j;
-        if (r < v.R) zs += c0[r] * (double)X[r * v.xr + o * v.xo];
-    }
-    zs = warp_sum(zs);
+    for (int m = 16; m > 0; m >>= 1) zs += __shfl_xor_sync(0xffffffffu, zs, m);
     if (lane == 0) {
         double acc = 0.0;
         for (int64_t g = sptr[o]; g < sptr[o + 1]; ++g) acc += dseg[g];
@@ -381,11 +593,24 @@ __global__ void __launch_bounds__(WARPS * 32)
     }
 }
 
-// Y^t: out[t * R + r] = H[r * T + t] (R x T row-major in, T x R row-major out), through
-// 32 x 32 shared-memory tiles so both sides stay coalesced.  CTA (32, 8).
+// out[i][r] = in(i, r) for r < R, zeros up to ld: the rows of W (in[i * R + r]).
+template <typename Tp>
+__global__ void __launch_bounds__(256) k_pad_rows(const Tp* __restrict__ in, int64_t n, int64_t R,
+                                                  int64_t ld, Tp* __restrict__ out) {
+    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < n * ld;
+         e += (int64_t)gridDim.x * 256) {
+        const int64_t i = e / ld, r = e % ld;
+        out[e] = r < R ? in[i * R + r] : Tp(0);
+    }
+}
+
+// Rows of a factor stored along the other index: out[c * ld + r] = in[r * cols + c] (rows x
+// cols row-major in), zeros for rows <= r < ld, through 32 x 32 shared-memory tiles so both
+// sides stay coalesced.  CTA (32, 8).
 template <typename Tp>
 __global__ void __launch_bounds__(256) k_transpose(const Tp* __restrict__ in, int64_t rows,
-                                                   int64_t cols, Tp* __restrict__ out) {
+                                                   int64_t cols, int64_t ld,
+                                                   Tp* __restrict__ out) {
     __shared__ Tp tile[32][33];
     const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 32;
     for (int i = threadIdx.y; i < 32; i += 8) {
@@ -395,7 +620,7 @@ __global__ void __launch_bounds__(256) k_transpose(const Tp* __restrict__ in, in
     __syncthreads();
     for (int i = threadIdx.y; i < 32; i += 8) {
         const int64_t c = c0 + i, r = r0 + threadIdx.x;
-        if (c < cols && r < rows) out[c * rows + r] = tile[threadIdx.x][i];
+        if (c < cols && r < ld) out[c * ld + r] = tile[threadIdx.x][i];
     }
 }
 
