@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "dna.h"
 
 namespace dna {
@@ -19,6 +21,41 @@ inline int after_launch() {
     ++launch_count();
     return cudaGetLastError() == cudaSuccess ? DNA_OK : DNA_ERR_CUDA;
 }
+
+#ifdef __CUDACC__
+// Kernels of an iteration are launched with programmatic stream serialisation: the next
+// kernel's launch, and the CTAs that find room, need not wait for this one's end.  Each such
+// kernel calls pdl_wait() before it touches global memory that another kernel writes; it
+// returns when the kernel before is done and visible (each waits for the one before it, so
+// everything earlier is done as well).  pdl_next() lets the kernel after this one be placed
+// from the moment every CTA of this one has called it.  The short kernels between the passes
+// call it at their start; the passes do not, unless they leave SMs idle, because CTAs placed
+// behind a full grid crowd on the SMs that end first (counts matrices 552, 345 us an
+// iteration in the FP32 and BF16 tensor-core forms without any of this, 554, 348 with it in
+// every kernel, 549, 342 as it is).  Other sizes: N=256 T=512 R=16 62 -> 57 us, N=4096 T=165
+// R=80 119 -> 115, sparse 36771 x 10212 (direct launches) 350 -> 298.  The grouped kernels,
+// long and many-waved, were slower with it (1220 -> 1250 us) and are launched plainly.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// The launch of a kernel that calls pdl_wait(); errors show in cudaGetLastError (after_launch).
+template <typename... P, typename... A>
+void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... a) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, std::forward<A>(a)...);
+}
+#endif
 
 // Partial-sum slots of the two-level factor sums.
 constexpr int FSUM_SPLITS = 64;

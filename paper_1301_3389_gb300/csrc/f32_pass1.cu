@@ -9,6 +9,7 @@ template <int RPT, bool WITH_B, int SG>
 __global__ void __launch_bounds__(NT, 2)
     k_pass1_f2(View v, float* __restrict__ Apart, float* __restrict__ Bpart, int64_t s_per,
                int* __restrict__ status) {
+    pdl_wait();
     extern __shared__ __align__(16) float smem_f2[];
     pass1_tile<RPT, WITH_B, SG>(v, Apart, Bpart, s_per, status, blockIdx.x, blockIdx.y, smem_f2);
 }
@@ -22,7 +23,7 @@ static int launch(const View& v, float* A, float* B, int splits, int64_t s_per, 
         cudaSuccess)
         return DNA_ERR_CUDA;
     const dim3 grid((unsigned)((v.O + OB - 1) / OB), (unsigned)splits);
-    k<<<grid, NT, smem, st>>>(v, A, B, s_per, status);
+    dna::launch_pdl(k, grid, dim3(NT), smem, st, v, A, B, s_per, status);
     return after_launch();
 }
 

@@ -8,6 +8,7 @@ template <int RPT, int NC, bool FULL>
 __global__ void __launch_bounds__(NT, 2)
     k_pass2_f2(View v, const float* __restrict__ X0, const float* __restrict__ X1, int64_t xr,
                int64_t xo, double* __restrict__ dpart, int64_t s_per, int* __restrict__ status) {
+    pdl_wait();
     extern __shared__ __align__(16) float smem_f2[];
     pass2_tile<RPT, NC, FULL>(v, X0, X1, xr, xo, dpart, s_per, status, blockIdx.x, blockIdx.y,
                               smem_f2);
@@ -22,7 +23,7 @@ static int launch(const View& v, const float* X0, const float* X1, int64_t xr, i
         cudaSuccess)
         return DNA_ERR_CUDA;
     const dim3 grid((unsigned)((v.O + OB - 1) / OB), (unsigned)splits);
-    k<<<grid, NT, smem, st>>>(v, X0, X1, xr, xo, dpart, s_per, status);
+    dna::launch_pdl(k, grid, dim3(NT), smem, st, v, X0, X1, xr, xo, dpart, s_per, status);
     return after_launch();
 }
 
@@ -65,6 +66,7 @@ template <int RPT>
 __global__ void __launch_bounds__(NT, 2)
     k_grad_v_f2(View v, float scale, float* __restrict__ dV, int64_t ldd,
                 int* __restrict__ status) {
+    pdl_wait();
     using H = Tiles<RPT>;
     extern __shared__ __align__(16) float smem_f2[];
     float* Xs = smem_f2;
@@ -120,7 +122,7 @@ static int launch_grad(const View& v, float scale, float* dV, int64_t ldd, int* 
         cudaSuccess)
         return DNA_ERR_CUDA;
     const dim3 grid((unsigned)((v.O + OB - 1) / OB), (unsigned)((v.S + SB - 1) / SB));
-    k<<<grid, NT, smem, st>>>(v, scale, dV, ldd, status);
+    dna::launch_pdl(k, grid, dim3(NT), smem, st, v, scale, dV, ldd, status);
     return after_launch();
 }
 

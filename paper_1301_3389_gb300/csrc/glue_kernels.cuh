@@ -53,6 +53,8 @@ __global__ void __launch_bounds__(1024) k_cand_fused(View v, const double* __res
                                                     Tp eps, Tp alpha, bf16* __restrict__ Xmk,
                                                     bf16* __restrict__ Xdk, int64_t rp,
                                                     int64_t plane) {
+    pdl_wait();
+    pdl_next();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t R = v.R, O = v.O;
     Tp* red = reinterpret_cast<Tp*>(smem_raw);                    // [TY][TO]
@@ -334,6 +336,8 @@ __global__ void __launch_bounds__(512) k_cand_reg(View v, const double* __restri
                                                   Tp eps, Tp alpha, bf16* __restrict__ Xmk,
                                                   bf16* __restrict__ Xdk, int64_t rp,
                                                   int64_t plane) {
+    pdl_wait();
+    pdl_next();
     cand_reg_tile<Tp, BF, RS>(v, c, Apart, Bpart, splits, Xmu, Xdna, eps, alpha, Xmk, Xdk, rp,
                               plane, blockIdx.x);
 }
@@ -345,6 +349,8 @@ __global__ void __launch_bounds__(512) k_cand_reg(View v, const double* __restri
 template <typename Tp, int VEC>
 __global__ void __launch_bounds__(256) k_split_sum(Tp* __restrict__ A, Tp* __restrict__ B,
                                                    int64_t n, int splits) {
+    pdl_wait();
+    pdl_next();
     Tp* M = blockIdx.y ? B : A;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * VEC;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * VEC; i < n; i += stride) {
@@ -373,6 +379,8 @@ __global__ void __launch_bounds__(256) k_split_sum(Tp* __restrict__ A, Tp* __res
 template <typename Tp, int VEC>
 __global__ void __launch_bounds__(256) k_split_sum_par(Tp* __restrict__ A, Tp* __restrict__ B,
                                                        int64_t n, int splits) {
+    pdl_wait();
+    pdl_next();
     __shared__ Tp red[8][32][VEC];
     Tp* M = blockIdx.y ? B : A;
     const int tx = threadIdx.x, ty = threadIdx.y;
@@ -429,6 +437,8 @@ __global__ void __launch_bounds__(256) k_select_fused(View v, const Tp* __restri
                                                       double* __restrict__ fpart, double reg,
                                                       const double* __restrict__ dcur,
                                                       int cur_splits) {
+    pdl_wait();
+    pdl_next();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t R = v.R, O = v.O;
     Tp* xs = reinterpret_cast<Tp*>(smem_raw);                   // [R][TO + 1]
@@ -535,6 +545,8 @@ template <typename Tp>
 __global__ void __launch_bounds__(256) k_mu_fused(View v, const double* __restrict__ c,
                                                   const Tp* __restrict__ Apart, int splits,
                                                   double* __restrict__ fpart) {
+    pdl_wait();
+    pdl_next();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t R = v.R, O = v.O;
     Tp* xs = reinterpret_cast<Tp*>(smem_raw);                   // [R][TO + 1]
@@ -619,6 +631,8 @@ struct OpsArgs {
 // the padding of the operand buffers is rewritten as zeros.
 template <typename Tp, int RT>
 __global__ void __launch_bounds__(256, 4) k_scale_ops(OpsArgs a) {
+    pdl_wait();
+    pdl_next();
     constexpr int NL = RT / 8;                 // elements per thread
     __shared__ Tp tile[RT][TO + 1];            // [r][i]
     __shared__ Tp fr[RT];

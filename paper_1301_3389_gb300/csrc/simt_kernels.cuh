@@ -244,6 +244,7 @@ template <typename Tp, int RB, bool WITH_B>
 __global__ void __launch_bounds__(NT, sizeof(Tp) == 4 ? 2 : 1)
     k_pass1(View v, Tp* __restrict__ Apart, Tp* __restrict__ Bpart, int64_t s_per,
             int* __restrict__ status, double* __restrict__ dcur) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pass1_tile<Tp, RB, WITH_B>(v, Apart, Bpart, s_per, status, blockIdx.x, blockIdx.y, blockIdx.z,
                                smem_raw, dcur);
@@ -362,6 +363,7 @@ template <typename Tp, int RB, int NC, bool FULL>
 __global__ void __launch_bounds__(NT, sizeof(Tp) == 4 ? 2 : 1)
     k_pass2(View v, const Tp* __restrict__ X0, const Tp* __restrict__ X1, int64_t xr, int64_t xo,
             double* __restrict__ dpart, int64_t s_per, int* __restrict__ status) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pass2_tile<Tp, RB, NC, FULL>(v, X0, X1, xr, xo, dpart, s_per, status, blockIdx.x, blockIdx.y,
                                  smem_raw);
@@ -557,6 +559,7 @@ __global__ void __launch_bounds__(256) k_grad_x(View v, const double* __restrict
 template <typename Tp, int RB>
 __global__ void __launch_bounds__(NT) k_grad_v(View v, double scale, Tp* __restrict__ dV,
                                                int64_t ldd, int* __restrict__ status) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Tp* Yt = reinterpret_cast<Tp*>(smem_raw);  // [RB][LD]
     Tp* Xs = Yt + RB * LD;                     // [RB][LD]
@@ -750,6 +753,7 @@ __global__ void __launch_bounds__(NT)
     k_adj_gemm(View v, const Tp* __restrict__ Abar, const Tp* __restrict__ Bbar,
                const double* __restrict__ vs, Tp* __restrict__ Hpart, Tp* __restrict__ Vbar,
                int64_t ldvb, int64_t s_per, int* __restrict__ status) {
+    pdl_wait();
     using C = AdjCfg<Tp, RB>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Tp* Xs = reinterpret_cast<Tp*>(smem_raw);  // [RB][LD] x(r, o)
@@ -870,6 +874,7 @@ template <typename Tp, int RB>
 __global__ void __launch_bounds__(NT)
     k_adj_wgrad(View v, const Tp* __restrict__ Abar, const Tp* __restrict__ Bbar,
                 Tp* __restrict__ Wpart, int64_t o_per, int* __restrict__ status) {
+    pdl_wait();
     using C = WgradCfg<Tp, RB>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Tp* Xs = reinterpret_cast<Tp*>(smem_raw);  // [RB][LD] x(r, o)
@@ -1076,6 +1081,8 @@ __global__ void __launch_bounds__(256) k_colsum_small(const double* __restrict__
                                                       int nsplit, int64_t R, double reg,
                                                       double* __restrict__ out, bool guard,
                                                       double* __restrict__ next = nullptr) {
+    pdl_wait();
+    pdl_next();
     __shared__ double red[256];
     const int64_t r = blockIdx.x;
     double t = 0.0;

@@ -37,11 +37,11 @@ int pass1_rb(const View& v, Tp* A, Tp* B, int splits, int64_t s_per, bool with_b
     if (with_b) {
         auto k = k_pass1<Tp, RB, true>;
         if (prep_smem(k, smem)) return DNA_ERR_CUDA;
-        k<<<grid, NT, smem, st>>>(v, A, B, s_per, status, dcur);
+        dna::launch_pdl(k, grid, dim3(NT), smem, st, v, A, B, s_per, status, dcur);
     } else {
         auto k = k_pass1<Tp, RB, false>;
         if (prep_smem(k, smem)) return DNA_ERR_CUDA;
-        k<<<grid, NT, smem, st>>>(v, A, B, s_per, status, dcur);
+        dna::launch_pdl(k, grid, dim3(NT), smem, st, v, A, B, s_per, status, dcur);
     }
     return launch_status();
 }
@@ -53,7 +53,7 @@ int pass2_rb(const View& v, const Tp* X0, const Tp* X1, int64_t xr, int64_t xo, 
     auto k = k_pass2<Tp, RB, NC, FULL>;
     if (prep_smem(k, smem)) return DNA_ERR_CUDA;
     dim3 grid((unsigned)((v.O + OB - 1) / OB), (unsigned)splits);
-    k<<<grid, NT, smem, st>>>(v, X0, X1, xr, xo, dpart, s_per, status);
+    dna::launch_pdl(k, grid, dim3(NT), smem, st, v, X0, X1, xr, xo, dpart, s_per, status);
     return launch_status();
 }
 
@@ -218,7 +218,7 @@ int grad_v_rb(const View& v, double scale, Tp* dV, int64_t ldd, int* status, cud
     auto k = k_grad_v<Tp, RB>;
     if (prep_smem(k, smem)) return DNA_ERR_CUDA;
     dim3 grid((unsigned)((v.O + OB - 1) / OB), (unsigned)((v.S + SB - 1) / SB));
-    k<<<grid, NT, smem, st>>>(v, scale, dV, ldd, status);
+    dna::launch_pdl(k, grid, dim3(NT), smem, st, v, scale, dV, ldd, status);
     return launch_status();
 }
 }  // namespace simt
@@ -243,7 +243,8 @@ int adj_gemm_rb(const View& v, const Tp* Abar, const Tp* Bbar, const double* vs,
     auto k = k_adj_gemm<Tp, RB>;
     if (prep_smem(k, smem)) return DNA_ERR_CUDA;
     dim3 grid((unsigned)((v.O + OB - 1) / OB), (unsigned)splits);
-    k<<<grid, NT, smem, st>>>(v, Abar, Bbar, vs, Hpart, Vbar, ldvb, s_per, status);
+    dna::launch_pdl(k, grid, dim3(NT), smem, st, v, Abar, Bbar, vs, Hpart, Vbar, ldvb, s_per,
+                    status);
     return launch_status();
 }
 }  // namespace simt
@@ -288,7 +289,7 @@ int adj_wgrad_rb(const View& v, const Tp* Abar, const Tp* Bbar, Tp* Wpart, int w
     auto k = k_adj_wgrad<Tp, RB>;
     if (prep_smem(k, smem)) return DNA_ERR_CUDA;
     dim3 grid((unsigned)((v.S + SB - 1) / SB), (unsigned)wsplits);
-    k<<<grid, NT, smem, st>>>(v, Abar, Bbar, Wpart, o_per, status);
+    dna::launch_pdl(k, grid, dim3(NT), smem, st, v, Abar, Bbar, Wpart, o_per, status);
     return launch_status();
 }
 }  // namespace simt
@@ -334,18 +335,18 @@ int Simt<Tp>::cand_fused(const View& v, const double* c, const Tp* A, const Tp* 
                 auto* bm = static_cast<glue::bf16*>(Xmk);
                 auto* bd = static_cast<glue::bf16*>(Xdk);
                 if (rs == 8)
-                    glue::k_cand_reg<Tp, true, 8><<<grid, blk, 0, st>>>(
-                        v, c, A, B, splits, Xmu, Xdna, (Tp)eps, (Tp)alpha, bm, bd, rp, plane);
+                    dna::launch_pdl(glue::k_cand_reg<Tp, true, 8>, grid, blk, 0, st, v, c, A, B,
+                                    splits, Xmu, Xdna, (Tp)eps, (Tp)alpha, bm, bd, rp, plane);
                 else
-                    glue::k_cand_reg<Tp, true, 16><<<grid, blk, 0, st>>>(
-                        v, c, A, B, splits, Xmu, Xdna, (Tp)eps, (Tp)alpha, bm, bd, rp, plane);
+                    dna::launch_pdl(glue::k_cand_reg<Tp, true, 16>, grid, blk, 0, st, v, c, A, B,
+                                    splits, Xmu, Xdna, (Tp)eps, (Tp)alpha, bm, bd, rp, plane);
             }
         } else if (rs == 8) {
-            glue::k_cand_reg<Tp, false, 8><<<grid, blk, 0, st>>>(
-                v, c, A, B, splits, Xmu, Xdna, (Tp)eps, (Tp)alpha, nullptr, nullptr, 0, 0);
+            dna::launch_pdl(glue::k_cand_reg<Tp, false, 8>, grid, blk, 0, st, v, c, A, B, splits,
+                            Xmu, Xdna, (Tp)eps, (Tp)alpha, nullptr, nullptr, 0, 0);
         } else {
-            glue::k_cand_reg<Tp, false, 16><<<grid, blk, 0, st>>>(
-                v, c, A, B, splits, Xmu, Xdna, (Tp)eps, (Tp)alpha, nullptr, nullptr, 0, 0);
+            dna::launch_pdl(glue::k_cand_reg<Tp, false, 16>, grid, blk, 0, st, v, c, A, B, splits,
+                            Xmu, Xdna, (Tp)eps, (Tp)alpha, nullptr, nullptr, 0, 0);
         }
         return simt::launch_status();
     }
@@ -354,15 +355,15 @@ int Simt<Tp>::cand_fused(const View& v, const double* c, const Tp* A, const Tp* 
         if constexpr (sizeof(Tp) == 4) {
             auto k = glue::k_cand_fused<Tp, true>;
             if (simt::prep_smem(k, smem)) return DNA_ERR_CUDA;
-            k<<<grid, dim3(32, glue::TY), smem, st>>>(v, c, A, B, splits, Xmu, Xdna, (Tp)eps, (Tp)alpha,
-                                               static_cast<glue::bf16*>(Xmk),
-                                               static_cast<glue::bf16*>(Xdk), rp, plane);
+            dna::launch_pdl(k, grid, dim3(32, glue::TY), smem, st, v, c, A, B, splits, Xmu, Xdna,
+                            (Tp)eps, (Tp)alpha, static_cast<glue::bf16*>(Xmk),
+                            static_cast<glue::bf16*>(Xdk), rp, plane);
         }
     } else {
         auto k = glue::k_cand_fused<Tp, false>;
         if (simt::prep_smem(k, smem)) return DNA_ERR_CUDA;
-        k<<<grid, dim3(32, glue::TY), smem, st>>>(v, c, A, B, splits, Xmu, Xdna, (Tp)eps, (Tp)alpha,
-                                           nullptr, nullptr, 0, 0);
+        dna::launch_pdl(k, grid, dim3(32, glue::TY), smem, st, v, c, A, B, splits, Xmu, Xdna,
+                        (Tp)eps, (Tp)alpha, nullptr, nullptr, 0, 0);
     }
     return simt::launch_status();
 }
@@ -383,20 +384,21 @@ int Simt<Tp>::split_sum(Tp* A, Tp* B, int64_t R, int64_t O, int splits, cudaStre
         const dim3 grid((unsigned)((work + 31) / 32), ab);
         if constexpr (sizeof(Tp) == 4)
             if (vec == 4) {
-                glue::k_split_sum_par<Tp, 4><<<grid, dim3(32, 8), 0, st>>>(A, B, n, splits);
+                dna::launch_pdl(glue::k_split_sum_par<Tp, 4>, grid, dim3(32, 8), 0, st, A, B, n,
+                                splits);
                 return simt::launch_status();
             }
-        glue::k_split_sum_par<Tp, 1><<<grid, dim3(32, 8), 0, st>>>(A, B, n, splits);
+        dna::launch_pdl(glue::k_split_sum_par<Tp, 1>, grid, dim3(32, 8), 0, st, A, B, n, splits);
         return simt::launch_status();
     }
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 8));
     const dim3 grid((unsigned)blocks, ab);
     if constexpr (sizeof(Tp) == 4)
         if (vec == 4) {
-            glue::k_split_sum<Tp, 4><<<grid, 256, 0, st>>>(A, B, n, splits);
+            dna::launch_pdl(glue::k_split_sum<Tp, 4>, grid, dim3(256), 0, st, A, B, n, splits);
             return simt::launch_status();
         }
-    glue::k_split_sum<Tp, 1><<<grid, 256, 0, st>>>(A, B, n, splits);
+    dna::launch_pdl(glue::k_split_sum<Tp, 1>, grid, dim3(256), 0, st, A, B, n, splits);
     return simt::launch_status();
 }
 
@@ -407,8 +409,8 @@ int Simt<Tp>::select_fused(const View& v, const Tp* Xmu, const Tp* Xdna, const d
     const size_t smem = glue::select_smem<Tp>(v.R);
     auto k = glue::k_select_fused<Tp>;
     if (simt::prep_smem(k, smem)) return DNA_ERR_CUDA;
-    k<<<(unsigned)glue_parts(v.O), dim3(32, 8), smem, st>>>(v, Xmu, Xdna, dpart, splits, choice,
-                                                           dfin, fpart, reg, dcur, cur_splits);
+    dna::launch_pdl(k, dim3((unsigned)glue_parts(v.O)), dim3(32, 8), smem, st, v, Xmu, Xdna,
+                    dpart, splits, choice, dfin, fpart, reg, dcur, cur_splits);
     return simt::launch_status();
 }
 
@@ -418,7 +420,8 @@ int Simt<Tp>::mu_fused(const View& v, const double* c, const Tp* A, int splits, 
     const size_t smem = glue::select_smem<Tp>(v.R);
     auto k = glue::k_mu_fused<Tp>;
     if (simt::prep_smem(k, smem)) return DNA_ERR_CUDA;
-    k<<<(unsigned)glue_parts(v.O), dim3(32, 8), smem, st>>>(v, c, A, splits, fpart);
+    dna::launch_pdl(k, dim3((unsigned)glue_parts(v.O)), dim3(32, 8), smem, st, v, c, A, splits,
+                    fpart);
     return simt::launch_status();
 }
 
@@ -426,8 +429,8 @@ template <typename Tp>
 int Simt<Tp>::part_sums(const double* part, int64_t nparts, int64_t R, double reg, double* out,
                         cudaStream_t st, double* next) {
     if (R <= 1024)   // a CTA per r: latency of one load round and a tree, not of nparts / 32
-        simt::k_colsum_small<0><<<(unsigned)R, 256, 0, st>>>(part, (int)nparts, R, reg, out, true,
-                                                             next);
+        dna::launch_pdl(simt::k_colsum_small<0>, dim3((unsigned)R), dim3(256), 0, st, part,
+                        (int)nparts, R, reg, out, true, next);
     else
         simt::k_colsum_final<<<(unsigned)((R + 31) / 32), dim3(32, 32), 0, st>>>(
             part, (int)nparts, R, reg, out, true, next);
@@ -458,11 +461,11 @@ int Simt<Tp>::scale_ops(const View& t, const double* f, bool xmul, void* Xk, voi
     const int64_t blocks = a.xtiles + ytiles;
     if (blocks == 0) return DNA_OK;
     if (rt == 32)
-        glue::k_scale_ops<Tp, 32><<<(unsigned)blocks, dim3(32, 8), 0, st>>>(a);
+        dna::launch_pdl(glue::k_scale_ops<Tp, 32>, dim3((unsigned)blocks), dim3(32, 8), 0, st, a);
     else if (rt == 64)
-        glue::k_scale_ops<Tp, 64><<<(unsigned)blocks, dim3(32, 8), 0, st>>>(a);
+        dna::launch_pdl(glue::k_scale_ops<Tp, 64>, dim3((unsigned)blocks), dim3(32, 8), 0, st, a);
     else
-        glue::k_scale_ops<Tp, 128><<<(unsigned)blocks, dim3(32, 8), 0, st>>>(a);
+        dna::launch_pdl(glue::k_scale_ops<Tp, 128>, dim3((unsigned)blocks), dim3(32, 8), 0, st, a);
     return simt::launch_status();
 }
 
@@ -529,7 +532,8 @@ template <typename Tp>
 int Simt<Tp>::raw_sums(const double* part, int64_t nparts, int64_t R, double* out,
                        cudaStream_t st) {
     if (R <= 1024)
-        simt::k_colsum_small<0><<<(unsigned)R, 256, 0, st>>>(part, (int)nparts, R, 0.0, out, false);
+        dna::launch_pdl(simt::k_colsum_small<0>, dim3((unsigned)R), dim3(256), 0, st, part,
+                        (int)nparts, R, 0.0, out, false, nullptr);
     else
         simt::k_colsum_final<<<(unsigned)((R + 31) / 32), dim3(32, 32), 0, st>>>(
             part, (int)nparts, R, 0.0, out, false);
@@ -555,9 +559,9 @@ int Simt<Tp>::sp_pass1(int64_t R, const SparseSegs& sg, const int32_t* idx, cons
                        int* status, cudaStream_t st) {
     if (sg.n == 0) return DNA_OK;
     return simt::by_lanes(R, [&](auto lpn) {
-        sparse::k_sp_pass1<Tp, decltype(lpn)::value>
-            <<<simt::sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(R4, sg, idx, val, Yr, Xr, Aseg,
-                                                                 Bseg, with_b, status);
+        dna::launch_pdl(sparse::k_sp_pass1<Tp, decltype(lpn)::value>, dim3(simt::sp_grid(sg.n)),
+                        dim3(sparse::WARPS * 32), 0, st, R4, sg, idx, val, Yr, Xr, Aseg, Bseg,
+                        with_b, status);
         return simt::launch_status();
     });
 }
@@ -570,8 +574,8 @@ int Simt<Tp>::sp_cand(const View& v, const SparseSegs& sg, const Tp* Aseg, const
         constexpr int LPN = decltype(lpn)::value;
         const unsigned grid = simt::sp_grid((v.O + 32 / LPN - 1) / (32 / LPN));
         auto k = mu ? sparse::k_sp_cand<Tp, LPN, true> : sparse::k_sp_cand<Tp, LPN, false>;
-        k<<<grid, sparse::WARPS * 32, 0, st>>>(v.O, v.R, R4, sg.sptr, Aseg, Bseg, Xr, c, v.vsum,
-                                               Xm, Xd, (Tp)eps, (Tp)alpha);
+        dna::launch_pdl(k, grid, dim3(sparse::WARPS * 32), 0, st, v.O, v.R, R4, sg.sptr, Aseg,
+                        Bseg, Xr, c, v.vsum, Xm, Xd, (Tp)eps, (Tp)alpha);
         return simt::launch_status();
     });
 }
@@ -582,9 +586,8 @@ int Simt<Tp>::sp_pass2(int64_t R, const SparseSegs& sg, const int32_t* idx, cons
                        cudaStream_t st) {
     if (sg.n == 0) return DNA_OK;
     return simt::by_lanes(R, [&](auto lpn) {
-        sparse::k_sp_pass2<Tp, decltype(lpn)::value>
-            <<<simt::sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(R4, sg, idx, val, Yr, Xm, Xd,
-                                                                 dseg);
+        dna::launch_pdl(sparse::k_sp_pass2<Tp, decltype(lpn)::value>, dim3(simt::sp_grid(sg.n)),
+                        dim3(sparse::WARPS * 32), 0, st, R4, sg, idx, val, Yr, Xm, Xd, dseg);
         return simt::launch_status();
     });
 }
@@ -596,8 +599,8 @@ int Simt<Tp>::sp_select(const View& v, const SparseSegs& sg, const double* dseg,
     return simt::by_lanes(v.R, [&](auto lpn) {
         constexpr int LPN = decltype(lpn)::value;
         auto k = mu ? sparse::k_sp_select<Tp, LPN, true> : sparse::k_sp_select<Tp, LPN, false>;
-        k<<<(unsigned)glue_parts(v.O), sparse::WARPS * 32, 0, st>>>(
-            v, R4, sg.sptr, dseg, Xm, Xd, c0, choice, dfin, fpart, reg, status);
+        dna::launch_pdl(k, dim3((unsigned)glue_parts(v.O)), dim3(sparse::WARPS * 32), 0, st, v,
+                        R4, sg.sptr, dseg, Xm, Xd, c0, choice, dfin, fpart, reg, status);
         return simt::launch_status();
     });
 }
@@ -623,7 +626,8 @@ int Simt<Tp>::sp_kl(const View& v, const SparseSegs& sg, const int32_t* idx, con
 template <typename Tp>
 int Simt<Tp>::pad_rows(const Tp* in, int64_t n, int64_t R, int64_t ld, Tp* out, cudaStream_t st) {
     const int64_t blocks = std::min<int64_t>((n * ld + 255) / 256, 152 * 16);
-    sparse::k_pad_rows<Tp><<<(unsigned)blocks, 256, 0, st>>>(in, n, R, ld, out);
+    dna::launch_pdl(sparse::k_pad_rows<Tp>, dim3((unsigned)blocks), dim3(256), 0, st, in, n, R,
+                    ld, out);
     return simt::launch_status();
 }
 
@@ -631,7 +635,7 @@ template <typename Tp>
 int Simt<Tp>::transpose(const Tp* in, int64_t rows, int64_t cols, int64_t ld, Tp* out,
                         cudaStream_t st) {
     const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((ld + 31) / 32));
-    sparse::k_transpose<Tp><<<grid, dim3(32, 8), 0, st>>>(in, rows, cols, ld, out);
+    dna::launch_pdl(sparse::k_transpose<Tp>, grid, dim3(32, 8), 0, st, in, rows, cols, ld, out);
     return simt::launch_status();
 }
 

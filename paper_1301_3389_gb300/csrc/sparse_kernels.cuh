@@ -246,6 +246,7 @@ __global__ void __launch_bounds__(WARPS * 32)
     k_sp_pass1(int64_t R4, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
                const Tp* __restrict__ Yr, const Tp* __restrict__ Xr, Tp* __restrict__ Aseg,
                Tp* __restrict__ Bseg, bool with_b, int* __restrict__ status) {
+    pdl_wait();
     constexpr int STEP = LPN / U;   // lanes that hold the same finished z
     const int lane = threadIdx.x & 31, sub = lane % LPN, lead = lane - sub, r = 4 * sub;
     const int64_t g = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
@@ -307,6 +308,8 @@ __global__ void __launch_bounds__(WARPS * 32)
               const Tp* __restrict__ Xr, const double* __restrict__ c,
               const double* __restrict__ vsum, Tp* __restrict__ Xm, Tp* __restrict__ Xd, Tp eps,
               Tp alpha) {
+    pdl_wait();
+    pdl_next();
     __shared__ Tp cs[4 * LPN], ics[4 * LPN];
     for (int k = threadIdx.x; k < 4 * LPN; k += WARPS * 32) {
         cs[k] = k < R ? (Tp)c[k] : Tp(1);
@@ -376,6 +379,7 @@ __global__ void __launch_bounds__(WARPS * 32)
     k_sp_pass2(int64_t R4, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
                const Tp* __restrict__ Yr, const Tp* __restrict__ Xm, const Tp* __restrict__ Xd,
                double* __restrict__ dseg) {
+    pdl_wait();
     const int lane = threadIdx.x & 31, sub = lane % LPN, r = 4 * sub;
     const int64_t g = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
     if (g >= sg.n) return;
@@ -436,6 +440,8 @@ __global__ void __launch_bounds__(WARPS * 32)
                 const Tp* __restrict__ Xd, const double* __restrict__ c0,
                 uint8_t* __restrict__ choice, double* __restrict__ dfin,
                 double* __restrict__ fpart, double reg, int* __restrict__ status) {
+    pdl_wait();
+    pdl_next();
     constexpr int G = 32 / LPN, NK = 4 / G;   // columns of a warp at once, rounds
     __shared__ Tp xs[4 * LPN][33];
     __shared__ Tp ch[4 * LPN], cl[4 * LPN];   // c0 = ch + cl
@@ -597,6 +603,8 @@ __global__ void __launch_bounds__(WARPS * 32)
 template <typename Tp>
 __global__ void __launch_bounds__(256) k_pad_rows(const Tp* __restrict__ in, int64_t n, int64_t R,
                                                   int64_t ld, Tp* __restrict__ out) {
+    pdl_wait();
+    pdl_next();
     for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < n * ld;
          e += (int64_t)gridDim.x * 256) {
         const int64_t i = e / ld, r = e % ld;
@@ -611,6 +619,8 @@ template <typename Tp>
 __global__ void __launch_bounds__(256) k_transpose(const Tp* __restrict__ in, int64_t rows,
                                                    int64_t cols, int64_t ld,
                                                    Tp* __restrict__ out) {
+    pdl_wait();
+    pdl_next();
     __shared__ Tp tile[32][33];
     const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 32;
     for (int i = threadIdx.y; i < 32; i += 8) {

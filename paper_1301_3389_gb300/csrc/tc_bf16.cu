@@ -108,6 +108,7 @@ __device__ __forceinline__ void pass1_body(const P1Args& a, int64_t bx, int64_t 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
 
     if (warp == W_PRODUCER) {
         // One thread services the three rings in whatever order their slots free up.
@@ -834,7 +835,7 @@ int launch_pass1(const P1Args& a, const TcMaps& m, int64_t O_pad, int splits, cu
         cudaSuccess)
         return DNA_ERR_CUDA;
     dim3 grid((unsigned)(O_pad / OBLK), (unsigned)splits);
-    k<<<grid, P1_THREADS, smem, st>>>(a, m.y, m.yt, m.y2t, m.v);
+    dna::launch_pdl(k, grid, dim3(P1_THREADS), smem, st, a, m.y, m.yt, m.y2t, m.v);
     return after_launch();
 }
 

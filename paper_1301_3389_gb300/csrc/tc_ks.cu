@@ -133,6 +133,8 @@ __global__ void __launch_bounds__(ks::P2K_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
+    if ((int)gridDim.x == ntiles) pdl_next();   // a tile each: SMs may be idle
 
     if (warp == W_PRODUCER) {
         if (lane == 0 && t_begin < t_end) {
@@ -313,11 +315,11 @@ int launch_pass2_kt(const P2Args& a, const TcMaps& m, int64_t O_pad, int splits,
     if (ntiles == 0) return DNA_OK;
     const int grid = ctas > 0 ? std::min(ctas, ntiles) : ntiles;
     if (SPLIT)
-        k<<<grid, ks::P2K_THREADS, smem, st>>>(a, nob, splits, ntiles, m.xm, m.xd, m.y, m.xm_l,
-                                               m.xd_l, m.y_l);
+        dna::launch_pdl(k, grid, dim3(ks::P2K_THREADS), smem, st, a, nob, splits, ntiles, m.xm,
+                        m.xd, m.y, m.xm_l, m.xd_l, m.y_l);
     else   // the lo maps are not read
-        k<<<grid, ks::P2K_THREADS, smem, st>>>(a, nob, splits, ntiles, m.xm, m.xd, m.y, m.xm,
-                                               m.xd, m.y);
+        dna::launch_pdl(k, grid, dim3(ks::P2K_THREADS), smem, st, a, nob, splits, ntiles, m.xm,
+                        m.xd, m.y, m.xm, m.xd, m.y);
     return after_launch();
 }
 
@@ -392,6 +394,8 @@ __global__ void __launch_bounds__(ks::P2K_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
+    if ((int)gridDim.x == nunits) pdl_next();   // a tile each: SMs may be idle
 
     if (warp == W_PRODUCER) {
         if (lane == 0 && nloc > 0) {
@@ -576,7 +580,8 @@ int launch_pass2_yr(const P2Args& a, const TcMaps& m, int64_t O_pad, int ctas, c
     if (nunits == 0) return DNA_OK;
     if (nunits > INT32_MAX) return DNA_ERR_ARG;
     const int grid = (int)std::min<int64_t>(ctas > 0 ? ctas : nunits, nunits);
-    k_tc_pass2_yr<<<grid, ks::P2K_THREADS, smem, st>>>(a, nob, (int)nunits, m.xm, m.xd, m.y);
+    dna::launch_pdl(k_tc_pass2_yr, grid, dim3(ks::P2K_THREADS), smem, st, a, nob, (int)nunits,
+                    m.xm, m.xd, m.y);
     return after_launch();
 }
 

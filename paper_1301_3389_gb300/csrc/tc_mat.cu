@@ -190,6 +190,8 @@ __global__ void __launch_bounds__(mat::A_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
+    if ((int)gridDim.x == ntiles) pdl_next();   // a tile each: SMs may be idle
 
     if (warp == W_PROD_A) {
         // One thread services three queues in whatever order they allow progress: Y
@@ -455,6 +457,8 @@ __global__ void __launch_bounds__(mat::B_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
+    if ((int)gridDim.x == ntiles) pdl_next();   // a tile each: SMs may be idle
 
     if (warp == W_PROD_B) {
         if (lane == 0 && t_first < ntiles) {
@@ -586,7 +590,8 @@ int launch_mat(const TcOperands& op, const TcMaps& m, float* Apart, float* Bpart
             return DNA_ERR_CUDA;
         const int ntiles = nob * splits_a;
         const int grid = op.ctas > 0 ? std::min(op.ctas, ntiles) : ntiles;
-        k<<<grid, A_THREADS, smem, st>>>(ra, splits_a, ntiles, m.y128, m.v, m.q, m.qb);
+        dna::launch_pdl(k, grid, dim3(A_THREADS), smem, st, ra, splits_a, ntiles, m.y128, m.v,
+                        m.q, m.qb);
         if (int e = after_launch()) return e;
     }
     ContractArgs ca{};
@@ -600,8 +605,8 @@ int launch_mat(const TcOperands& op, const TcMaps& m, float* Apart, float* Bpart
     const int nop = (nob + 1) / 2, nrb = RP / RB;
     const int ntiles = (WITH_B ? 2 : 1) * nrb * nop * splits;
     const int grid = op.ctas > 0 ? std::min(op.ctas, ntiles) : ntiles;
-    k<<<grid, B_THREADS, smem, st>>>(ca, nob, nop, nrb, splits, ntiles, status, m.q, m.qb,
-                                     m.yt256, m.y2t256);
+    dna::launch_pdl(k, grid, dim3(B_THREADS), smem, st, ca, nob, nop, nrb, splits, ntiles, status,
+                    m.q, m.qb, m.yt256, m.y2t256);
     return after_launch();
 }
 

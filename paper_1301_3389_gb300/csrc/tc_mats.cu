@@ -201,6 +201,8 @@ __global__ void __launch_bounds__(mats::A_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
+    if ((int)gridDim.x == ntiles) pdl_next();   // a tile each: SMs may be idle
 
     if (warp == W_PROD_A) {
         // K-slices of every chunk in the MMA thread's order: Y hi, Y lo [128 s][64 r] and
@@ -469,6 +471,8 @@ __global__ void __launch_bounds__(mats::B_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
+    if ((int)gridDim.x == ntiles) pdl_next();   // a tile each: SMs may be idle
 
     if (warp == W_PROD_B) {
         if (lane == 0 && t_first < ntiles) {
@@ -629,8 +633,8 @@ int launch_mats(const TcOperands& op, const TcMaps& m, float* Apart, float* Bpar
             return DNA_ERR_CUDA;
         const int ntiles = nob * splits_a;
         const int grid = op.ctas > 0 ? std::min(op.ctas, ntiles) : ntiles;
-        k<<<grid, A_THREADS, smem, st>>>(ra, splits_a, ntiles, m.y128, m.y128_l, m.x_l, m.q,
-                                         m.q_l, m.qb, m.qb_l);
+        dna::launch_pdl(k, grid, dim3(A_THREADS), smem, st, ra, splits_a, ntiles, m.y128,
+                        m.y128_l, m.x_l, m.q, m.q_l, m.qb, m.qb_l);
         if (int e = after_launch()) return e;
     }
     ContractArgs ca{};
@@ -644,8 +648,8 @@ int launch_mats(const TcOperands& op, const TcMaps& m, float* Apart, float* Bpar
     const int nrb = RP / RB;
     const int ntiles = (WITH_B ? 2 : 1) * nrb * nob * splits;
     const int grid = op.ctas > 0 ? std::min(op.ctas, ntiles) : ntiles;
-    k<<<grid, B_THREADS, smem, st>>>(ca, nob, nrb, splits, ntiles, status, m.q, m.q_l, m.qb,
-                                     m.qb_l, m.yt256, m.yt256_l, m.y2t256, m.y2t256_l);
+    dna::launch_pdl(k, grid, dim3(B_THREADS), smem, st, ca, nob, nrb, splits, ntiles, status, m.q,
+                    m.q_l, m.qb, m.qb_l, m.yt256, m.yt256_l, m.y2t256, m.y2t256_l);
     return after_launch();
 }
 

@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(P1_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
 
     if (warp == W_PRODUCER) {
         // one thread services the three rings in whatever order their slots free up; each
@@ -589,6 +590,7 @@ __device__ __forceinline__ void pass2s_body(const P2Args& a, int64_t nch, int64_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();   // the set-up above overlaps the previous kernel's end
 
     if (warp == W_PRODUCER) {
         if (lane == 0 && u0 < u1) {
@@ -827,8 +829,8 @@ int launch_pass1s(const P1Args& a, bool with_b, const TcMaps& m, int64_t O_pad, 
     const int ntiles = nwhich * nob * splits;
     if (ntiles == 0) return DNA_OK;
     const int grid = ctas > 0 ? std::min(ctas, ntiles) : ntiles;
-    k<<<grid, P1_THREADS, smem, st>>>(a, nwhich, nob, ntiles, m.x, m.x_l, m.y, m.y_l, m.yt,
-                                       m.yt_l, m.y2t, m.y2t_l, m.v);
+    dna::launch_pdl(k, grid, dim3(P1_THREADS), smem, st, a, nwhich, nob, ntiles, m.x, m.x_l, m.y,
+                    m.y_l, m.yt, m.yt_l, m.y2t, m.y2t_l, m.v);
     return after_launch();
 }
 
@@ -877,7 +879,8 @@ int launch_pass2s(const P2Args& a, const TcMaps& m, int64_t O_pad, int slots, in
     const CUtensorMap& xd = FULL ? m.x : m.xd;
     const CUtensorMap& xdl = FULL ? m.x_l : NP == 2 ? m.xd_l : m.xd;
     const CUtensorMap& yl = NP == 2 ? m.y_l : m.y;
-    k<<<grid, P1_THREADS, smem, st>>>(a, nch, U, slots, xm, xml, xd, xdl, m.y, yl, m.v);
+    dna::launch_pdl(k, grid, dim3(P1_THREADS), smem, st, a, nch, U, slots, xm, xml, xd, xdl, m.y,
+                    yl, m.v);
     return after_launch();
 }
 
