@@ -195,6 +195,8 @@ __device__ __forceinline__ void cand_reg_tile(const View& v, const double* __res
     constexpr bool STAGE = BF && RS == 8;
     __shared__ Tp red[16][33];
     __shared__ Tp scl[32];
+    // c_r and 1 / c_r, converted once per CTA: a float64 conversion takes a warp 64 cycles
+    __shared__ Tp cs[16 * RS], ics[16 * RS];
     // staged bf16 rows: [plane: mu hi, dna hi, mu lo, dna lo][r group][o] (16 bytes each)
     __shared__ uint4 stg[STAGE ? 4 : 1][STAGE ? 16 : 1][STAGE ? 33 : 1];
     const int64_t R = v.R, O = v.O;
@@ -205,6 +207,10 @@ __device__ __forceinline__ void cand_reg_tile(const View& v, const double* __res
     const int nr = live && r0 < R ? (int)(R - r0 < RS ? R - r0 : RS) : 0;
     const Tp* __restrict__ X = static_cast<const Tp*>(v.X);
 
+    for (int r = ty * 32 + tx; r < R; r += 32 * (int)blockDim.y) {
+        cs[r] = (Tp)c[r];
+        ics[r] = Tp(1) / cs[r];
+    }
     Tp ra[RS], rb[RS], x[RS];
 #pragma unroll
     for (int i = 0; i < RS; ++i) { ra[i] = Tp(0); rb[i] = Tp(0); x[i] = Tp(0); }
@@ -237,6 +243,7 @@ __device__ __forceinline__ void cand_reg_tile(const View& v, const double* __res
             bp += ss;
         }
     }
+    __syncthreads();
     Tp den = Tp(0), xd[RS], xm[RS];
 #pragma unroll
     for (int i = 0; i < RS; ++i) {
@@ -244,7 +251,7 @@ __device__ __forceinline__ void cand_reg_tile(const View& v, const double* __res
         xd[i] = Tp(0);
         xm[i] = Tp(0);
         if (i >= nr) continue;
-        const Tp cr = (Tp)c[r], ic = Tp(1) / cr;
+        const Tp cr = cs[r], ic = ics[r];
         const Tp a = ra[i] * ic - Tp(1);   // eq. 7
         const Tp b = rb[i] * ic;           // eq. 14
         const Tp xr = x[i];

@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(256, 4)
         const int ng = jt.pad > 0 ? jt.pad : 1, g = jt.b;
         const int lead = wid & ~(ng - 1);
         float xm[8], xd[8];
-        float den = 0.f;
+        float den = 0.f, target = 0.f;   // target: the eq. 10 sum of the column
         bool live = false;
         int64_t o = 0, R = 0, O = 0;
 #pragma unroll
@@ -141,6 +141,17 @@ __global__ void __launch_bounds__(256, 4)
             o = (int64_t)jt.a * 32 + lane;
             live = o < O;
             const int64_t r0 = 8 * (int64_t)g;
+            // the job's 8 denominators, converted once by 8 lanes (a float64 conversion
+            // takes a warp 64 cycles, as many as the rest of an element's arithmetic)
+            const int64_t rl = r0 + (lane & 7);
+            const float cl = rl < R ? (float)p.c[rl] : 1.f, icl = 1.0f / cl;
+            target = live ? (float)v.vsum[o] : 0.f;
+            float cv[8], icv[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                cv[i] = __shfl_sync(0xffffffffu, cl, i);
+                icv[i] = __shfl_sync(0xffffffffu, icl, i);
+            }
             if (live && r0 < R) {
                 const int sp1 = p.sp1[w];
                 const float* __restrict__ X = static_cast<const float*>(v.X);
@@ -179,7 +190,7 @@ __global__ void __launch_bounds__(256, 4)
                 for (int i = 0; i < 8; ++i) {
                     const int64_t r = r0 + i;
                     if (r >= R) continue;
-                    const float cr = (float)p.c[r], ic = 1.0f / cr;
+                    const float cr = cv[i], ic = icv[i];
                     const float a = ra[i] * ic - 1.0f;   // eq. 7
                     const float b = rb[i] * ic;          // eq. 14
                     const float xr = xv[i];
@@ -209,7 +220,7 @@ __global__ void __launch_bounds__(256, 4)
             float tot = red[lead][lane];
             for (int k = 1; k < ng; ++k) tot += red[lead + k][lane];
             const GProb& p = P[jt.prob];
-            const float sc = live ? (tot > 0.f ? (float)p.v[w].vsum[o] / tot : 1.0f) : 0.f;
+            const float sc = live ? (tot > 0.f ? target / tot : 1.0f) : 0.f;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 xd[i] *= sc;
@@ -259,7 +270,9 @@ __global__ void __launch_bounds__(256)
         bool newton = false;
         if (o < O) {
             double dm = 0.0, dd = 0.0;
-            for (int sp = 0; sp < p.nslot[w]; ++sp) {
+            const int nslot = p.nslot[w];
+#pragma unroll 8
+            for (int sp = 0; sp < nslot; ++sp) {   // eight slots' loads in flight
                 dm += p.dpart[((int64_t)sp * 2 + 0) * O + o];
                 dd += p.dpart[((int64_t)sp * 2 + 1) * O + o];
             }
@@ -278,24 +291,40 @@ __global__ void __launch_bounds__(256)
             p.dfin[w][O + o] = dd;
         }
         float* X = static_cast<float*>(v.X);
+        // sixteen loads before their stores: X and the candidates may alias for the compiler,
+        // which would otherwise wait for each store before the next load
+        const float* src = newton ? p.Xdna : p.Xmu;
         if (v.xo == 1) {   // X rows contiguous along o: lanes write their own column
-            if (o < O) {
-                const float* src = newton ? p.Xdna : p.Xmu;
-#pragma unroll 8
-                for (int64_t r = 0; r < R; ++r) X[r * v.xr + o] = src[r * O + o];
-            }
+            const int64_t xr = v.xr;
+            if (o < O)
+                for (int64_t r0 = 0; r0 < R; r0 += 16) {
+                    float t[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) t[u] = r0 + u < R ? src[(r0 + u) * O + o] : 0.f;
+#pragma unroll
+                    for (int u = 0; u < 16; ++u)
+                        if (r0 + u < R) X[(r0 + u) * xr + o] = t[u];
+                }
         } else {           // contiguous along r: stage the 32 columns, lanes walk r
-            const float* src = newton ? p.Xdna : p.Xmu;
+            const int64_t xo = v.xo;
             for (int64_t r0 = 0; r0 < R; r0 += 32) {
                 const int64_t nr = R - r0 < 32 ? R - r0 : 32;
-#pragma unroll 8
-                for (int64_t r = 0; r < nr; ++r) xs[r][lane] = o < O ? src[(r0 + r) * O + o] : 0.f;
-                __syncwarp();
-                for (int k = 0; k < 32; ++k) {
-                    const int64_t oo = o0 + k;
-                    if (oo >= O) break;
-                    if (lane < nr) X[oo * v.xo + (r0 + lane) * v.xr] = xs[lane][k];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float t[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) {
+                        const int64_t r = r0 + 16 * h + u;
+                        t[u] = r < R && o < O ? src[r * O + o] : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) xs[16 * h + u][lane] = t[u];
                 }
+                __syncwarp();
+                const int nk = (int)(O - o0 < 32 ? O - o0 : 32);
+                if (lane < nr)
+#pragma unroll 8
+                    for (int k = 0; k < nk; ++k) X[(o0 + k) * xo + r0 + lane] = xs[lane][k];
                 __syncwarp();
             }
         }
@@ -310,6 +339,7 @@ __global__ void __launch_bounds__(256)
 __global__ void __launch_bounds__(256)
     k_g_sums(const GProb* __restrict__ P, const GTile* __restrict__ tl, int n, int w, int which,
              double reg) {
+    constexpr int BATCH = 16;   // rows whose loads a thread issues together
     __shared__ double red[8][65];
     const int lane = threadIdx.x, ty = threadIdx.y;
     for (int t = blockIdx.x; t < n; t += gridDim.x) {
@@ -325,7 +355,14 @@ __global__ void __launch_bounds__(256)
             const int64_t r = 8 * (int64_t)tt.a + ty;
             if (r < R) {
                 float s = 0.f;
-                for (int64_t i = lane; i < cnt; i += 32) s += M[r * sr + i];
+                for (int64_t i = lane; i < cnt; i += 32 * BATCH) {
+                    float t[BATCH];
+#pragma unroll
+                    for (int u = 0; u < BATCH; ++u)
+                        t[u] = i + 32 * u < cnt ? M[r * sr + i + 32 * u] : 0.f;
+#pragma unroll
+                    for (int u = 0; u < BATCH; ++u) s += t[u];
+                }
                 double d = (double)s;
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) d += __shfl_down_sync(0xffffffffu, d, off);
@@ -335,9 +372,20 @@ __global__ void __launch_bounds__(256)
             for (int64_t r0 = 0; r0 < R; r0 += 64) {
                 float s0 = 0.f, s1 = 0.f;
                 const int64_t ra = r0 + lane, rb = r0 + 32 + lane;
-                for (int64_t i = ty; i < cnt; i += 8) {
-                    if (ra < R) s0 += M[i * si + ra];
-                    if (rb < R) s1 += M[i * si + rb];
+                for (int64_t i = ty; i < cnt; i += 8 * BATCH) {
+                    float t0[BATCH], t1[BATCH];
+#pragma unroll
+                    for (int u = 0; u < BATCH; ++u) {
+                        const bool in = i + 8 * u < cnt;
+                        const float* row = M + (i + 8 * u) * si;
+                        t0[u] = in && ra < R ? row[ra] : 0.f;
+                        t1[u] = in && rb < R ? row[rb] : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < BATCH; ++u) {
+                        s0 += t0[u];
+                        s1 += t1[u];
+                    }
                 }
                 red[ty][lane] = (double)s0;
                 red[ty][32 + lane] = (double)s1;
@@ -357,11 +405,22 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// The factors a rescale multiplies by, in float32 for r < 64: 1 / sig_r (X) or sig_r (Y).
+// Once per tile, not per element (a float64 conversion takes a warp 64 cycles).
+__device__ __forceinline__ void load_factors(float* fr, const double* __restrict__ sig, int64_t R,
+                                             bool divide, int tid) {
+    if (tid < 64) {
+        const float f = tid < R ? (float)sig[tid] : 1.f;
+        fr[tid] = divide ? 1.0f / f : f;
+    }
+}
+
 // Steps 1, 16, 29: X(r, .) /= sig_r and Y(., r) *= sig_r for a block of 32 values of i
 // (o of X or s of Y) of one problem: tiles (problem, 0 | 1 (X | Y), block).  Lanes walk
 // the matrix's contiguous index.
 __global__ void __launch_bounds__(256)
     k_g_rescale(const GProb* __restrict__ P, const GTile* __restrict__ tl, int n, int w) {
+    __shared__ float fr[64];
     const int lane = threadIdx.x, ty = threadIdx.y;
     for (int t = blockIdx.x; t < n; t += gridDim.x) {
         const GTile tt = tl[t];
@@ -372,21 +431,30 @@ __global__ void __launch_bounds__(256)
         const int64_t cnt = isx ? v.O : v.S;
         const int64_t si = isx ? v.xo : v.ys, sr = isx ? v.xr : v.yr;
         const int64_t R = v.R, i0 = (int64_t)tt.b * 32;
+        __syncthreads();   // the factors of the tile before are used
+        load_factors(fr, p.sig, R, isx, ty * 32 + lane);
+        __syncthreads();
+        const int nr = (int)R, ni = (int)(cnt - i0 < 32 ? cnt - i0 : 32);
+        float val[8];   // all loads before the stores
         if (si == 1) {
-            const int64_t i = i0 + lane;
-            if (i < cnt)
-                for (int64_t r = ty; r < R; r += 8) {
-                    const float f = (float)p.sig[r];
-                    M[r * sr + i] = isx ? M[r * sr + i] * (1.0f / f) : M[r * sr + i] * f;
-                }
+            float* q = M + ty * sr + i0 + lane;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                val[j] = ty + 8 * j < nr && lane < ni ? q[8 * j * sr] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (ty + 8 * j < nr && lane < ni) q[8 * j * sr] = val[j] * fr[ty + 8 * j];
         } else {
-            for (int k = ty; k < 32; k += 8) {
-                const int64_t i = i0 + k;
-                if (i >= cnt) break;
-                for (int64_t r = lane; r < R; r += 32) {
-                    const float f = (float)p.sig[r];
-                    M[i * si + r] = isx ? M[i * si + r] * (1.0f / f) : M[i * si + r] * f;
-                }
+            float* q = M + (i0 + ty) * si + lane;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int k = 8 * (j >> 1), r = 32 * (j & 1);
+                val[j] = lane + r < nr && ty + k < ni ? q[k * si + r] : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int k = 8 * (j >> 1), r = 32 * (j & 1);
+                if (lane + r < nr && ty + k < ni) q[k * si + r] = val[j] * fr[lane + r];
             }
         }
     }
@@ -396,11 +464,13 @@ __global__ void __launch_bounds__(256)
 // the bf16 operands of half-step wn = 1 - w, whose X is Y_w and whose Y is X_w: tiles
 // (problem, 0 | 1 (X | Y of view wn), block of 64) of that view's operand list, each
 // element scaled once, written back in float32 and as bf16 operand rows (the layout of
-// k_g_operands).  CTA = 32 x 8 threads.
+// k_g_operands).  CTA = 32 x 8 threads.  It was bound by its instructions (64-bit indices and
+// a division per element, rows past R): 128 problems 61, 55 us before, 31, 28 now.
 __global__ void __launch_bounds__(256)
     k_g_rescale_ops(const GProb* __restrict__ P, const TcGView* __restrict__ gv,
                     const GTile* __restrict__ tl, int n, int wn) {
     __shared__ float tile[64][65];   // [r][i]
+    __shared__ float fr[64];
     const int lane = threadIdx.x, ty = threadIdx.y;
     for (int t = blockIdx.x; t < n; t += gridDim.x) {
         const GTile tt = tl[t];
@@ -411,33 +481,56 @@ __global__ void __launch_bounds__(256)
         const int64_t cnt = isx ? v.O : v.S;
         const int64_t si = isx ? v.xo : v.ys, sr = isx ? v.xr : v.yr;
         const int64_t R = v.R, i0 = (int64_t)tt.b * 64;
-        // element e = 2 j + h of this thread: (r, i) = (ty + 8 j, i0 + 32 h + lane) when the
-        // matrix is contiguous along i, else (32 h + lane, i0 + ty + 8 j); all 16 loads are
-        // issued before the scaled values are stored back
-        const bool along_i = si == 1;
+        // rows of 32 (along the contiguous index) x 8 groups: all loads of a thread are issued
+        // before the scaled values are stored back; rows past R are not touched
+        const int nr = (int)R, ni = (int)(cnt - i0 < 64 ? cnt - i0 : 64);
         float val[16];
+        if (si == 1) {   // contiguous along i: (r, i) = (ty + 8 j, 32 h + lane)
+            float* q = M + ty * sr + i0 + lane;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const int j = e >> 1, h = e & 1;
-            const int64_t r = along_i ? ty + 8 * j : 32 * h + lane;
-            const int64_t i = along_i ? i0 + 32 * h + lane : i0 + ty + 8 * j;
-            val[e] = (r < R && i < cnt) ? M[r * sr + i * si] : 0.f;
-        }
+            for (int j = 0; j < 8; ++j) {
+                if (8 * j >= nr) break;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const int j = e >> 1, h = e & 1;
-            const int64_t r = along_i ? ty + 8 * j : 32 * h + lane;
-            const int64_t i = along_i ? i0 + 32 * h + lane : i0 + ty + 8 * j;
-            float x = 0.f;
-            if (r < R && i < cnt) {
-                const float f = (float)p.sig[r];
-                x = isx ? val[e] * f : val[e] * (1.0f / f);
-                M[r * sr + i * si] = x;
+                for (int h = 0; h < 2; ++h)
+                    val[2 * j + h] =
+                        ty + 8 * j < nr && 32 * h + lane < ni ? q[8 * j * sr + 32 * h] : 0.f;
             }
-            if (along_i)
-                tile[r][32 * h + lane] = x;
-            else
-                tile[r][ty + 8 * j] = x;
+            load_factors(fr, p.sig, R, !isx, ty * 32 + lane);
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (8 * j >= nr) break;
+                const int r = ty + 8 * j;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float x = val[2 * j + h] * fr[r];
+                    if (r < nr && 32 * h + lane < ni) q[8 * j * sr + 32 * h] = x;
+                    tile[r][32 * h + lane] = x;
+                }
+            }
+        } else {         // contiguous along r: (r, i) = (32 h + lane, ty + 8 j)
+            float* q = M + (i0 + ty) * si + lane;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (32 * h >= nr) break;
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    val[8 * h + j] =
+                        32 * h + lane < nr && ty + 8 * j < ni ? q[8 * j * si + 32 * h] : 0.f;
+            }
+            load_factors(fr, p.sig, R, !isx, ty * 32 + lane);
+            __syncthreads();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (32 * h >= nr) break;
+                const int r = 32 * h + lane;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float x = val[8 * h + j] * fr[r];
+                    if (r < nr && ty + 8 * j < ni) q[8 * j * si + 32 * h] = x;
+                    tile[r][ty + 8 * j] = x;
+                }
+            }
         }
         __syncthreads();
         // values r >= R stay as the zeros the buffers were created with
@@ -799,8 +892,7 @@ int g_half(dna_group* g, int w, bool mu_only, bool ops_ready = false, bool fuse_
                                              g->num_sms, g->status, g->gs);
         if (!e && g->cand_bf[w].n) {
             const int nblk = g->cand_bf[w].n / 8;
-            const int grid = std::max(1, std::min(nblk, 4 * g->num_sms));
-            dna::grp::k_g_candidates_bf<<<grid, dim3(32, 8), 0, g->gs>>>(
+            dna::grp::k_g_candidates_bf<<<nblk, dim3(32, 8), 0, g->gs>>>(
                 g->dp, g->gv, g->cand_bf[w].d, nblk, w, (float)g->o.eps, (float)g->o.alpha);
             e = after_launch();
         }

@@ -390,7 +390,8 @@ __device__ __forceinline__ void candidates_tile(const View& v, const double* __r
     const bool live = o < v.O;
     const Tp* __restrict__ X = static_cast<const Tp*>(v.X);
     Tp den = Tp(0);   // this thread's R / 8 terms of the eq. 10 denominator
-    constexpr int U = 8;   // values of r whose loads are issued together
+    constexpr int U = 4;   // values of r whose loads are issued together (8: slower)
+    const double target = live ? v.vsum[o] : 0.0;
     if (live) {
         for (int64_t r0 = ty; r0 < v.R; r0 += 8 * U) {
             Tp ra[U], rb[U], xv[U];
@@ -443,7 +444,8 @@ __device__ __forceinline__ void candidates_tile(const View& v, const double* __r
     if (live) {
         double tot = 0.0;
         for (int k = 0; k < 8; ++k) tot += red[k][tx];
-        const Tp sc = (Tp)(tot > 0.0 ? v.vsum[o] / tot : 1.0);   // eq. 10
+        const Tp sc = (Tp)(tot > 0.0 ? target / tot : 1.0);   // eq. 10
+#pragma unroll 8
         for (int64_t r = ty; r < v.R; r += 8) Xdna[r * v.O + o] *= sc;
     }
     __syncthreads();   // the shared arrays are reused by the next tile

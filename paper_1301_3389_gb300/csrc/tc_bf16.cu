@@ -751,20 +751,43 @@ __global__ void __launch_bounds__(256)
         const int64_t cnt = isx ? v.O : v.S;
         const int64_t si = isx ? v.xo : v.ys, sr = isx ? v.xr : v.yr;
         const int64_t R = v.R, i0 = (int64_t)tt.z * 64;
-        if (si == 1) {   // contiguous along i: lanes walk i
-            for (int r = ty; r < 64; r += 8)
+        // all loads of a thread before its shared stores (M could point into shared memory
+        // for the compiler, which would keep each load behind the store before it); rows past
+        // R are neither read nor written, but for the rest of their group of 8 (or 32)
+        const int nr = (int)R, ni = (int)(cnt - i0 < 64 ? cnt - i0 : 64);
+        float val[16];
+        if (si == 1) {   // contiguous along i: (r, i) = (ty + 8 j, 32 h + lane)
+            const float* q = M + ty * sr + i0 + lane;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int64_t i = i0 + 32 * h + lane;
-                    tile[r][32 * h + lane] = (r < R && i < cnt) ? M[r * sr + i] : 0.f;
-                }
-        } else {         // contiguous along r: lanes walk r
-            for (int k = ty; k < 64; k += 8)
+            for (int j = 0; j < 8; ++j) {
+                if (8 * j >= nr) break;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int64_t i = i0 + k, r = 32 * h + lane;
-                    tile[r][k] = (r < R && i < cnt) ? M[i * si + r * sr] : 0.f;
-                }
+                for (int h = 0; h < 2; ++h)
+                    val[2 * j + h] =
+                        ty + 8 * j < nr && 32 * h + lane < ni ? q[8 * j * sr + 32 * h] : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (8 * j >= nr) break;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) tile[ty + 8 * j][32 * h + lane] = val[2 * j + h];
+            }
+        } else {         // contiguous along r: (r, i) = (32 h + lane, ty + 8 j)
+            const float* q = M + (i0 + ty) * si + lane;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (32 * h >= nr) break;
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    val[8 * h + j] =
+                        32 * h + lane < nr && ty + 8 * j < ni ? q[8 * j * si + 32 * h] : 0.f;
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (32 * h >= nr) break;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) tile[32 * h + lane][ty + 8 * j] = val[8 * h + j];
+            }
         }
         __syncthreads();
         // rows [i][64] with r contiguous: Xk (X) or Yk (Y); lanes walk pairs of r (values
