@@ -787,7 +787,9 @@ int step_core(dna_ctx* c, int w, bool mu_only, bool prepared, int stop) {
         // the tensor-core forms keep the ascending order of splits, since bf16 operands make
         // a selection near a tie depend on the last bit
         const int parts = stop == STOP_PASS2 ? 1 : sp1;
-        const bool presum = parts > 4 || ((int64_t)parts * v.O >= 32768 && parts > 1);
+        const bool wide = sizeof(Tp) == 4 && !S::cand_in_registers(c->R);   // loads them all
+        const bool presum =
+            parts > 4 || ((int64_t)parts * v.O >= 32768 && parts > 1 && !wide);
         e = phase(c, DNA_PHASE_CANDIDATES, presum ? 2 : 1, [&] {
             if (presum)
                 if (int r = S::split_sum(A, B, c->R, v.O, parts, st, tc)) return r;

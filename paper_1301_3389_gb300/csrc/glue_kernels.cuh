@@ -37,22 +37,20 @@ __device__ __forceinline__ void split1(float x, bf16& h, bf16& l) {
     l = __float2bfloat16_rn(x - __bfloat162float(h));
 }
 
-// Dynamic shared memory of k_cand_fused: red [TY][TO]; cs, ics [R]; sc; xs, ms [R][TO + 1].
+// Dynamic shared memory of k_cand_fused: red [TY][TO]; cs, ics [R]; sc; xs [R][TO + 1].
 template <typename Tp>
-constexpr size_t cand_smem(int64_t R, bool bf) {
-    return sizeof(Tp) * (2 * (size_t)R + (bf ? 2 : 1) * (size_t)R * (TO + 1) + TO + TY * TO);
+constexpr size_t cand_smem(int64_t R) {
+    return sizeof(Tp) * (2 * (size_t)R + (size_t)R * (TO + 1) + TO + TY * TO);
 }
 
-// CTA = 32 columns o (threadIdx.x) x 32 groups of r (threadIdx.y); grid covers O (or O_pad
-// when bf16 copies are written: the padding rows are written as zeros).
-template <typename Tp, bool BF>
+// The candidates in float64 above rank 128: CTA = 32 columns o (threadIdx.x) x 32 groups of r
+// (threadIdx.y).
+template <typename Tp>
 __global__ void __launch_bounds__(1024) k_cand_fused(View v, const double* __restrict__ c,
                                                     const Tp* __restrict__ Apart,
                                                     const Tp* __restrict__ Bpart, int splits,
                                                     Tp* __restrict__ Xmu, Tp* __restrict__ Xdna,
-                                                    Tp eps, Tp alpha, bf16* __restrict__ Xmk,
-                                                    bf16* __restrict__ Xdk, int64_t rp,
-                                                    int64_t plane) {
+                                                    Tp eps, Tp alpha) {
     pdl_wait();
     pdl_next();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -62,7 +60,6 @@ __global__ void __launch_bounds__(1024) k_cand_fused(View v, const double* __res
     Tp* ics = cs + R;                                             // [R]
     Tp* scl = ics + R;                                            // [TO]
     Tp* xs = scl + TO;                                            // [R][TO + 1]: x, then x_dna
-    Tp* ms = xs + R * (TO + 1);                                   // [R][TO + 1]: x_mu (BF)
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
     const int64_t o0 = (int64_t)blockIdx.x * TO, o = o0 + tx;
     const bool live = o < O;
@@ -124,7 +121,6 @@ __global__ void __launch_bounds__(1024) k_cand_fused(View v, const double* __res
             if (!live) xd = Tp(0);
             if (live) Xmu[r * O + o] = xmu;
             xs[r * (TO + 1) + tx] = xd;
-            if constexpr (BF) ms[r * (TO + 1) + tx] = live ? xmu : Tp(0);
             den += cs[r] * xd;
         }
     }
@@ -146,32 +142,6 @@ __global__ void __launch_bounds__(1024) k_cand_fused(View v, const double* __res
     for (int64_t r = ty; r < R; r += TY) {
         const Tp xd = xs[r * (TO + 1) + tx] * sc;
         if (live) Xdna[r * O + o] = xd;
-        if constexpr (BF) xs[r * (TO + 1) + tx] = xd;
-    }
-    if constexpr (BF) {
-        __syncthreads();
-        // K-major bf16 rows [o][rp]: lanes walk pairs of r
-        {
-            const int i = ty;
-            const int64_t oi = o0 + i;
-            for (int64_t r = 2 * tx; r < rp; r += 64) {
-                float m0 = 0.f, m1 = 0.f, d0 = 0.f, d1 = 0.f;
-                if (r < R) { m0 = (float)ms[r * (TO + 1) + i]; d0 = (float)xs[r * (TO + 1) + i]; }
-                if (r + 1 < R) {
-                    m1 = (float)ms[(r + 1) * (TO + 1) + i];
-                    d1 = (float)xs[(r + 1) * (TO + 1) + i];
-                }
-                const uint32_t mh = pack2(m0, m1), dh = pack2(d0, d1);
-                *reinterpret_cast<uint32_t*>(Xmk + oi * rp + r) = mh;
-                *reinterpret_cast<uint32_t*>(Xdk + oi * rp + r) = dh;
-                if (plane) {   // lo planes: x - bf16(x)
-                    *reinterpret_cast<uint32_t*>(Xmk + plane + oi * rp + r) =
-                        pack2(m0 - lo_half(mh), m1 - hi_half(mh));
-                    *reinterpret_cast<uint32_t*>(Xdk + plane + oi * rp + r) =
-                        pack2(d0 - lo_half(dh), d1 - hi_half(dh));
-                }
-            }
-        }
     }
 }
 
@@ -347,6 +317,153 @@ __global__ void __launch_bounds__(512) k_cand_reg(View v, const double* __restri
     pdl_next();
     cand_reg_tile<Tp, BF, RS>(v, c, Apart, Bpart, splits, Xmu, Xdna, eps, alpha, Xmk, Xdk, rp,
                               plane, blockIdx.x);
+}
+
+// The candidates for 256 < R <= 512 in float32.  CTA = 16 columns x 32 groups of r (512
+// threads, two CTAs per SM, so that one's loads overlap the other's arithmetic and stores);
+// group g holds r = g + 32 u, u < 16, eight values at a time: their X and every split's A and
+// B are loaded together, the MU candidates are stored at once, the Newton candidates wait in
+// registers for the eq. 10 scale (each group's terms in ascending r, then a fixed butterfly
+// over the 32 groups).  With BF the grid covers O_pad and the bf16 rows [o][rp] (hi, and with
+// `plane` lo planes) are staged in shared memory (row length rp + 2: no bank conflicts) and
+// stored 128 bytes per warp instruction, zeros in the padding.  Bound by memory: N=8192
+// T=32768 R=512 H half-step, BF16: 162 us, and 56 us for the sum of two splits before it, with
+// 1024 threads around [R][32] tiles in shared memory -> 134 us with
+// that sum included (515 MB; the W half-step, one split, 41 -> 34 us).
+constexpr int CW_COLS = 16;
+constexpr size_t cand_wide_smem(int64_t rp, bool bf, bool lo) {
+    return sizeof(float) * 1024 + (bf ? sizeof(bf16) * (lo ? 4 : 2) * CW_COLS * (size_t)(rp + 2) : 0);
+}
+template <bool BF>
+__global__ void __launch_bounds__(512, 2)
+    k_cand_wide(View v, const double* __restrict__ c, const float* __restrict__ Apart,
+                const float* __restrict__ Bpart, int splits, float* __restrict__ Xmu,
+                float* __restrict__ Xdna, float eps, float alpha, bf16* __restrict__ Xmk,
+                bf16* __restrict__ Xdk, int64_t rp, int64_t plane) {
+    pdl_wait();
+    pdl_next();
+    constexpr int G = 32, U = 8;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* cs = reinterpret_cast<float*>(smem_raw);   // [512] c_r
+    float* ics = cs + 512;                            // [512] 1 / c_r
+    bf16* stg = reinterpret_cast<bf16*>(ics + 512);   // [plane: mu, dna, mu lo, dna lo][16][rp + 2]
+    __shared__ float red[G][CW_COLS + 1];
+    __shared__ float scl[CW_COLS];
+    const int tid = threadIdx.x, tx = tid % CW_COLS, g = tid / CW_COLS;
+    const int R = (int)v.R, ldo = (int)rp + 2;
+    const int64_t O = v.O, o0 = (int64_t)blockIdx.x * CW_COLS, o = o0 + tx;
+    const bool live = o < O;
+    const int64_t ss = v.R * O;
+    for (int r = tid; r < R; r += 512) {
+        cs[r] = (float)c[r];
+        ics[r] = 1.0f / cs[r];
+    }
+    const float* __restrict__ Xp = static_cast<const float*>(v.X) + o * v.xo;
+    bf16* srow = stg + tx * ldo;
+    const int pl = CW_COLS * ldo;   // elements of one staged plane
+    float xd[2 * U], den = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r0 = g + G * U * h;   // r = r0 + 32 u
+        float x[U], ra[U], rb[U];
+        {
+            const float* xp = Xp + r0 * v.xr;
+            const float* ap = Apart + r0 * O + o;
+            const float* bp = Bpart + r0 * O + o;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool in = live && r0 + G * u < R;
+                x[u] = in ? xp[G * u * v.xr] : 0.f;
+                ra[u] = in ? ap[G * u * O] : 0.f;
+                rb[u] = in ? bp[G * u * O] : 0.f;
+            }
+            for (int sp = 1; sp < splits; ++sp) {
+                ap += ss;
+                bp += ss;
+                float a1[U], b1[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool in = live && r0 + G * u < R;
+                    a1[u] = in ? ap[G * u * O] : 0.f;
+                    b1[u] = in ? bp[G * u * O] : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) { ra[u] += a1[u]; rb[u] += b1[u]; }
+            }
+        }
+        if (h == 0) __syncthreads();   // cs, ics
+        float* mp = Xmu + r0 * O + o;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int r = r0 + G * u;
+            float xm = 0.f, d = 0.f;
+            if (r < R) {
+                const float ic = ics[r];
+                const float a = ra[u] * ic - 1.0f;   // eq. 7
+                const float b = rb[u] * ic;          // eq. 14
+                xm = x[u] * (ra[u] * ic);            // eq. 11 (no cancellation)
+                if (a < 0.f) {                       // eq. 15, gain floored at eps
+                    const float xb = x[u] * b;
+                    const float gn = simt::dev_div(xb, xb - a);
+                    d = x[u] * (gn > eps ? gn : eps);
+                } else {                             // eq. 17, step capped at alpha x
+                    const float stp = b > 0.f ? simt::dev_div(a, b) : 0.f;
+                    const float cap = alpha * x[u];
+                    d = x[u] + (stp < cap ? stp : cap);
+                }
+                if (!live) { xm = 0.f; d = 0.f; }
+                if (live) mp[G * u * O] = xm;
+                den += cs[r] * d;
+            }
+            xd[U * h + u] = d;
+            if (BF && r < rp) {
+                const bf16 hi = __float2bfloat16_rn(xm);
+                srow[r] = hi;
+                if (plane) srow[2 * pl + r] = __float2bfloat16_rn(xm - __bfloat162float(hi));
+            }
+        }
+    }
+    red[g][tx] = den;
+    __syncthreads();
+    if (tid < 32 * CW_COLS) {   // warp w: column w's 32 group sums
+        const int col = tid >> 5, lane = tid & 31;
+        float tot = red[lane][col];
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, m);
+        const int64_t oc = o0 + col;
+        if (lane == 0)
+            scl[col] = oc < O ? (tot > 0.f ? (float)v.vsum[oc] / tot : 1.0f) : 0.f;   // eq. 10
+    }
+    __syncthreads();
+    const float sc = scl[tx];
+    float* dp = Xdna + g * O + o;
+#pragma unroll
+    for (int u = 0; u < 2 * U; ++u) {
+        const int r = g + G * u;
+        const float d = xd[u] * sc;
+        if (live && r < R) dp[G * u * O] = d;
+        if (BF && r < rp) {
+            const bf16 hi = __float2bfloat16_rn(d);
+            srow[pl + r] = hi;
+            if (plane) srow[3 * pl + r] = __float2bfloat16_rn(d - __bfloat162float(hi));
+        }
+    }
+    if constexpr (BF) {
+        __syncthreads();
+        // 16 rows of rp values per plane, 4-byte words: a warp stores 128 bytes of a row
+        const int wpr = (int)rp / 2, nw = CW_COLS * wpr;
+        for (int k = tid; k < nw; k += 512) {
+            const int row = k / wpr, w = k % wpr;
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(stg + row * ldo) + w;
+            const int64_t at = (o0 + row) * rp + 2 * w;
+            *reinterpret_cast<uint32_t*>(Xmk + at) = src[0];
+            *reinterpret_cast<uint32_t*>(Xdk + at) = src[pl / 2];
+            if (plane) {
+                *reinterpret_cast<uint32_t*>(Xmk + plane + at) = src[pl];
+                *reinterpret_cast<uint32_t*>(Xdk + plane + at) = src[pl / 2 * 3];
+            }
+        }
+    }
 }
 
 // A[0][i] = A[0][i] + A[1][i] + ... + A[splits-1][i] (ascending, the order the candidates

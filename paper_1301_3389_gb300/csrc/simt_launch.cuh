@@ -350,20 +350,20 @@ int Simt<Tp>::cand_fused(const View& v, const double* c, const Tp* A, const Tp* 
         }
         return simt::launch_status();
     }
-    const size_t smem = glue::cand_smem<Tp>(v.R, bf);
-    if (bf) {
-        if constexpr (sizeof(Tp) == 4) {
-            auto k = glue::k_cand_fused<Tp, true>;
-            if (simt::prep_smem(k, smem)) return DNA_ERR_CUDA;
-            dna::launch_pdl(k, grid, dim3(32, glue::TY), smem, st, v, c, A, B, splits, Xmu, Xdna,
-                            (Tp)eps, (Tp)alpha, static_cast<glue::bf16*>(Xmk),
-                            static_cast<glue::bf16*>(Xdk), rp, plane);
-        }
+    if constexpr (sizeof(Tp) == 4) {   // float32 above the registers' ranks: R <= 512
+        const unsigned cols = (unsigned)(((bf ? O_pad : v.O) + glue::CW_COLS - 1) / glue::CW_COLS);
+        const size_t smem = glue::cand_wide_smem(rp, bf, plane != 0);
+        auto k = bf ? glue::k_cand_wide<true> : glue::k_cand_wide<false>;
+        if (v.R > 512 || (bf && rp > 512) || simt::prep_smem(k, smem)) return DNA_ERR_CUDA;
+        dna::launch_pdl(k, cols, dim3(512), smem, st, v, c, A, B, splits, Xmu, Xdna, (Tp)eps,
+                        (Tp)alpha, static_cast<glue::bf16*>(Xmk), static_cast<glue::bf16*>(Xdk),
+                        rp, plane);
     } else {
-        auto k = glue::k_cand_fused<Tp, false>;
+        const size_t smem = glue::cand_smem<Tp>(v.R);
+        auto k = glue::k_cand_fused<Tp>;
         if (simt::prep_smem(k, smem)) return DNA_ERR_CUDA;
         dna::launch_pdl(k, grid, dim3(32, glue::TY), smem, st, v, c, A, B, splits, Xmu, Xdna,
-                        (Tp)eps, (Tp)alpha, nullptr, nullptr, 0, 0);
+                        (Tp)eps, (Tp)alpha);
     }
     return simt::launch_status();
 }
