@@ -18,10 +18,12 @@ template <typename Tp> constexpr int rblock_for(int64_t R) {
 
 inline int launch_status() { return after_launch(); }
 
+// Opts a kernel in to its dynamic shared memory.  The limit without opting in is 48 KB of
+// static and dynamic memory together, and the kernels here have up to 12 KB of static arrays.
 template <typename Kern>
 inline int prep_smem(Kern k, size_t bytes) {
     static_assert(sizeof(Kern) > 0, "");
-    if (bytes > 48 * 1024) {
+    if (bytes > 32 * 1024) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
             cudaSuccess)
             return DNA_ERR_CUDA;
