@@ -211,6 +211,29 @@ void plan_split(int64_t S, int64_t nblocks_os, int slots, int chunk, int* splits
     *splits = (int)((S + *per - 1) / *per);
 }
 
+// Splits of pass 2 of the split FP32 form at R > 128 (k_tc_pass2_kt).  Its tiles load their
+// candidates with every chunk, so a shorter split costs only its four cost slots per column
+// (64 bytes, written once and read once by the selection): the time of the chunks on the
+// busiest SM (about 1.2 us per chunk and 64 ranks) plus the slots' at 6 TB/s.  N=2100 T=2600
+// R=300: 6 and 7 splits of 3 chunks on 126 and 119 SMs instead of 4 and 5 of 5 on 84 and 85,
+// 52 -> 26 us with the five K-slices of rank_slices.
+void plan_pass2_kt(int64_t S, int64_t nob, int sms, int chunk, int64_t R, int* splits,
+                   int64_t* per) {
+    const int64_t chunks = (S + chunk - 1) / chunk;
+    const double chunk_us = 1.2 * (double)((R + 63) / 64);
+    const double slot_us = (double)(nob * 128) * 64.0 * 2.0 / 6.0e6;
+    int64_t best = chunks;
+    double best_us = 1e300;
+    for (int64_t pc = chunks; pc >= 1; --pc) {
+        const int64_t sp = (chunks + pc - 1) / pc;
+        if (sp > 32) break;
+        const double us = (double)((nob * sp + sms - 1) / sms * pc) * chunk_us + (double)sp * slot_us;
+        if (us < best_us) { best_us = us; best = pc; }
+    }
+    *per = best * chunk;
+    *splits = (int)((S + *per - 1) / *per);
+}
+
 // Splits of a float32 pass on the CUDA cores (f32_pass.cuh: chunks and o-blocks of 64), by
 // the time they should take in microseconds: an SM works its share of the CTAs off at
 // chunk_us per chunk whether one or two of them are resident, but a lone CTA hides its own
@@ -308,15 +331,12 @@ void plan_all(dna_ctx* c) {
             // the split FP32 kernel
             const int64_t rblocks = (c->split ? 2 : 1) * (c->rp > 128 ? c->rp / 256 : 1);
             // the split form, and pass 1 at ranks above 128, stream s in chunks of 128
-            const int sch = c->split ? (int)SPLIT_CHUNK : tch;
             const int sch1 = c->split || c->rp > 128 ? (int)SPLIT_CHUNK : tch;
             // the split form's pass 1 at R <= 128 accumulates a whole split in tensor
             // memory, so its splits are at most SPLIT_MAX_CHUNKS chunks; at R > 128 the
             // contraction kernel cuts each split into such segments itself
             plan_split(Sdim, c->pad_o[w] / tob * rblocks, c->num_sms, sch1, &c->tsp1[w],
                        &c->tper1[w], part, c->split && c->rp <= 128 ? SPLIT_MAX_CHUNKS : 0);
-            plan_split(Sdim, c->pad_o[w] / tob, c->num_sms, c->rp > 256 ? (int)SPLIT_CHUNK : sch,
-                       &c->tsp2[w], &c->tper2[w], 2.0 / (double)Sdim);
             // pass 2 of the split form at R <= 128 and of the BF16 form at R <= 256 balances
             // (o-block, chunk) units over the SMs instead; otherwise each split has four
             // cost slots (one per column group of the epilogue warps)
@@ -325,8 +345,11 @@ void plan_all(dna_ctx* c) {
             else if (!c->split && c->rp == 512) {   // Y-resident pass 2: a slot per s-block
                 c->tsp2[w] = (int)((Sdim + SPLIT_CHUNK - 1) / SPLIT_CHUNK);
                 c->tper2[w] = SPLIT_CHUNK;
-            } else
+            } else {
+                plan_pass2_kt(Sdim, c->pad_o[w] / tob, c->num_sms, (int)SPLIT_CHUNK, c->R,
+                              &c->tsp2[w], &c->tper2[w]);
                 c->tsp2[w] *= 4;
+            }
         }
     }
 }

@@ -886,14 +886,16 @@ int TcBf16::make_maps(TcMaps* m, const TcOperands& op, const float* V, int64_t v
         e = make_map(&m->v, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, V, (uint64_t)op.O, (uint64_t)op.S,
                      (uint64_t)vs * 4, OBLK, SCH, CU_TENSOR_MAP_SWIZZLE_NONE);
     if (!e && op.Qg) {      // the Q, Qbar workspace of pass 1 at RP > 128, and larger boxes
+        const uint32_t rbw = (uint32_t)rank_block_rows(op.R);   // rows of one r-block
         e = make_map(&m->q, BF, op.Qg, (uint64_t)op.ldq, op.O_pad, (uint64_t)op.ldq * 2, 64, OBLK, SW);
         if (!e) e = make_map(&m->qb, BF, op.Qbg, (uint64_t)op.ldq, op.O_pad, (uint64_t)op.ldq * 2, 64,
                              OBLK, SW);
         if (!e) e = make_map(&m->y128, BF, op.Yk, rp, op.S_pad, rp * 2, 64, 128, SW);
-        if (!e) e = make_map(&m->yt256, BF, op.Ytk, op.S_pad, rp, op.S_pad * 2, SCH, 256, SW);
-        if (!e) e = make_map(&m->y2t256, BF, op.Y2tk, op.S_pad, rp, op.S_pad * 2, SCH, 256, SW);
+        if (!e) e = make_map(&m->yt256, BF, op.Ytk, op.S_pad, rp, op.S_pad * 2, SCH, rbw, SW);
+        if (!e) e = make_map(&m->y2t256, BF, op.Y2tk, op.S_pad, rp, op.S_pad * 2, SCH, rbw, SW);
     }
     if (!e && op.Qg && op.plane) {   // lo planes of pass 1 of the split form at RP > 128
+        const uint32_t rbw = (uint32_t)rank_block_rows(op.R);
         const bf16* ql = static_cast<const bf16*>(op.Qg) + op.qplane;
         const bf16* qbl = static_cast<const bf16*>(op.Qbg) + op.qplane;
         e = make_map(&m->q_l, BF, ql, (uint64_t)op.ldq, op.O_pad, (uint64_t)op.ldq * 2, 64, OBLK, SW);
@@ -902,9 +904,9 @@ int TcBf16::make_maps(TcMaps* m, const TcOperands& op, const float* V, int64_t v
         if (!e) e = make_map(&m->y128_l, BF, static_cast<const bf16*>(op.Yk) + op.plane, rp, op.S_pad,
                              rp * 2, 64, 128, SW);
         if (!e) e = make_map(&m->yt256_l, BF, static_cast<const bf16*>(op.Ytk) + op.plane, op.S_pad,
-                             rp, op.S_pad * 2, SCH, 256, SW);
+                             rp, op.S_pad * 2, SCH, rbw, SW);
         if (!e) e = make_map(&m->y2t256_l, BF, static_cast<const bf16*>(op.Y2tk) + op.plane,
-                             op.S_pad, rp, op.S_pad * 2, SCH, 256, SW);
+                             op.S_pad, rp, op.S_pad * 2, SCH, rbw, SW);
     }
     if (!e && op.plane) {   // lo planes of the split FP32 form
         const bf16* yl = static_cast<const bf16*>(op.Yk) + op.plane;

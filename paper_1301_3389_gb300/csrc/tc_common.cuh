@@ -92,6 +92,18 @@ __device__ __forceinline__ void split2(float v0, float v1, uint32_t& hi, uint32_
     lo = pack_bf16x2(v0 - h0, v1 - h1);
 }
 
+// Padded ranks 256 and 512 hold zeros above R.  The kernels of RP > 128 take only the 64-wide
+// K-slices of r that hold a factor value, and the contractions cut r into ceil(R / 256) equal
+// blocks of a multiple of 16 instead of blocks of 256: the skipped products are exact zeros
+// added to each sum, so the results keep their bits.  N=2100 T=2600 R=300 (RP = 512: 5 of 8
+// slices, two blocks of 160 instead of 256), FP32 form: ratios 41 -> 32 us, contraction 45 -> 38 (H), 34 -> 27 (W), pass 2 (with its
+// splits, plan_pass2_kt) 52 -> 26.
+__host__ __device__ constexpr int rank_slices(int64_t R) { return (int)((R + 63) / 64); }
+__host__ __device__ constexpr int rank_blocks(int64_t R) { return (int)((R + 255) / 256); }
+__host__ __device__ constexpr int rank_block_rows(int64_t R) {
+    return (int)((R + 16 * rank_blocks(R) - 1) / (16 * rank_blocks(R)) * 16);
+}
+
 // X rows [o][rp] (bf16, global) -> tensor memory, 16-column unit `unit` (32 values of r)
 // of the lane quadrant addressed by taddr.
 __device__ __forceinline__ void x_to_tmem(const bf16* __restrict__ X, int64_t rp, int64_t o,

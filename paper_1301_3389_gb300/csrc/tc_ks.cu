@@ -102,7 +102,8 @@ __global__ void __launch_bounds__(ks::P2K_THREADS, 1)
                   const __grid_constant__ CUtensorMap tmXdl, const __grid_constant__ CUtensorMap tmYl) {
     using L = ks::Layout2<SPLIT>;
     using namespace ks;
-    constexpr int KST = L::KST, KS = RP / 64;
+    constexpr int KST = L::KST;
+    const int KS = rank_slices(a.R);   // K-slices of r in use
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -360,7 +361,8 @@ __global__ void __launch_bounds__(ks::P2K_THREADS, 1)
                   const __grid_constant__ CUtensorMap tmXd, const __grid_constant__ CUtensorMap tmY) {
     using L = ks::LayoutY;
     using namespace ks;
-    constexpr int KST = L::KST, KS = L::KS;
+    constexpr int KST = L::KST;
+    const int KS = rank_slices(a.R);   // K-slices of r in use (at most L::KS)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));

@@ -70,6 +70,7 @@ struct RatioArgs {
     int64_t vs;
     const bf16* X;             // [O_pad][rp]
     int64_t rp;
+    int k64;                   // 64-wide K-slices of r in use
     bf16* Q;                   // [O_pad][ldq]
     bf16* Qb;
     int64_t ldq;
@@ -92,7 +93,7 @@ __device__ __forceinline__ ATile a_tile(int t, int nsplit, const RatioArgs& a) {
 constexpr int B_EPI = 8;                     // epilogue warps of the contract kernel
 constexpr int W_PROD_B = B_EPI, W_MMA_B = B_EPI + 1;
 constexpr int B_THREADS = (B_EPI + 2) * 32;
-constexpr int RB = 256;                      // r per tile of the contract kernel
+constexpr int RB = 256;                      // most r per tile of the contract kernel
 
 // A tile covers two o-blocks (M = 256 as two 128-row MMAs that share each Yt slice), one
 // 256-wide r-block, one split of s and one accumulator kind (A, or B): shared-memory
@@ -101,7 +102,7 @@ constexpr int RB = 256;                      // r per tile of the contract kerne
 struct LayoutB {
     static constexpr int KST = 3;
     static constexpr uint32_t Q_TILE = OBLK * 64 * 2;    // [128 o][64 s]
-    static constexpr uint32_t Y_TILE = RB * 64 * 2;      // [256 r][64 s]
+    static constexpr uint32_t Y_TILE = RB * 64 * 2;      // [rbw r][64 s]
     // Q (or Qbar) of the two o-blocks, then Yt (or Y2t)
     static constexpr uint32_t STAGE = 2 * Q_TILE + Y_TILE;
     static constexpr uint32_t BAR = KST * STAGE;
@@ -114,6 +115,7 @@ enum { C_KFULL = 0, C_KEMPTY = 3, C_ACCFULL = 6, C_ACCEMPTY = 7, C_DRAIN = 8, C_
 
 struct ContractArgs {
     int64_t S, O, R, s_per;    // s_per: a multiple of 64
+    int rbw;                   // r per tile (rank_block_rows)
     float* Apart;              // [splits][R][O]
     float* Bpart;
 };
@@ -147,14 +149,18 @@ __device__ __forceinline__ BTile b_tile(int t, int nop, int nrb, int nsplit,
 }  // namespace mat
 
 // ---------------------------------------------------------------- ratios kernel
-template <int RP, bool WITH_B>
+// FULL: every slice of the padded rank is in use (the counts are constants then: with the
+// count from an argument N=8192 T=32768 R=512 takes 489 us instead of 470)
+template <int RP, bool WITH_B, bool FULL>
 __global__ void __launch_bounds__(mat::A_THREADS, 1)
     k_tc_ratios(mat::RatioArgs a, int nsplit, int ntiles, const __grid_constant__ CUtensorMap tmY,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmQ,
                 const __grid_constant__ CUtensorMap tmQb) {
     using namespace mat;
     using L = LayoutA<RP>;
-    constexpr int KST = L::KST, VST = L::VST, KS = RP / 128;
+    constexpr int KST = L::KST, VST = L::VST;
+    // slices of 128, the last one half empty if K64 is odd
+    const int K64 = FULL ? RP / 64 : a.k64, KS = (K64 + 1) / 2;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -216,10 +222,12 @@ __global__ void __launch_bounds__(mat::A_THREADS, 1)
                     const uint32_t dst = sbase + st * L::Y_SLICE;
                     const int32_t r0 = 128 * sy;
                     const int32_t s0 = (int32_t)(xy.s_begin + (int64_t)ky * SC);
-                    mbar_arrive_expect_tx(&bar[A_KFULL + st], L::Y_SLICE);
+                    const int nsub = FULL ? 2 : min(2, K64 - 2 * sy);
+                    mbar_arrive_expect_tx(&bar[A_KFULL + st], nsub * L::Y_SUB);
 #pragma unroll
                     for (int hs = 0; hs < 2; ++hs)     // sub-tile hs: r0 + 64 hs .. + 63, 128 s
-                        tma_load_2d(dst + hs * L::Y_SUB, &tmY, r0 + 64 * hs, s0, &bar[A_KFULL + st]);
+                        if (hs < nsub)
+                            tma_load_2d(dst + hs * L::Y_SUB, &tmY, r0 + 64 * hs, s0, &bar[A_KFULL + st]);
                     ++kk;
                     if (++sy == KS) {
                         sy = 0;
@@ -304,10 +312,16 @@ __global__ void __launch_bounds__(mat::A_THREADS, 1)
                         tc_fence_after();
                         const uint32_t ys = sbase + (j % KST) * L::Y_SLICE;
 #pragma unroll
-                        for (int kq = 0; kq < 8; ++kq)
+                        for (int kq = 0; kq < 4; ++kq)
                             mma_bf16_tmem_a(tz, tmem + L::TX + (uint32_t)(8 * ks + kq) * 8u,
-                                            desc_sw128(ys + (kq >> 2) * L::Y_SUB + 32u * (kq & 3)),
-                                            idesc, (ks > 0 || kq > 0) ? 1u : 0u);
+                                            desc_sw128(ys + 32u * kq), idesc,
+                                            (ks > 0 || kq > 0) ? 1u : 0u);
+                        if (FULL || 2 * ks + 1 < K64)
+#pragma unroll
+                            for (int kq = 4; kq < 8; ++kq)
+                                mma_bf16_tmem_a(tz, tmem + L::TX + (uint32_t)(8 * ks + kq) * 8u,
+                                                desc_sw128(ys + L::Y_SUB + 32u * (kq - 4)), idesc,
+                                                1u);
                         mma_commit(&bar[A_KEMPTY + j % KST]);
                     }
                     if (ok) mma_commit(&bar[A_ZFULL + b]);
@@ -340,7 +354,7 @@ __global__ void __launch_bounds__(mat::A_THREADS, 1)
             if (t == t_begin || a_tile(t - 1, nsplit, a).o0 != x.o0) {
                 // a new o-block: its X rows into tensor memory (every GEMM1 of the previous
                 // tile has completed: its last Z was read below)
-                for (int unit = cg; unit < RP / 32; unit += 4)
+                for (int unit = cg; unit < 2 * K64; unit += 4)
                     x_to_tmem(a.X, a.rp, o, unit, tmem + L::TX + lane_off);
                 tmem_st_wait();
                 tc_fence_before();
@@ -478,12 +492,12 @@ __global__ void __launch_bounds__(mat::B_THREADS, 1)
                         break;
                     const uint32_t dst = sbase + st * L::STAGE;
                     const int32_t s0 = (int32_t)(x.s_begin + 64 * (int64_t)sl);
-                    const int32_t r0 = RB * x.rb, o0 = (int32_t)x.o0;
+                    const int32_t r0 = a.rbw * x.rb, o0 = (int32_t)x.o0;
                     uint64_t* fb = &bar[C_KFULL + st];
-                    mbar_arrive_expect_tx(fb, L::STAGE - (two ? 0u : L::Q_TILE));
+                    mbar_arrive_expect_tx(fb, (two ? 2u : 1u) * L::Q_TILE + (uint32_t)a.rbw * 128u);
                     tma_load_2d(dst, mq, s0, o0, fb);                              // [128 o][64 s]
                     if (two) tma_load_2d(dst + L::Q_TILE, mq, s0, o0 + OBLK, fb);
-                    tma_load_2d(dst + 2 * L::Q_TILE, my, s0, r0, fb);              // [256 r][64 s]
+                    tma_load_2d(dst + 2 * L::Q_TILE, my, s0, r0, fb);              // [rbw r][64 s]
                 }
             }
             if (*abort)
@@ -494,7 +508,7 @@ __global__ void __launch_bounds__(mat::B_THREADS, 1)
         if (lane == 0) {
             bool ok = true;
             int j = 0, tt = 0;
-            constexpr uint32_t idesc = idesc_bf16(OBLK, RB);
+            const uint32_t idesc = idesc_bf16(OBLK, (uint32_t)a.rbw);
             for (int t = t_first; ok && t < ntiles; t += t_step, ++tt) {
                 const BTile x = b_tile(t, nop, nrb, nsplit, a);
                 const int nsl = x.nsl;
@@ -540,16 +554,23 @@ __global__ void __launch_bounds__(mat::B_THREADS, 1)
                 float* dst = x.which ? a.Bpart : a.Apart;
                 const int64_t base = (int64_t)x.split * a.R;
 #pragma unroll 1
-                for (int c = 0; c < RB / 32; ++c) {
+                for (int c = 0; 32 * c < a.rbw; ++c) {
                     uint32_t r32[32];
                     tmem_ld32(tmem + (uint32_t)(RB * h + 32 * c) + lane_off, r32);
                     tmem_ld_wait();
-                    if (o < a.O)
+                    if (o < a.O) {
+                        const int r0 = a.rbw * x.rb + 32 * c;
+                        const int nr = min((int)a.R - r0, a.rbw - 32 * c);   // rows to store
+                        float* col = dst + (base + r0) * a.O + o;
+                        if (nr >= 32) {
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            const int64_t r = (int64_t)RB * x.rb + 32 * c + i;
-                            if (r < a.R) dst[(base + r) * a.O + o] = __uint_as_float(r32[i]);
+                            for (int i = 0; i < 32; ++i) col[i * a.O] = __uint_as_float(r32[i]);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i)
+                                if (i < nr) col[i * a.O] = __uint_as_float(r32[i]);
                         }
+                    }
                 }
             }
             tc_fence_before();
@@ -579,12 +600,12 @@ int launch_mat(const TcOperands& op, const TcMaps& m, float* Apart, float* Bpart
     ra.s_per = (chunks + nsa - 1) / nsa * SC;
     const int splits_a = (int)((op.S + ra.s_per - 1) / ra.s_per);
     ra.V = op.V; ra.vs = op.vs;
-    ra.X = static_cast<const bf16*>(op.Xk); ra.rp = RP;
+    ra.X = static_cast<const bf16*>(op.Xk); ra.rp = RP; ra.k64 = rank_slices(op.R);
     ra.Q = static_cast<bf16*>(op.Qg); ra.Qb = static_cast<bf16*>(op.Qbg); ra.ldq = op.ldq;
     ra.status = status;
     {
         const uint32_t smem = LayoutA<RP>::TOTAL + 1024;
-        auto k = k_tc_ratios<RP, WITH_B>;
+        auto k = 64 * ra.k64 == RP ? k_tc_ratios<RP, WITH_B, true> : k_tc_ratios<RP, WITH_B, false>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess)
             return DNA_ERR_CUDA;
@@ -596,13 +617,14 @@ int launch_mat(const TcOperands& op, const TcMaps& m, float* Apart, float* Bpart
     }
     ContractArgs ca{};
     ca.S = op.S; ca.O = op.O; ca.R = op.R; ca.s_per = s_per;
+    ca.rbw = rank_block_rows(op.R);
     ca.Apart = Apart; ca.Bpart = Bpart;
     const uint32_t smem = LayoutB::TOTAL + 1024;
     auto k = k_tc_contract<WITH_B>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return DNA_ERR_CUDA;
-    const int nop = (nob + 1) / 2, nrb = RP / RB;
+    const int nop = (nob + 1) / 2, nrb = rank_blocks(op.R);
     const int ntiles = (WITH_B ? 2 : 1) * nrb * nop * splits;
     const int grid = op.ctas > 0 ? std::min(op.ctas, ntiles) : ntiles;
     dna::launch_pdl(k, grid, dim3(B_THREADS), smem, st, ca, nob, nop, nrb, splits, ntiles, status,

@@ -12,8 +12,8 @@
 //             hi and lo bf16 planes (Q[o][s], Qbar[o][s]) to a workspace through a ring of
 //             three staging buffers stored by TMA;
 //   contract  A[o, r] += sum_s Q[o, s] Yt[r, s] (CTAs of which = 0) and
-//             B[o, r] += sum_s Qbar[o, s] Y2t[r, s] (which = 1) over (o-block, 256-wide
-//             r-block, split of s) tiles, the three products per K-step into one 128 x 256
+//             B[o, r] += sum_s Qbar[o, s] Y2t[r, s] (which = 1) over (o-block, r-block of
+//             up to 256, split of s) tiles, the three products per K-step into one 128 x 256
 //             accumulator, written per split ([split][R][O]).  The tensor pipe's float32
 //             accumulation is not round-to-nearest, so one accumulation covers at most 1024
 //             values of s: a longer split runs as segments of 1024 into alternating
@@ -74,6 +74,7 @@ struct RatioArgs {
     int64_t vs;
     const bf16* X;            // hi plane [O_pad][rp]
     int64_t rp;
+    int ks;                   // 64-wide K-slices of r in use
     int* status;
 };
 
@@ -106,7 +107,7 @@ __device__ __forceinline__ void put_row16(uint32_t tile, int row, int cg, const 
 constexpr int B_EPI = 8;                      // epilogue warps of the contract kernel
 constexpr int W_PROD_B = B_EPI, W_MMA_B = B_EPI + 1;
 constexpr int B_THREADS = (B_EPI + 2) * 32;
-constexpr int RB = 256;                       // r per tile of the contract kernel
+constexpr int RB = 256;                       // most r per tile of the contract kernel
 // K-slices of 64 values of s that one accumulation in tensor memory takes at most (1024
 // values: the tensor pipe's float32 accumulation stays short); a longer tile adds its
 // segments into the float32 partial in order with round-to-nearest adds
@@ -115,7 +116,7 @@ constexpr int SEG_SL = 16;
 struct LayoutB {
     static constexpr int KST = 2;
     static constexpr uint32_t Q_TILE = OBLK * 64 * 2;    // [128 o][64 s]
-    static constexpr uint32_t Y_TILE = RB * 64 * 2;      // [256 r][64 s]
+    static constexpr uint32_t Y_TILE = RB * 64 * 2;      // [rbw r][64 s]
     // Q hi, Q lo, Yt hi, Yt lo (which = 0) or Qbar hi, Qbar lo, Y2t hi, Y2t lo (which = 1)
     static constexpr uint32_t STAGE = 2 * Q_TILE + 2 * Y_TILE;
     static constexpr uint32_t BAR = KST * STAGE;
@@ -128,6 +129,7 @@ enum { C_KFULL = 0, C_KEMPTY = 2, C_ACCFULL = 4, C_ACCEMPTY = 6, C_DRAIN = 8, C_
 
 struct ContractArgs {
     int64_t S, O, R, s_per;   // s_per: a multiple of 64
+    int rbw;                  // r per tile (rank_block_rows)
     float* Apart;             // [splits][R][O]
     float* Bpart;
 };
@@ -169,7 +171,8 @@ __global__ void __launch_bounds__(mats::A_THREADS, 1)
                  const __grid_constant__ CUtensorMap tmQbl) {
     using namespace mats;
     using L = LayoutA<RP>;
-    constexpr int KST = L::KST, KS = RP / 64;
+    constexpr int KST = L::KST;
+    const int KS = a.ks;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -328,7 +331,7 @@ __global__ void __launch_bounds__(mats::A_THREADS, 1)
                 // a new o-block: its X hi rows into tensor memory (every GEMM of the previous
                 // tile has completed: its last Z was read below)
 #pragma unroll 1
-                for (int unit = cg; unit < RP / 32; unit += 4)
+                for (int unit = cg; unit < 2 * KS; unit += 4)
                     x_to_tmem(a.X, a.rp, o, unit, tmem + L::TX + lane_off);
                 tmem_st_wait();
                 tc_fence_before();
@@ -496,12 +499,12 @@ __global__ void __launch_bounds__(mats::B_THREADS, 1)
                         break;
                     const uint32_t dst = sbase + st * L::STAGE;
                     const int32_t s0 = (int32_t)(x.s_begin + 64 * (int64_t)sl);
-                    const int32_t r0 = RB * x.rb, o0 = (int32_t)x.o0;
+                    const int32_t r0 = a.rbw * x.rb, o0 = (int32_t)x.o0;
                     uint64_t* fb = &bar[C_KFULL + st];
-                    mbar_arrive_expect_tx(fb, L::STAGE);
+                    mbar_arrive_expect_tx(fb, 2 * L::Q_TILE + 2 * (uint32_t)a.rbw * 128u);
                     tma_load_2d(dst, mq, s0, o0, fb);                             // [128 o][64 s]
                     tma_load_2d(dst + L::Q_TILE, mql, s0, o0, fb);
-                    tma_load_2d(dst + 2 * L::Q_TILE, my, s0, r0, fb);             // [256 r][64 s]
+                    tma_load_2d(dst + 2 * L::Q_TILE, my, s0, r0, fb);             // [rbw r][64 s]
                     tma_load_2d(dst + 2 * L::Q_TILE + L::Y_TILE, myl, s0, r0, fb);
                 }
             }
@@ -513,7 +516,7 @@ __global__ void __launch_bounds__(mats::B_THREADS, 1)
         if (lane == 0) {
             bool ok = true;
             int j = 0, sg = 0;
-            constexpr uint32_t idesc = idesc_bf16(OBLK, RB);
+            const uint32_t idesc = idesc_bf16(OBLK, (uint32_t)a.rbw);
             for (int t = t_first; ok && t < ntiles; t += t_step) {
                 const int nsl = b_tile(t, nob, nrb, nsplit, a).nsl;
                 // segments of at most SEG_SL K-slices, each into the next accumulator
@@ -582,17 +585,26 @@ __global__ void __launch_bounds__(mats::B_THREADS, 1)
                     if (o < a.O) {
                         // the tile's segments in order: the first writes, the later ones add
                         // (the previous sums' loads all issued before any store)
-                        const int64_t r0 = (int64_t)RB * x.rb + 128 * hf + 32 * c;
+                        const int64_t r0 = (int64_t)a.rbw * x.rb + 128 * hf + 32 * c;
                         float* col = dst + (base + r0) * a.O + o;
-                        const int64_t left = a.R - r0;
-                        const int nr = left < 32 ? (int)left : 32;
-                        float prev[32];
+                        const int left = min((int)(a.R - r0), a.rbw - 128 * hf - 32 * c);
+                        const int nr = min(left, 32);
+                        if (sl0 > 0) {
+                            float prev[32];
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            prev[i] = (sl0 > 0 && i < nr) ? col[(int64_t)i * a.O] : 0.f;
+                            for (int i = 0; i < 32; ++i)
+                                prev[i] = i < nr ? col[(int64_t)i * a.O] : 0.f;
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (i < nr) col[(int64_t)i * a.O] = prev[i] + __uint_as_float(r32[i]);
+                            for (int i = 0; i < 32; ++i)
+                                if (i < nr) col[(int64_t)i * a.O] = prev[i] + __uint_as_float(r32[i]);
+                        } else if (nr >= 32) {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) col[(int64_t)i * a.O] = __uint_as_float(r32[i]);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i)
+                                if (i < nr) col[(int64_t)i * a.O] = __uint_as_float(r32[i]);
+                        }
                     }
                 }
                 tc_fence_before();
@@ -623,7 +635,7 @@ int launch_mats(const TcOperands& op, const TcMaps& m, float* Apart, float* Bpar
     ra.s_per = (chunks + nsa - 1) / nsa * SC;
     const int splits_a = (int)((op.S + ra.s_per - 1) / ra.s_per);
     ra.V = op.V; ra.vs = op.vs;
-    ra.X = static_cast<const bf16*>(op.Xk); ra.rp = RP;
+    ra.X = static_cast<const bf16*>(op.Xk); ra.rp = RP; ra.ks = rank_slices(op.R);
     ra.status = status;
     {
         const uint32_t smem = LayoutA<RP>::TOTAL + 1024;
@@ -639,13 +651,14 @@ int launch_mats(const TcOperands& op, const TcMaps& m, float* Apart, float* Bpar
     }
     ContractArgs ca{};
     ca.S = op.S; ca.O = op.O; ca.R = op.R; ca.s_per = s_per;
+    ca.rbw = rank_block_rows(op.R);
     ca.Apart = Apart; ca.Bpart = Bpart;
     const uint32_t smem = LayoutB::TOTAL + 1024;
     auto k = k_tcs_contract<WITH_B>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return DNA_ERR_CUDA;
-    const int nrb = RP / RB;
+    const int nrb = rank_blocks(op.R);
     const int ntiles = (WITH_B ? 2 : 1) * nrb * nob * splits;
     const int grid = op.ctas > 0 ? std::min(op.ctas, ntiles) : ntiles;
     dna::launch_pdl(k, grid, dim3(B_THREADS), smem, st, ca, nob, nrb, splits, ntiles, status, m.q,

@@ -1,4 +1,5 @@
-"""Ranks above 256 in float32, where the candidates kernel walks r in groups of 32 and
+"""Ranks above 128, where the tensor-core forms take only the 64-wide slices of a padded rank
+that hold values and cut r into equal blocks; and ranks above 256 in float32, where the candidates kernel walks r in groups of 32 and
 writes the bf16 rows of the tensor-core forms: the edges of its rank range, column counts
 that leave a partial CTA, one and several splits of the sums.  Each half-step starts from
 the GPU's own state and is held to the element-wise one-step bounds of gpu_helpers; the FP32
@@ -33,6 +34,12 @@ def one_iteration(form, N, T, R):
             W, H, _ = (o.dna_step_h if which == 0 else o.dna_step_w)(V, W0, H0, choice=mask)
             Wg, Hg = gp.WH()
             assert rel_fro(Wg, W) < TOL[form] and rel_fro(Hg, H) < TOL[form], which
+
+
+@pytest.mark.parametrize("form", ["f32t", "bf16"])
+@pytest.mark.parametrize("R", [129, 144, 145, 192, 193, 256, 300, 320, 400, 448, 449])
+def test_rank_slices(form, R):
+    one_iteration(form, 700, 1300, R)
 
 
 @pytest.mark.parametrize("form", ["f32", "f32t", "bf16"])
