@@ -356,7 +356,9 @@ void plan_all(dna_ctx* c) {
 
 void free_all(dna_ctx* c) {
     void* ptrs[] = {c->own_V, c->own_W, c->own_H, c->Vt, c->colsum_v, c->rowsum_v, c->c, c->sig,
-                    c->fwork, c->gpart, c->vpart, c->Apart, c->Bpart, c->Xmu, c->Xdna, c->dpart, c->dfin_h, c->dfin_w,
+                    c->fwork, c->gpart, c->vpart, c->Apart, c->Bpart, c->Xmu, c->Xdna,
+                    c->Bpart ? nullptr : c->dpart,   // behind Bpart in the dense forms
+                    c->dfin_h, c->dfin_w,
                     c->choice_h, c->choice_w, c->kl_dev, c->kl_part, c->status, c->Xk, c->Yk, c->Ytk,
                     c->Y2tk, c->Xmk, c->Xdk, c->Vp, c->Qg, c->Qbg, c->cptr, c->ridx, c->cval, c->Hr, c->Wr, c->c0,
                     c->seg_col[0], c->seg_col[1], c->seg_k0[0], c->seg_k0[1], c->seg_k1[0],
@@ -395,10 +397,13 @@ int alloc_workspace(dna_ctx* c) {
     e |= dmalloc(&c->gpart, sizeof(double) * (size_t)(dna::Simt<Tp>::glue_parts(M) * R));
     e |= dmalloc(&c->vpart, sizeof(double) * (size_t)(((N + 31) / 32) * T + ((T + 31) / 32) * N));
     e |= dmalloc(&c->Apart, sizeof(Tp) * (size_t)ap);
-    e |= dmalloc(&c->Bpart, sizeof(Tp) * (size_t)ap);
+    // the cost slots behind the partial sums (one allocation: cudaMalloc takes a new 2 MB page
+    // when the small blocks outgrow the last one, about 0.5 ms)
+    const size_t bp = (sizeof(Tp) * (size_t)ap + 255) / 256 * 256;
+    e |= dmalloc(&c->Bpart, bp + sizeof(double) * (size_t)dp);
+    if (c->Bpart) c->dpart = reinterpret_cast<double*>(static_cast<char*>(c->Bpart) + bp);
     e |= dmalloc(&c->Xmu, sizeof(Tp) * (size_t)(R * M));
     e |= dmalloc(&c->Xdna, sizeof(Tp) * (size_t)(R * M));
-    e |= dmalloc(&c->dpart, sizeof(double) * (size_t)dp);
     e |= dmalloc(&c->dfin_h, sizeof(double) * 2 * T);
     e |= dmalloc(&c->dfin_w, sizeof(double) * 2 * N);
     e |= dmalloc(&c->choice_h, (size_t)T);
