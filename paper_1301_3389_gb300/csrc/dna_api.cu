@@ -438,8 +438,6 @@ int alloc_workspace(dna_ctx* c) {
         }
     }
     if (e != DNA_OK) return DNA_ERR_ALLOC;
-    // the padding columns of the transposed copy of V are read by 16-byte copies: zero them
-    if (cudaMemset(c->Vt, 0, sizeof(Tp) * (size_t)T * c->ldvt) != cudaSuccess) return DNA_ERR_CUDA;
     if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess) return DNA_ERR_CUDA;
     if (cudaMemset(c->choice_h, 0, (size_t)T) != cudaSuccess) return DNA_ERR_CUDA;
     if (cudaMemset(c->choice_w, 0, (size_t)N) != cudaSuccess) return DNA_ERR_CUDA;
@@ -580,6 +578,14 @@ int bind_csr(dna_ctx* c, const int64_t* rptr, const int32_t* cidx, const Tp* val
 
 template <typename Tp>
 int prepare(dna_ctx* c, const void* Vsrc = nullptr) {
+    // the padding columns of the transposed copy of V are read by 16-byte copies: zero them, on
+    // the context's stream (a clear on the default stream could land behind work queued there,
+    // after the copy was made)
+    if (c->ldvt > c->N &&
+        cudaMemset2DAsync(static_cast<Tp*>(c->Vt) + c->N, sizeof(Tp) * (size_t)c->ldvt, 0,
+                          sizeof(Tp) * (size_t)(c->ldvt - c->N), (size_t)c->T,
+                          c->stream) != cudaSuccess)
+        return DNA_ERR_CUDA;
     // Vsrc: V in pinned host memory, read by the transpose kernel and copied into c->V
     return phase(c, DNA_PHASE_PREPARE, 3, [&] {
         return dna::Simt<Tp>::prepare_v(
@@ -1391,7 +1397,8 @@ int dna_bind(dna_ctx* c, const void* V, int64_t ldv, void* W, void* H) {
         c->ldvp = (c->T + 3) / 4 * 4;
         if (!c->Vp) {
             if (dmalloc(&c->Vp, sizeof(float) * (size_t)(c->N * c->ldvp))) return DNA_ERR_ALLOC;
-            if (cudaMemset(c->Vp, 0, sizeof(float) * (size_t)(c->N * c->ldvp)) != cudaSuccess)
+            if (cudaMemsetAsync(c->Vp, 0, sizeof(float) * (size_t)(c->N * c->ldvp), c->stream) !=
+                cudaSuccess)
                 return DNA_ERR_CUDA;
         }
         if (cudaMemcpy2DAsync(c->Vp, sizeof(float) * c->ldvp, V, sizeof(float) * ldv,
