@@ -1,5 +1,5 @@
 // Fused per-half-step kernels between the two O(NRT) passes, for the single-problem path:
-//   k_cand_fused   candidates (steps 6 and 11, eq. 10, 11, 15, 17) and, for the tensor-core
+//   k_cand_reg, k_cand_wide, k_cand_fused   candidates (steps 6 and 11, eq. 10, 11, 15, 17) and, for the tensor-core
 //                  form, their bf16 operand copies;
 //   k_select_fused selection (steps 15 / 28) and the per-block partial sums of the new
 //                  factor that the step 16 / 29 normalisation divides by;
