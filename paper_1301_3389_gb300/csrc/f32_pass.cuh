@@ -458,6 +458,11 @@ __device__ __forceinline__ void two_add(float& s, float& e, float t) {
     e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(t, b)));
     s = n;
 }
+// The value of such a sum: s alone once a term was infinite or NaN (the error term of an
+// infinite sum is inf - inf), so that an infinite cost stays infinite.
+__device__ __forceinline__ double two_value(float s, float e) {
+    return isfinite(s) ? (double)s + (double)e : (double)s;
+}
 
 template <int RPT, int NC>
 struct Pass2 : Tiles<RPT> {
@@ -549,7 +554,7 @@ __device__ __forceinline__ void pass2_tile(const View& v, const float* __restric
     for (int k = 0; k < NC; ++k)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            red[(zp.sl * NC + k) * OB + 4 * zp.ol + j] = (double)hi[k][j] + (double)lo[k][j];
+            red[(zp.sl * NC + k) * OB + 4 * zp.ol + j] = two_value(hi[k][j], lo[k][j]);
     __syncthreads();
     const int tid = threadIdx.x;
     if (tid < NC * OB) {

@@ -104,7 +104,11 @@ struct Sum<float> {
         add(b);
         e = __fadd_rn(e, eb);
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+    // s alone once a term was infinite or NaN (e is then inf - inf): an infinite cost stays
+    // infinite
+    __device__ __forceinline__ double value() const {
+        return isfinite(s) ? (double)s + (double)e : (double)s;
+    }
 };
 // the sum over groups of LPN lanes
 template <int LPN, typename Tp>

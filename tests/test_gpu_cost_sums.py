@@ -1,0 +1,107 @@
+"""The sums behind the selection and d_KL in the float32 forms: an infinite term (z = 0 where
+v > 0) leaves +infinity, as float64 sums would, not a value that no comparison holds for; the
+call reports DNA_ERR_NONFINITE all the same."""
+import ctypes
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _lib():
+    import paper_1301_3389_gb300._lib as L
+    return L
+
+
+class Bound:
+    """V, W, H bound to a context of the dense or sparse form, or to a group of one problem."""
+
+    def __init__(self, form, V, W, H):
+        import torch
+        L = self.L = _lib()
+        self.form = form
+        self.N, self.T = V.shape
+        R = W.shape[1]
+        V, self.W, self.H = (torch.from_numpy(np.ascontiguousarray(x, dtype=np.float32)).cuda()
+                             for x in (V, W, H))
+        self.keep = [V]
+        bf16 = form in ("bf16", "group_bf16")
+        opts = L.make_opts(dtype=L.DNA_BF16 if bf16 else L.DNA_F32)
+        if form.startswith("group"):
+            self.h = L.dna_group_create([self.N], [self.T], [R], opts)
+            L.dna_group_set_stream(self.h)
+            L.dna_group_bind(self.h, [V], [self.W], [self.H])
+        elif form == "sparse":
+            nz = V.nonzero()
+            rows = torch.bincount(nz[:, 0], minlength=self.N).cumsum(0)
+            self.keep = [torch.cat([rows.new_zeros(1), rows]), nz[:, 1].to(torch.int32),
+                         V[nz[:, 0], nz[:, 1]].contiguous()]
+            self.h = L.dna_create_sparse(self.N, self.T, R, nz.shape[0], opts)
+            L.dna_set_stream(self.h)
+            L.dna_bind_csr(self.h, *self.keep, self.W, self.H)
+        else:
+            self.h = L.dna_create(self.N, self.T, R, opts)
+            L.dna_set_stream(self.h)
+            L.dna_bind(self.h, V, self.W, self.H)
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        (self.L.dna_group_destroy if self.form.startswith("group") else self.L.dna_destroy)(self.h)
+
+    def step(self, which):
+        g = "group_" if self.form.startswith("group") else ""
+        getattr(self.L, f"dna_{g}step_{'HW'[which]}")(self.h)
+
+    def kl(self):
+        """(return code, value)"""
+        if self.form.startswith("group"):
+            out = np.zeros(1)
+            return self.L.LIB.dna_group_kl(self.h, out.ctypes.data), float(out[0])
+        out = ctypes.c_double()
+        return self.L.LIB.dna_kl(self.h, ctypes.byref(out)), out.value
+
+    def choice(self, which):
+        out = np.zeros((self.T, self.N)[which], dtype=np.uint8)
+        if self.form.startswith("group"):
+            code = self.L.LIB.dna_group_get_choice(self.h, 0, which, out.ctypes.data, len(out))
+        else:
+            code = self.L.LIB.dna_get_choice(self.h, which, out.ctypes.data, len(out))
+        return code, out
+
+    def costs(self, which):
+        dm, dd = np.zeros((self.T, self.N)[which]), np.zeros((self.T, self.N)[which])
+        code = self.L.LIB.dna_get_costs(self.h, which, dm.ctypes.data, dd.ctypes.data, len(dm))
+        return code, dm, dd
+
+
+@pytest.mark.parametrize("which", [0, 1])
+@pytest.mark.parametrize("form", ["f32", "group_f32", "sparse"])
+def test_infinite_mu_cost_keeps_newton(form, which):
+    """Column 0 (row 0 for the W step): the MU gain of component a is v y / z = 2e-38, so the
+    MU z of row 0, 1e-8 * 2e-38, underflows to 0 where v = 2e-38 > 0: infinite cost.  The
+    Newton gain is floored at eps = 0.01 and its cost is finite."""
+    V = np.array([[2e-38, 0.0, 1.0], [0.0, 1.0, 2.0], [1.0, 1.0, 3.0]])
+    Y = np.array([[1e-8, 0.0], [1.0, 0.0], [0.0, 1.0]])
+    X = np.ones((2, 3))
+    # the third column needs z > 0 everywhere; its selection does not matter
+    with Bound(form, *((V, Y, X) if which == 0 else (V.T, X.T, Y.T))) as b:
+        b.step(which)
+        code, choice = b.choice(which)
+        assert code == b.L.DNA_ERR_NONFINITE and choice[0] == 1
+        if not form.startswith("group"):
+            code, dm, dd = b.costs(which)
+            assert code == b.L.DNA_ERR_NONFINITE
+            assert dm[0] == np.inf and np.isfinite(dd[0]) and np.isfinite(dm[1:]).all()
+
+
+@pytest.mark.parametrize("R", [4, 40])
+@pytest.mark.parametrize("form", ["f32", "bf16", "group_f32", "group_bf16", "sparse"])
+def test_infinite_kl(form, R):
+    rng = np.random.default_rng(R)
+    V, W, H = rng.random((150, 70)) + 0.1, rng.random((150, R)), rng.random((R, 70))
+    W[5] = 0.0
+    with Bound(form, V, W, H) as b:
+        assert b.kl() == (b.L.DNA_ERR_NONFINITE, np.inf)
