@@ -161,8 +161,8 @@ int mu_step(dna_ctx* ctx, int which);
 int mu_iterate(dna_ctx* ctx, int iters);
 
 /* d_KL(V, W H) of eq. 1 in float64, written to *out (host memory): per element
- * z + v log(v / z) - v (z where v = 0), summed in float32 over short runs and in float64
- * beyond.  Z is formed by the context's engine (for F32 with ENGINE_TENSOR: the split
+ * z + v log(v / z) - v (z where v = 0), summed in float32 over short runs and no coarser
+ * than in float64 beyond (float64, or three float32 values per sum).  Z is formed by the context's engine (for F32 with ENGINE_TENSOR: the split
  * bf16 tensor-core product; for BF16: the CUDA-core float32 product).  Synchronises the
  * context's stream; also returns any error recorded by earlier kernels. */
 int dna_kl(dna_ctx* ctx, double* out);

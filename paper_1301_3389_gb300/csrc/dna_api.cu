@@ -99,6 +99,7 @@ struct dna_ctx {
     void* Hr = nullptr;      // H^t as rows (T x R4)
     void* Wr = nullptr;      // W as padded rows (N x R4), used where W's own rows are not
     double* c0 = nullptr;
+    void* c3 = nullptr;      // c0 as sums of three values [3][<= 128]
     // segments of at most sparse::SEG non-zeros per view (0: columns of V, 1: rows), built
     // at bind, with their partial sums
     int32_t* seg_col[2] = {nullptr, nullptr};
@@ -360,7 +361,7 @@ void free_all(dna_ctx* c) {
                     c->Bpart ? nullptr : c->dpart,   // behind Bpart in the dense forms
                     c->dfin_h, c->dfin_w,
                     c->choice_h, c->choice_w, c->kl_dev, c->kl_part, c->status, c->Xk, c->Yk, c->Ytk,
-                    c->Y2tk, c->Xmk, c->Xdk, c->Vp, c->Qg, c->Qbg, c->cptr, c->ridx, c->cval, c->Hr, c->Wr, c->c0,
+                    c->Y2tk, c->Xmk, c->Xdk, c->Vp, c->Qg, c->Qbg, c->cptr, c->ridx, c->cval, c->Hr, c->Wr, c->c0, c->c3,
                     c->seg_col[0], c->seg_col[1], c->seg_k0[0], c->seg_k0[1], c->seg_k1[0],
                     c->seg_k1[1], c->seg_ptr[0], c->seg_ptr[1], c->Aseg, c->Bseg, c->dseg,
                     c->dcur, c->wg_part, c->wg_cpart};
@@ -457,6 +458,7 @@ int alloc_sparse_workspace(dna_ctx* c) {
     e |= dmalloc(&c->rowsum_v, sizeof(double) * N);
     e |= dmalloc(&c->c, sizeof(double) * R);
     e |= dmalloc(&c->c0, sizeof(double) * R);
+    e |= dmalloc(&c->c3, sizeof(Tp) * 3 * 128);
     e |= dmalloc(&c->sig, sizeof(double) * R);
     e |= dmalloc(&c->fwork, sizeof(double) * dna::FSUM_SPLITS * R);
     e |= dmalloc(&c->gpart, sizeof(double) * (size_t)(dna::Simt<Tp>::glue_parts(M) * R));
@@ -555,7 +557,7 @@ int bind_csr(dna_ctx* c, const int64_t* rptr, const int32_t* cidx, const Tp* val
         if (q) cudaFree(q);
     if (dmalloc(&c->Aseg, sizeof(Tp) * (size_t)(maxseg * c->R4)) ||
         dmalloc(&c->Bseg, sizeof(Tp) * (size_t)(maxseg * c->R4)) ||
-        dmalloc(&c->dseg, sizeof(double) * (size_t)(2 * maxseg)))
+        dmalloc(&c->dseg, (sizeof(Tp) == 4 ? 32 : 16) * (size_t)maxseg))
         return DNA_ERR_ALLOC;
     for (int w = 0; w < 2; ++w) {
         const int64_t O = w ? N : T;
@@ -950,7 +952,7 @@ int sparse_half_step(dna_ctx* c, int w, bool mu_only, bool prepared, bool next) 
     if (!e)
         e = phase(c, DNA_PHASE_CANDIDATES, 1, [&] {
             return S::sp_cand(v, sg, Aseg, Bseg, Xr, c->R4, c->c, Xm, Xd, c->o.eps, c->o.alpha,
-                              mu_only, st);
+                              mu_only, c->c0, static_cast<Tp*>(c->c3), st);
         });
     if (!e && !mu_only)
         e = phase(c, DNA_PHASE_PASS2, 1, [&] {
@@ -958,7 +960,7 @@ int sparse_half_step(dna_ctx* c, int w, bool mu_only, bool prepared, bool next) 
         });
     if (!e)
         e = phase(c, DNA_PHASE_SELECT, 1, [&] {
-            return S::sp_select(v, sg, c->dseg, Xm, Xd, c->R4, c->c0, w ? c->choice_w : c->choice_h,
+            return S::sp_select(v, sg, c->dseg, Xm, Xd, c->R4, static_cast<const Tp*>(c->c3), w ? c->choice_w : c->choice_h,
                                 w ? c->dfin_w : c->dfin_h, c->gpart, w ? c->o.rho : c->o.lambda,
                                 mu_only, c->status, st);
         });

@@ -204,13 +204,13 @@ template <typename Tp> struct Simt {
                         int* status, cudaStream_t st);
     static int sp_cand(const View& v, const SparseSegs& sg, const Tp* Aseg, const Tp* Bseg,
                        const Tp* Xr, int64_t R4, const double* c, Tp* Xm, Tp* Xd, double eps,
-                       double alpha, bool mu, cudaStream_t st);
+                       double alpha, bool mu, const double* c0, Tp* c3, cudaStream_t st);
     static int sp_pass2(int64_t R, const SparseSegs& sg, const int32_t* idx, const Tp* val,
                         const Tp* Yr, const Tp* Xm, const Tp* Xd, int64_t R4, double* dseg,
                         cudaStream_t st);
     // selection and the new X with its per-block sums fpart (mu: Xm is kept)
     static int sp_select(const View& v, const SparseSegs& sg, const double* dseg, const Tp* Xm,
-                         const Tp* Xd, int64_t R4, const double* c0, uint8_t* choice, double* dfin,
+                         const Tp* Xd, int64_t R4, const Tp* c3, uint8_t* choice, double* dfin,
                          double* fpart, double reg, bool mu, int* status, cudaStream_t st);
     static int sp_kl(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
                      const Tp* Yr, const Tp* Xr, int64_t R4, const double* c0, double* dseg,

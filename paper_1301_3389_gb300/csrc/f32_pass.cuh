@@ -31,6 +31,7 @@
 #include <stdint.h>
 
 #include "dna_internal.h"
+#include "sum3.cuh"
 
 namespace dna {
 namespace f2 {
@@ -450,121 +451,194 @@ __device__ __forceinline__ void pass1_tile(const View& v, float* __restrict__ Ap
     }
 }
 
-// s += t with the rounding error kept in e (the two-sum of Knuth): the cost sums run over
-// thousands of chunks, and a float64 add per chunk and column would cost more than the
-// chunk's FMAs at small ranks (64 cycles a warp instruction on this GPU).
-__device__ __forceinline__ void two_add(float& s, float& e, float t) {
-    const float n = __fadd_rn(s, t), b = __fsub_rn(n, s);
-    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(t, b)));
-    s = n;
-}
-// The value of such a sum: s alone once a term was infinite or NaN (the error term of an
-// infinite sum is inf - inf), so that an infinite cost stays infinite.
-__device__ __forceinline__ double two_value(float s, float e) {
-    return isfinite(s) ? (double)s + (double)e : (double)s;
-}
+// Chunks after which pass 2 moves its Sum3 to float64 (sum3.cuh: a run this long is at least as
+// exact as float64 adds).
+constexpr int SUM_RUN = 256;
 
 template <int RPT, int NC>
 struct Pass2 : Tiles<RPT> {
     using T = Tiles<RPT>;
     static constexpr int STAGES = NC == 1 || RPT <= 6 ? 2 : 1;
     static constexpr size_t tiles = sizeof(float) * (NC * T::X + STAGES * T::Y);
-    static constexpr size_t red = sizeof(double) * 16 * NC * OB;
+    static constexpr size_t red = 3 * sizeof(float) * 16 * NC * OB;
     static constexpr size_t smem = tiles > red ? tiles : red;
 };
 
-// Cost partials of NC candidates for one (o-block, split of s): dpart [splits][NC][O].
+// This thread's cost sums of NC candidates over one (o-block, split of s), for the columns
+// 4 ol + j: chunks of four terms in float32, added up in S (Sum3 or Sum64), which after
+// every SUM_RUN chunks but the last ones is moved to acc.
 // FULL = false: sum_{v>0} (-v log z) + sum z; FULL = true: the terms of eq. 1.
-template <int RPT, int NC, bool FULL>
-__device__ __forceinline__ void pass2_tile(const View& v, const float* __restrict__ X0,
+template <int RPT, int NC, bool FULL, class S>
+__device__ __forceinline__ void pass2_sums(const View& v, const float* __restrict__ X0,
                                            const float* __restrict__ X1, int64_t xr, int64_t xo,
-                                           double* __restrict__ dpart, int64_t s_per,
-                                           int* __restrict__ status, int64_t tile_o,
-                                           int64_t tile_s, float* sm) {
+                                           int64_t o0, int64_t s_begin, int64_t s_end, int nch,
+                                           int& bad, float* sm, S (&sums)[NC][4],
+                                           double* __restrict__ acc) {
     using H = Pass2<RPT, NC>;
     constexpr int ST = H::STAGES;
     float* Xs = sm;                       // [NC][RB][LDX]
     float* Ys = Xs + NC * H::X;           // [ST][64 s][LDR]
     const float* __restrict__ V = static_cast<const float*>(v.V);
     const float* __restrict__ Y = static_cast<const float*>(v.Y);
-    const int64_t o0 = tile_o * OB;
-    const int64_t s_begin = tile_s * s_per, s_end = min(v.S, s_begin + s_per);
-    const int nch = (int)((s_end - s_begin + SB - 1) / SB);
     const int nq = (int)((v.R + 3) / 4);
     const bool wide = v_wide(v);
     const ZPos zp = z_pos();
 
-    float hi[NC][4], lo[NC][4];
-#pragma unroll
-    for (int c = 0; c < NC; ++c)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) { hi[c][j] = 0.f; lo[c][j] = 0.f; }
     load_x<H::RB>(Xs, X0, xr, xo, o0, v.O, v.R);
     if (NC > 1) load_x<H::RB>(Xs + H::X, X1, xr, xo, o0, v.O, v.R);
     load_y<H::RB>(Ys, Y, v.ys, v.yr, s_begin, v.S, v.R);
     cp_commit();
-    int bad = 0;
-    for (int c = 0; c < nch; ++c) {
-        const int64_t s0 = s_begin + (int64_t)c * SB;
-        const float* Yc = Ys + (ST == 2 ? (c & 1) * H::Y : 0);
-        if (ST == 1 && c > 0) {
+    for (int c0 = 0; c0 < nch; c0 += SUM_RUN) {
+        const int c1 = min(nch, c0 + SUM_RUN);
+        for (int c = c0; c < c1; ++c) {
+            const int64_t s0 = s_begin + (int64_t)c * SB;
+            const float* Yc = Ys + (ST == 2 ? (c & 1) * H::Y : 0);
+            if (ST == 1 && c > 0) {
+                __syncthreads();
+                load_y<H::RB>(Ys, Y, v.ys, v.yr, s0, v.S, v.R);
+                cp_commit();
+            }
+            float vv[4][4];   // in flight behind the z FMAs
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                load_v(v, V, wide, s0 + zp.sl + 16 * i, s_end, o0 + 4 * zp.ol, vv[i]);
+            cp_wait<0>();
             __syncthreads();
-            load_y<H::RB>(Ys, Y, v.ys, v.yr, s0, v.S, v.R);
-            cp_commit();
+            if (ST == 2 && c + 1 < nch) {
+                load_y<H::RB>(Ys + (~c & 1) * H::Y, Y, v.ys, v.yr, s0 + SB, v.S, v.R);
+                cp_commit();
+            }
+            u64 z[NC][4][2];
+            z_tile<H::RB, NC>(Yc, Xs, zp, nq, z);
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                float run[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 z0 = unpack2(z[k][i][0]), z1 = unpack2(z[k][i][1]);
+                    const float zr[4] = {z0.x, z0.y, z1.x, z1.y};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float zz = zr[j], x = vv[i][j];
+                        const bool pos = x > 0.f;
+                        bad |= (pos && !(zz > 0.f)) ? 1 : 0;
+                        // branch-free: the v = 0 terms are discarded by the select
+                        const float t = FULL ? (x * logf(x / zz) - x) : (-x * logf(zz));
+                        run[j] += pos ? zz + t : zz;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sums[k][j].add(run[j]);
+            }
         }
-        float vv[4][4];   // in flight behind the z FMAs
+        if (c1 < nch)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            load_v(v, V, wide, s0 + zp.sl + 16 * i, s_end, o0 + 4 * zp.ol, vv[i]);
-        cp_wait<0>();
-        __syncthreads();
-        if (ST == 2 && c + 1 < nch) {
-            load_y<H::RB>(Ys + (~c & 1) * H::Y, Y, v.ys, v.yr, s0 + SB, v.S, v.R);
-            cp_commit();
-        }
-        u64 z[NC][4][2];
-        z_tile<H::RB, NC>(Yc, Xs, zp, nq, z);
-#pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            float run[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 z0 = unpack2(z[k][i][0]), z1 = unpack2(z[k][i][1]);
-                const float zr[4] = {z0.x, z0.y, z1.x, z1.y};
+            for (int k = 0; k < NC; ++k)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float zz = zr[j], x = vv[i][j];
-                    const bool pos = x > 0.f;
-                    bad |= (pos && !(zz > 0.f)) ? 1 : 0;
-                    // branch-free: the v = 0 terms are discarded by the select
-                    const float t = FULL ? (x * logf(x / zz) - x) : (-x * logf(zz));
-                    run[j] += pos ? zz + t : zz;
+                    acc[4 * k + j] = (c0 ? acc[4 * k + j] : 0.0) + sums[k][j].value();
+                    sums[k][j] = S();
                 }
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) two_add(hi[k][j], lo[k][j], run[j]);
-        }
     }
-    if (bad) atomicOr(status, STATUS_NONFINITE);
+}
 
-    // the 16 threads of each column, added in order
-    __syncthreads();
-    double* red = reinterpret_cast<double*>(sm);   // [16][NC][64]
+// The threads' float64 sums into red [16][NC][64].
+template <int NC, class S>
+__device__ __forceinline__ void put_sums(double* __restrict__ red, ZPos zp,
+                                         const S (&sums)[NC][4], const double* __restrict__ acc,
+                                         bool moved) {
 #pragma unroll
     for (int k = 0; k < NC; ++k)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            red[(zp.sl * NC + k) * OB + 4 * zp.ol + j] = two_value(hi[k][j], lo[k][j]);
+            red[(zp.sl * NC + k) * OB + 4 * zp.ol + j] =
+                (moved ? acc[4 * k + j] : 0.0) + sums[k][j].value();
+}
+
+// The tile once more with float64 adds (rare: a call of its own, so that the usual path keeps
+// its registers).
+template <int RPT, int NC, bool FULL>
+__device__ __noinline__ void pass2_again(const View& v, const float* X0, const float* X1,
+                                         int64_t xr, int64_t xo, int64_t o0, int64_t s_begin,
+                                         int64_t s_end, int nch, float* sm) {
+    Sum64 sums[NC][4];
+    double acc[4 * NC];
+    int bad = 0;
+    pass2_sums<RPT, NC, FULL>(v, X0, X1, xr, xo, o0, s_begin, s_end, nch, bad, sm, sums, acc);
     __syncthreads();
-    const int tid = threadIdx.x;
-    if (tid < NC * OB) {
-        const int k = tid / OB, oo = tid % OB;
-        double sum = 0.0;
+    put_sums<NC>(reinterpret_cast<double*>(sm), z_pos(), sums, acc, nch > SUM_RUN);
+}
+
+// Cost partials of NC candidates for one (o-block, split of s): dpart [splits][NC][O].  The
+// sums run as Sum3 (a float64 add per chunk and column would take as long as the chunk's FMAs
+// at small ranks; against pairs of float32, which are coarser than float64, iterations take
+// 55.6 -> 55.5 us at N=256 T=512 R=16, 590 -> 596 at N=1024 T=11554 R=80, and 1156 -> 1175 for
+// 48 problems in a group; a test of the range in the loop cost another 20).  Where a sum is
+// infinite or has left float32's range, the tile is formed once more with float64 adds.
+template <int RPT, int NC, bool FULL>
+__device__ __forceinline__ void pass2_tile(const View& v, const float* __restrict__ X0,
+                                           const float* __restrict__ X1, int64_t xr, int64_t xo,
+                                           double* __restrict__ dpart, int64_t s_per,
+                                           int* __restrict__ status, int64_t tile_o,
+                                           int64_t tile_s, float* sm) {
+    const int64_t o0 = tile_o * OB;
+    const int64_t s_begin = tile_s * s_per, s_end = min(v.S, s_begin + s_per);
+    const int nch = (int)((s_end - s_begin + SB - 1) / SB);
+    const ZPos zp = z_pos();
+    int bad = 0;
+    double acc_mem[4 * NC];   // long splits only: kept out of the registers
+    double* acc = acc_mem;
+    asm volatile("" : "+l"(acc));
+    Sum3 sums[NC][4];
+    pass2_sums<RPT, NC, FULL>(v, X0, X1, xr, xo, o0, s_begin, s_end, nch, bad, sm, sums, acc);
+    if (bad) atomicOr(status, STATUS_NONFINITE);
+
+    // the 16 threads of each column, added in order
+    const bool moved = nch > SUM_RUN;
+    bool redo = false;
 #pragma unroll
-        for (int h = 0; h < 16; ++h) sum += red[(h * NC + k) * OB + oo];
-        const int64_t o = o0 + oo;
-        if (o < v.O) dpart[(tile_s * NC + k) * v.O + o] = sum;
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            redo |= Sum3::large(sums[k][j].s) || isnan(sums[k][j].s);
+            if (moved) redo |= !isfinite(acc[4 * k + j]);
+        }
+    const int tid = threadIdx.x, k = tid / OB, oo = tid % OB;
+    double sum = 0.0;
+    redo = __syncthreads_or(redo);   // and every read of the tiles is done
+    if (redo || moved) {
+        double* red = reinterpret_cast<double*>(sm);   // [16][NC][64]
+        if (redo)
+            pass2_again<RPT, NC, FULL>(v, X0, X1, xr, xo, o0, s_begin, s_end, nch, sm);
+        else
+            put_sums<NC>(red, zp, sums, acc, moved);
+        __syncthreads();
+        if (tid < NC * OB)
+#pragma unroll
+            for (int h = 0; h < 16; ++h) sum += red[(h * NC + k) * OB + oo];
+    } else {   // as Sum3 too: one conversion to float64 per column
+        constexpr int PL = 16 * NC * OB;   // [s, e, f][16][NC][64]
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const Sum3* x = sums[c];
+            float* p = sm + (zp.sl * NC + c) * OB + 4 * zp.ol;
+            *reinterpret_cast<float4*>(p) = make_float4(x[0].s, x[1].s, x[2].s, x[3].s);
+            *reinterpret_cast<float4*>(p + PL) = make_float4(x[0].e, x[1].e, x[2].e, x[3].e);
+            *reinterpret_cast<float4*>(p + 2 * PL) = make_float4(x[0].f, x[1].f, x[2].f, x[3].f);
+        }
+        __syncthreads();
+        if (tid < NC * OB) {
+            Sum3 t;
+#pragma unroll
+            for (int h = 0; h < 16; ++h) {
+                const float* p = sm + (h * NC + k) * OB + oo;
+                t.add(p[0], p[PL], p[2 * PL]);
+            }
+            sum = t.value();
+        }
     }
+    const int64_t o = o0 + oo;
+    if (tid < NC * OB && o < v.O) dpart[(tile_s * NC + k) * v.O + o] = sum;
 }
 
 }  // namespace f2

@@ -571,13 +571,13 @@ int Simt<Tp>::sp_pass1(int64_t R, const SparseSegs& sg, const int32_t* idx, cons
 template <typename Tp>
 int Simt<Tp>::sp_cand(const View& v, const SparseSegs& sg, const Tp* Aseg, const Tp* Bseg,
                       const Tp* Xr, int64_t R4, const double* c, Tp* Xm, Tp* Xd, double eps,
-                      double alpha, bool mu, cudaStream_t st) {
+                      double alpha, bool mu, const double* c0, Tp* c3, cudaStream_t st) {
     return simt::by_lanes(v.R, [&](auto lpn) {
         constexpr int LPN = decltype(lpn)::value;
         const unsigned grid = simt::sp_grid((v.O + 32 / LPN - 1) / (32 / LPN));
         auto k = mu ? sparse::k_sp_cand<Tp, LPN, true> : sparse::k_sp_cand<Tp, LPN, false>;
         dna::launch_pdl(k, grid, dim3(sparse::WARPS * 32), 0, st, v.O, v.R, R4, sg.sptr, Aseg,
-                        Bseg, Xr, c, v.vsum, Xm, Xd, (Tp)eps, (Tp)alpha);
+                        Bseg, Xr, c, v.vsum, Xm, Xd, (Tp)eps, (Tp)alpha, c0, c3);
         return simt::launch_status();
     });
 }
@@ -596,13 +596,13 @@ int Simt<Tp>::sp_pass2(int64_t R, const SparseSegs& sg, const int32_t* idx, cons
 
 template <typename Tp>
 int Simt<Tp>::sp_select(const View& v, const SparseSegs& sg, const double* dseg, const Tp* Xm,
-                        const Tp* Xd, int64_t R4, const double* c0, uint8_t* choice, double* dfin,
+                        const Tp* Xd, int64_t R4, const Tp* c3, uint8_t* choice, double* dfin,
                         double* fpart, double reg, bool mu, int* status, cudaStream_t st) {
     return simt::by_lanes(v.R, [&](auto lpn) {
         constexpr int LPN = decltype(lpn)::value;
         auto k = mu ? sparse::k_sp_select<Tp, LPN, true> : sparse::k_sp_select<Tp, LPN, false>;
         dna::launch_pdl(k, dim3((unsigned)glue_parts(v.O)), dim3(sparse::WARPS * 32), 0, st, v,
-                        R4, sg.sptr, dseg, Xm, Xd, c0, choice, dfin, fpart, reg, status);
+                        R4, sg.sptr, dseg, Xm, Xd, c3, choice, dfin, fpart, reg, status);
         return simt::launch_status();
     });
 }

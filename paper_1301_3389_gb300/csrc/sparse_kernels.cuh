@@ -23,11 +23,12 @@
 // and 46, 61 us.)
 // Each segment writes its partial sums [seg][R4], which the candidates kernel adds per
 // column in order.  Sums over lanes run in a fixed order, so every result is
-// bit-reproducible; costs are summed across lanes in pairs of float32 (value and rounding
-// error, about 48 bits) because a float64 add costs 64 cycles per warp on this GPU.
+// bit-reproducible; the candidates' costs are summed across lanes and segments as three float32
+// values each (sum3.cuh, no coarser than float64) because a float64 add costs 64 cycles per
+// warp on this GPU.
 // Measured at 36771 x 10212, 1.34 M non-zeros, R = 64 (H and W view, microseconds): pass 1
 // 60, 73 -> 47, 66, pass 2 57, 70 -> 40, 54, sums of segments and candidates 20, 78 -> 6, 20,
-// cost sums and selection 27, 81 -> 7, 15.
+// cost sums and selection 27, 81 -> 9, 15.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -36,6 +37,7 @@
 
 #include "dna_internal.h"
 #include "simt_kernels.cuh"
+#include "sum3.cuh"
 
 namespace dna {
 namespace sparse {
@@ -66,55 +68,70 @@ __device__ __forceinline__ void store4(double* p, const Four<double>& x) {
     *reinterpret_cast<double2*>(p + 2) = make_double2(x.v[2], x.v[3]);
 }
 
-// A sum with its rounding error (float32), or a plain float64 sum.
+// A sum over lanes or segments that loses nothing against float64: float64 itself, or for
+// float32 values three of them (sum3.cuh).
 template <typename Tp>
 struct Sum;
 template <>
 struct Sum<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double t) { s += t; }
-    __device__ __forceinline__ void add_product(double hi, double lo, double x) {
-        s += (hi + lo) * x;
+    __device__ __forceinline__ void add_product(double c, double, double, double x) { s += c * x; }
+    // += what lane ^ m hands over
+    __device__ __forceinline__ void add_from(const Sum& mine, int m) {
+        s += __shfl_xor_sync(0xffffffffu, mine.s, m);
     }
-    __device__ __forceinline__ void add_lane(int m) { s += __shfl_xor_sync(0xffffffffu, s, m); }
+    // += lane ^ m's sum
+    __device__ __forceinline__ void add_lane(int m) { add_from(*this, m); }
+    __device__ __forceinline__ void add_sum(const Sum& x) { s += x.s; }
+    __device__ __forceinline__ bool past_range() const { return false; }
     __device__ __forceinline__ double value() const { return s; }
 };
 template <>
-struct Sum<float> {
-    float s = 0.f, e = 0.f;
-    __device__ __forceinline__ void add(float t) {   // two-sum of Knuth
-        const float n = __fadd_rn(s, t), b = __fsub_rn(n, s);
-        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(t, b)));
-        s = n;
-    }
-    // the exact product of x with the two-float number hi + lo, to float32 of the error
-    __device__ __forceinline__ void add_product(float hi, float lo, float x) {
-        const float p = __fmul_rn(hi, x);
+struct Sum<float> : Sum3 {
+    __device__ __forceinline__ void add_sum(const Sum& x) { add(x.s, x.e, x.f); }
+    __device__ __forceinline__ bool past_range() const { return large(s); }
+    // the product of x with c0 + c1 + c2 (a float64 number cut in three)
+    __device__ __forceinline__ void add_product(float c0, float c1, float c2, float x) {
+        const float p = __fmul_rn(c0, x), q = __fmul_rn(c1, x);
         add(p);
-        e = __fadd_rn(e, __fmaf_rn(lo, x, __fmaf_rn(hi, x, -p)));
+        add_low(__fmaf_rn(c0, x, -p));
+        add_low(q);
+        f = __fadd_rn(f, __fmaf_rn(c2, x, __fmaf_rn(c1, x, -q)));
+    }
+    __device__ __forceinline__ void add_from(const Sum& mine, int m) {
+        const float ts = __shfl_xor_sync(0xffffffffu, mine.s, m);
+        const float te = __shfl_xor_sync(0xffffffffu, mine.e, m);
+        const float tf = __shfl_xor_sync(0xffffffffu, mine.f, m);
+        add(ts, te, tf);
     }
     __device__ __forceinline__ void add_lane(int m) {
-        const float t = __shfl_xor_sync(0xffffffffu, s, m);
-        const float u = __shfl_xor_sync(0xffffffffu, e, m);
-        // the same order on both sides of the exchange: the lower lane's pair first
+        const float ts = __shfl_xor_sync(0xffffffffu, s, m);
+        const float te = __shfl_xor_sync(0xffffffffu, e, m);
+        const float tf = __shfl_xor_sync(0xffffffffu, f, m);
+        // the same order on both sides of the exchange: the lower lane's sum first
         const bool up = (threadIdx.x & m) != 0;
-        const float a = up ? t : s, b = up ? s : t, ea = up ? u : e, eb = up ? e : u;
-        s = a;
-        e = ea;
-        add(b);
-        e = __fadd_rn(e, eb);
-    }
-    // s alone once a term was infinite or NaN (e is then inf - inf): an infinite cost stays
-    // infinite
-    __device__ __forceinline__ double value() const {
-        return isfinite(s) ? (double)s + (double)e : (double)s;
+        const float bs = up ? s : ts, be = up ? e : te, bf = up ? f : tf;
+        s = up ? ts : s;
+        e = up ? te : e;
+        f = up ? tf : f;
+        add(bs, be, bf);
     }
 };
-// the sum over groups of LPN lanes
+// the sums of x and y over groups of LPN lanes: x's in the lower half of the group, y's in the
+// upper half (each half hands the other its own values first)
 template <int LPN, typename Tp>
-__device__ __forceinline__ Sum<Tp> group_add(Sum<Tp> x) {
+__device__ __forceinline__ Sum<Tp> group_add2(const Sum<Tp>& x, const Sum<Tp>& y) {
+    const bool up = (threadIdx.x & (LPN / 2)) != 0;
+    Sum<Tp> t = up ? y : x;
+    t.add_from(up ? x : y, LPN / 2);
 #pragma unroll
-    for (int m = LPN / 2; m > 0; m >>= 1) x.add_lane(m);
+    for (int m = LPN / 4; m > 0; m >>= 1) t.add_lane(m);
+    return t;
+}
+__device__ __forceinline__ double warp_sum(double x) {
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) x += __shfl_xor_sync(0xffffffffu, x, m);
     return x;
 }
 template <int LPN, typename Tp>
@@ -124,30 +141,69 @@ __device__ __forceinline__ Tp group_sum(Tp x) {
     return x;
 }
 
-// The two cost sums of a segment, 16 bytes: as value and rounding error in float32 (the
-// conversion to float64 would cost six float64 instructions per warp and segment, a quarter
-// of pass 2; the selection converts 32 columns at once).
-__device__ __forceinline__ void store_costs(double* dseg, int64_t g, const Sum<float>& m,
-                                            const Sum<float>& d) {
-    reinterpret_cast<float4*>(dseg)[g] = make_float4(m.s, m.e, d.s, d.e);
+// The two cost sums of a segment, added over the warp's lanes and stored.  float32: two words of
+// 16 bytes, each s, e, f and 0, or a float64 number, 0 and 1 where a lane's sum is near the end
+// of float32's range (converting every segment's sums to float64 would cost ten float64
+// instructions per warp and segment, a quarter of pass 2; the selection converts 32 columns
+// at once).  float64: one word of 16 bytes.
+__device__ __forceinline__ void store_costs(double* dseg, int64_t g, float m, float d) {
+    const int lane = threadIdx.x & 31;
+    float4* out = reinterpret_cast<float4*>(dseg) + 2 * g;
+    if (__any_sync(0xffffffffu, Sum3::large(m) || Sum3::large(d))) {
+        const double wm = warp_sum((double)m), wd = warp_sum((double)d);
+        if (lane < 2) {
+            const double t = lane ? wd : wm;
+            out[lane] = make_float4(__int_as_float(__double2loint(t)),
+                                    __int_as_float(__double2hiint(t)), 0.f, 1.f);
+        }
+        return;
+    }
+    // the lower half warp adds m, the upper half d
+    const bool up = lane >= 16;
+    Sum<float> x;
+    x.add(up ? d : m);
+    x.add(__shfl_xor_sync(0xffffffffu, up ? m : d, 16));
+#pragma unroll
+    for (int k = 8; k > 0; k >>= 1) x.add_lane(k);
+    if (lane % 16 == 0) out[lane / 16] = make_float4(x.s, x.e, x.f, 0.f);
 }
-__device__ __forceinline__ void store_costs(double* dseg, int64_t g, const Sum<double>& m,
-                                            const Sum<double>& d) {
-    reinterpret_cast<double2*>(dseg)[g] = make_double2(m.s, d.s);
+__device__ __forceinline__ void store_costs(double* dseg, int64_t g, double m, double d) {
+    m = warp_sum(m);
+    d = warp_sum(d);
+    if (threadIdx.x % 32 == 0) reinterpret_cast<double2*>(dseg)[g] = make_double2(m, d);
 }
-__device__ __forceinline__ void add_costs(const double* dseg, int64_t g, Sum<float>& m,
-                                          Sum<float>& d) {
-    const float4 t = reinterpret_cast<const float4*>(dseg)[g];
-    m.add(t.x);
-    m.e = __fadd_rn(m.e, t.y);
-    d.add(t.z);
-    d.e = __fadd_rn(d.e, t.w);
+__device__ __forceinline__ double word_value(const float4& t) {
+    if (t.w != 0.f) return __hiloint2double(__float_as_int(t.y), __float_as_int(t.x));
+    Sum3 x;
+    x.s = t.x;
+    x.e = t.y;
+    x.f = t.z;
+    return x.value();
 }
-__device__ __forceinline__ void add_costs(const double* dseg, int64_t g, Sum<double>& m,
-                                          Sum<double>& d) {
-    const double2 t = reinterpret_cast<const double2*>(dseg)[g];
-    m.add(t.x);
-    d.add(t.y);
+// += the costs of the segments g0, g0 + step, ... < g1; whether a float64 number was among them
+// (the sums are then of no use)
+__device__ __forceinline__ bool add_costs(const double* dseg, int64_t g0, int64_t g1, int step,
+                                          Sum<float>& m, Sum<float>& d) {
+    const float4* w = reinterpret_cast<const float4*>(dseg);
+    bool wide = false;
+#pragma unroll 8
+    for (int64_t g = g0; g < g1; g += step) {
+        const float4 tm = w[2 * g], td = w[2 * g + 1];
+        wide |= tm.w != 0.f || td.w != 0.f;
+        m.add(tm.x, tm.y, tm.z);
+        d.add(td.x, td.y, td.z);
+    }
+    return wide;
+}
+__device__ __forceinline__ bool add_costs(const double* dseg, int64_t g0, int64_t g1, int step,
+                                          Sum<double>& m, Sum<double>& d) {
+#pragma unroll 8
+    for (int64_t g = g0; g < g1; g += step) {
+        const double2 t = reinterpret_cast<const double2*>(dseg)[g];
+        m.add(t.x);
+        d.add(t.y);
+    }
+    return false;
 }
 
 // The non-zeros of a segment are read 32 at a time with one coalesced load (lane l holds
@@ -304,16 +360,27 @@ __global__ void __launch_bounds__(WARPS * 32)
 
 // The candidates of view column o, a group of LPN lanes per column: A and B as the sums of
 // the column's segments in order, then eq. 11 (Xm), eq. 15 / 17 and the eq. 10
-// renormalisation (Xd), rows [O][R4] with zeros past R.  MU: Xm only.
+// renormalisation (Xd), rows [O][R4] with zeros past R.  MU: Xm only.  c3 [3][4 LPN] receives the
+// column sums c0 of Y, each as a sum of up to three values of the element type.
 template <typename Tp, int LPN, bool MU>
 __global__ void __launch_bounds__(WARPS * 32)
     k_sp_cand(int64_t O, int64_t R, int64_t R4, const int64_t* __restrict__ sptr,
               const Tp* __restrict__ Aseg, const Tp* __restrict__ Bseg,
               const Tp* __restrict__ Xr, const double* __restrict__ c,
               const double* __restrict__ vsum, Tp* __restrict__ Xm, Tp* __restrict__ Xd, Tp eps,
-              Tp alpha) {
+              Tp alpha, const double* __restrict__ c0, Tp* __restrict__ c3) {
     pdl_wait();
     pdl_next();
+    if (!MU && blockIdx.x == 0)   // c0 as sums of three values, for the selection
+        for (int k = threadIdx.x; k < 4 * LPN; k += WARPS * 32) {
+            double t = k < R ? c0[k] : 0.0;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const Tp part = (Tp)t;
+                c3[i * 4 * LPN + k] = part;
+                t -= (double)part;
+            }
+        }
     __shared__ Tp cs[4 * LPN], ics[4 * LPN];
     for (int k = threadIdx.x; k < 4 * LPN; k += WARPS * 32) {
         cs[k] = k < R ? (Tp)c[k] : Tp(1);
@@ -376,8 +443,8 @@ __global__ void __launch_bounds__(WARPS * 32)
 
 // Pass 2 (steps 7-9, 12-14 on the non-zeros of one segment): the partial sums
 // sum_{v>0} -v log z_MU and sum_{v>0} -v log z_DNA as the pair g of dseg.  A lane adds
-// the terms of its non-zeros in the element type (at most SEG / U of them), the lanes' sums
-// are added with their rounding errors.
+// the terms of its non-zeros in the element type (at most SEG / U of them); the lanes' sums are
+// added by store_costs.
 template <typename Tp, int LPN>
 __global__ void __launch_bounds__(WARPS * 32)
     k_sp_pass2(int64_t R4, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
@@ -425,12 +492,7 @@ __global__ void __launch_bounds__(WARPS * 32)
             }
         }
     });
-    Sum<Tp> lm, ld;
-    lm.add(lm_t);
-    ld.add(ld_t);
-    lm = group_add<32>(lm);
-    ld = group_add<32>(ld);
-    if (lane == 0) store_costs(dseg, g, lm, ld);
+    store_costs(dseg, g, lm_t, ld_t);
 }
 
 // The cost of each candidate (the segments' sums in order, sum_s z = sum_r c0_r x(r, o), and
@@ -441,15 +503,16 @@ template <typename Tp, int LPN, bool MU>
 __global__ void __launch_bounds__(WARPS * 32)
     k_sp_select(View v, int64_t R4, const int64_t* __restrict__ sptr,
                 const double* __restrict__ dseg, const Tp* __restrict__ Xm,
-                const Tp* __restrict__ Xd, const double* __restrict__ c0,
+                const Tp* __restrict__ Xd, const Tp* __restrict__ c3,
                 uint8_t* __restrict__ choice, double* __restrict__ dfin,
                 double* __restrict__ fpart, double reg, int* __restrict__ status) {
     pdl_wait();
     pdl_next();
     constexpr int G = 32 / LPN, NK = 4 / G;   // columns of a warp at once, rounds
     __shared__ Tp xs[4 * LPN][33];
-    __shared__ Tp ch[4 * LPN], cl[4 * LPN];   // c0 = ch + cl
+    __shared__ Tp cc[3][4 * LPN];             // c0 as a sum of up to three values
     __shared__ Sum<Tp> sums[4][32];           // per column: sum z and sum x of both candidates
+    __shared__ Sum<Tp> parts[WARPS][2][32];   // per column: shares of the segments' costs
     __shared__ int kept[32];
     const int64_t R = v.R, O = v.O, o0 = (int64_t)blockIdx.x * 32;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, sub = lane % LPN, r = 4 * sub;
@@ -463,50 +526,67 @@ __global__ void __launch_bounds__(WARPS * 32)
         if (!MU) xd[k] = in ? load4(Xd + o * R4 + r) : zero;
     }
     if (!MU) {
-        for (int k = tid; k < 4 * LPN; k += WARPS * 32) {
-            const double t = k < R ? c0[k] : 0.0;
-            ch[k] = (Tp)t;
-            cl[k] = (Tp)(t - (double)ch[k]);
-        }
+        for (int k = tid; k < 3 * 4 * LPN; k += WARPS * 32) cc[k / (4 * LPN)][k % (4 * LPN)] = c3[k];
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < NK; ++k) {
             Sum<Tp> zm, zd, pm, pd;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                zm.add_product(ch[r + i], cl[r + i], x[k].v[i]);
-                zd.add_product(ch[r + i], cl[r + i], xd[k].v[i]);
+                zm.add_product(cc[0][r + i], cc[1][r + i], cc[2][r + i], x[k].v[i]);
+                zd.add_product(cc[0][r + i], cc[1][r + i], cc[2][r + i], xd[k].v[i]);
             }
-            zm = group_add<LPN>(zm);
-            zd = group_add<LPN>(zd);
+            zm = group_add2<LPN>(zm, zd);   // in the upper half of the group zd's sum
             if (reg != 0.0) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     pm.add(x[k].v[i]);
                     pd.add(xd[k].v[i]);
                 }
-                pm = group_add<LPN>(pm);
-                pd = group_add<LPN>(pd);
+                pm = group_add2<LPN>(pm, pd);
             }
-            if (sub == 0) {
-                const int col = 4 * w + k * G + lane / LPN;
-                sums[0][col] = zm;
-                sums[1][col] = zd;
-                sums[2][col] = pm;
-                sums[3][col] = pd;
+            if (sub % (LPN / 2) == 0) {
+                const int col = 4 * w + k * G + lane / LPN, which = sub != 0;
+                sums[which][col] = zm;
+                sums[2 + which][col] = pm;
             }
         }
-        __syncthreads();
-        if (w == 0) {   // lane = column: float64 for 32 columns at once
-            const int64_t o = o0 + lane;
+        // lane = column: the segments' costs in order, or, where a column of the CTA has many of
+        // them, warp w those at w, w + 8, ... and the eight sums in order
+        const int64_t o = o0 + lane, g0 = o < O ? sptr[o] : 0, g1 = o < O ? sptr[o + 1] : 0;
+        const bool many = __syncthreads_or(g1 - g0 > WARPS);
+        Sum<Tp> lm, ld;
+        bool wide = false;
+        if (many || w == 0)
+            wide = add_costs(dseg, g0 + (many ? w : 0), g1, many ? WARPS : 1, lm, ld);
+        if (many) {
+            parts[w][0][lane] = lm;
+            parts[w][1][lane] = ld;
+            wide = __syncthreads_or(wide);
+            if (w == 0)
+#pragma unroll
+                for (int k = 1; k < WARPS; ++k) {
+                    lm.add_sum(parts[k][0][lane]);
+                    ld.add_sum(parts[k][1][lane]);
+                }
+        }
+        if (w == 0) {   // float64 for 32 columns at once
             bool newton = false;
             if (o < O) {
-                Sum<Tp> lm, ld;
-                const int64_t g1 = sptr[o + 1];
-#pragma unroll 16
-                for (int64_t g = sptr[o]; g < g1; ++g) add_costs(dseg, g, lm, ld);
-                double dm = lm.value() + sums[0][lane].value();
-                double dd = ld.value() + sums[1][lane].value();
+                const Sum<Tp> zm = sums[0][lane], zd = sums[1][lane];
+                lm.add_sum(zm);
+                ld.add_sum(zd);
+                double dm = lm.value(), dd = ld.value();
+                if constexpr (sizeof(Tp) == 4)
+                    if (wide || lm.past_range() || ld.past_range()) {
+                        dm = dd = 0.0;
+                        for (int64_t g = g0; g < g1; ++g) {
+                            dm += word_value(reinterpret_cast<const float4*>(dseg)[2 * g]);
+                            dd += word_value(reinterpret_cast<const float4*>(dseg)[2 * g + 1]);
+                        }
+                        dm += zm.value();
+                        dd += zd.value();
+                    }
                 if (reg != 0.0) {
                     dm += reg * sums[2][lane].value();
                     dd += reg * sums[3][lane].value();
@@ -552,7 +632,7 @@ __global__ void __launch_bounds__(WARPS * 32)
 }
 
 // d_KL (eq. 1) of the H view, per segment: sum over its non-zeros of v log(v / z) - v into
-// dseg[g] (float64).
+// dseg[g]: a lane's terms (at most SEG / U of them) in the element type, the lanes in float64.
 template <typename Tp, int LPN>
 __global__ void __launch_bounds__(WARPS * 32)
     k_sp_kl(int64_t R4, Segs sg, const int32_t* __restrict__ idx, const Tp* __restrict__ val,
@@ -573,9 +653,7 @@ __global__ void __launch_bounds__(WARPS * 32)
         const Tp vl = __shfl_sync(0xffffffffu, c.v, first + sub / STEP);
         if (sub % STEP == 0 && vl > Tp(0)) acc_t += vl * log(vl / z) - vl;
     });
-    Sum<Tp> acc;
-    acc.add(acc_t);
-    const double t = group_add<32>(acc).value();
+    const double t = warp_sum((double)acc_t);
     if (lane == 0) dseg[g] = t;
 }
 

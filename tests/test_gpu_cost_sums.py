@@ -1,6 +1,7 @@
-"""The sums behind the selection and d_KL in the float32 forms: an infinite term (z = 0 where
-v > 0) leaves +infinity, as float64 sums would, not a value that no comparison holds for; the
-call reports DNA_ERR_NONFINITE all the same."""
+"""The sums behind the selection and d_KL in the float32 forms, against what float64 sums give.
+An infinite term (z = 0 where v > 0) leaves +infinity, not a value that no comparison holds
+for; the call reports DNA_ERR_NONFINITE all the same.  Terms that are exact in float32 and
+whose sum is exact in float64 are added exactly, and sums past float32's range stay finite."""
 import ctypes
 
 import numpy as np
@@ -105,3 +106,75 @@ def test_infinite_kl(form, R):
     W[5] = 0.0
     with Bound(form, V, W, H) as b:
         assert b.kl() == (b.L.DNA_ERR_NONFINITE, np.inf)
+
+
+# 1 + 2^-27 + 2^-52: exact in float64, and neither in float32 nor in a pair of float32 values
+PARTS = (1.0, 2.0 ** -27, 2.0 ** -52)
+# columns of the dense problems: two o-blocks of 64 per SM, so that one CTA runs over all rows
+COLS = 2 * 64 * 152
+
+
+def _spread(rows, values, N, T):
+    """V = 0 (N x T), W (N x 1) with `values` in `rows`, H (1 x T) with 1 in column 0."""
+    W = np.zeros((N, 1))
+    W[list(rows), 0] = values
+    H = np.zeros((1, T))
+    H[0, 0] = 1.0
+    return np.zeros((N, T), dtype=np.float32), W, H
+
+
+@pytest.mark.parametrize("form,rows,N", [("f32", (0, 64, 128), 192), ("bf16", (0, 64, 128), 192),
+                                         ("group_f32", (0, 64, 128), 192),
+                                         ("group_bf16", (0, 64, 128), 192),
+                                         ("f32", (0, 64 * 300, 64 * 301), 64 * 310)])
+def test_kl_exact(form, rows, N):
+    """d_KL of V = 0 is the sum of z: the rows' values, each in another chunk of one thread."""
+    V, W, H = _spread(rows, PARTS, N, 1 if form.startswith("group") else COLS)
+    with Bound(form, V, W, H) as b:
+        assert b.kl() == (b.L.DNA_OK, sum(PARTS))
+
+
+def test_kl_exact_sparse():
+    """v = z at three non-zeros: each term v log(v / z) - v is -v, and their sum and that of z
+    cancel exactly (rows of different 32-row blocks, so that the sum of z is exact too)."""
+    W = np.zeros((70, 1))
+    W[[0, 32, 64], 0] = PARTS
+    with Bound("sparse", W, W, np.ones((1, 1))) as b:
+        assert b.kl() == (b.L.DNA_OK, 0.0)
+
+
+@pytest.mark.parametrize("form,rows,N", [("f32", (0, 64, 128), 192), ("sparse", (0, 32, 64), 70)])
+def test_costs_exact(form, rows, N):
+    """v = z = 1 at one entry (a = 0, so both candidates are the starting x = 1, and log z = 0)
+    and v = 0 elsewhere: both costs are the sum of z."""
+    V, W, H = _spread(rows, PARTS, N, COLS if form == "f32" else 1)
+    V[0, 0] = 1.0
+    with Bound(form, V, W, H) as b:
+        b.step(0)
+        code, dm, dd = b.costs(0)
+        assert code == b.L.DNA_OK and dm[0] == sum(PARTS) and dd[0] == sum(PARTS)
+
+
+@pytest.mark.parametrize("form,N", [("f32", 256), ("sparse", 256)])
+def test_costs_past_float32_range(form, N):
+    """v = z = 2e36 in four rows: -v log z is -1.7e38 in each, -6.7e38 in all.  Both candidates
+    are the starting column up to rounding: 1e-5 of the sum (float32 terms, |z' / z - 1| and
+    |log z' - log z| / 84 a few float32 roundings)."""
+    rows, v = (0, 64, 128, 192), float(np.float32(2e36))
+    V, W, H = _spread(rows, 1.0, N, COLS if form == "f32" else 1)
+    V[list(rows), 0] = v
+    H[0, 0] = v
+    ref = 4.0 * (v - v * np.log(v))
+    with Bound(form, V, W, H) as b:
+        b.step(0)
+        code, dm, dd = b.costs(0)
+        assert code == b.L.DNA_OK
+        assert abs(dm[0] - ref) <= 1e-5 * abs(ref) and abs(dd[0] - ref) <= 1e-5 * abs(ref)
+
+
+def test_kl_past_float32_range():
+    """V = 0, z = 2e38 in two rows of different chunks: their sum."""
+    z = np.float32(2e38)
+    for form, T in (("f32", COLS), ("group_f32", 1)):
+        with Bound(form, *_spread((0, 64), z, 128, T)) as b:
+            assert b.kl() == (b.L.DNA_OK, 2.0 * float(z))
