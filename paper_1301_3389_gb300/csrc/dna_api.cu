@@ -45,13 +45,14 @@ struct dna_ctx {
     void* Xmu = nullptr;         // [R][O]
     void* Xdna = nullptr;
     double* dpart = nullptr;     // [splits][2][O]
-    double* dfin_h = nullptr;    // [2][T]
-    double* dfin_w = nullptr;    // [2][N]
-    uint8_t* choice_h = nullptr; // T
-    uint8_t* choice_w = nullptr; // N
     double* kl_dev = nullptr;    // 1
     double* kl_part = nullptr;   // REDUCE_PARTS partial sums of d_KL
+    void* state = nullptr;       // one block, zero at creation:
+    double* dfin_h = nullptr;    // [2][T]
+    double* dfin_w = nullptr;    // [2][N]
     int* status = nullptr;       // 1
+    uint8_t* choice_h = nullptr; // T
+    uint8_t* choice_w = nullptr; // N
     // split plans (pass 1 and pass 2 / KL) for the H view and the W view
     int sp1[2] = {1, 1}, sp2[2] = {1, 1};
     int64_t per1[2] = {0, 0}, per2[2] = {0, 0};
@@ -166,6 +167,31 @@ int dmalloc(P** p, size_t bytes) {
         return DNA_ERR_ALLOC;
     }
     return DNA_OK;
+}
+
+// What a caller may read of a context before its first step, in one block: the costs, the status
+// word and the selections.  Zeroed on a stream of its own and waited for: a clear on the default
+// stream would run behind whatever is queued there, perhaps after the context's first kernels
+// (it would then wipe a reported error or the selections).
+int alloc_state(dna_ctx* c) {
+    const size_t dh = sizeof(double) * 2 * (size_t)c->T, dw = sizeof(double) * 2 * (size_t)c->N;
+    const size_t bytes = dh + dw + 8 + (size_t)c->T + (size_t)c->N;
+    if (dmalloc(&c->state, bytes)) return DNA_ERR_ALLOC;
+    unsigned char* p = static_cast<unsigned char*>(c->state);
+    c->dfin_h = reinterpret_cast<double*>(p);
+    c->dfin_w = reinterpret_cast<double*>(p + dh);
+    c->status = reinterpret_cast<int*>(p + dh + dw);
+    c->choice_h = p + dh + dw + 8;
+    c->choice_w = c->choice_h + c->T;
+    cudaStream_t st = nullptr;
+    bool ok = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess;
+    if (ok) {
+        ok = cudaMemsetAsync(c->state, 0, bytes, st) == cudaSuccess;
+        ok = cudaStreamSynchronize(st) == cudaSuccess && ok;
+        ok = cudaStreamDestroy(st) == cudaSuccess && ok;
+    }
+    if (!ok) cudaGetLastError();
+    return ok ? DNA_OK : DNA_ERR_CUDA;
 }
 
 View make_view(const dna_ctx* c, bool wstep) {
@@ -359,8 +385,7 @@ void free_all(dna_ctx* c) {
     void* ptrs[] = {c->own_V, c->own_W, c->own_H, c->Vt, c->colsum_v, c->rowsum_v, c->c, c->sig,
                     c->fwork, c->gpart, c->vpart, c->Apart, c->Bpart, c->Xmu, c->Xdna,
                     c->Bpart ? nullptr : c->dpart,   // behind Bpart in the dense forms
-                    c->dfin_h, c->dfin_w,
-                    c->choice_h, c->choice_w, c->kl_dev, c->kl_part, c->status, c->Xk, c->Yk, c->Ytk,
+                    c->state, c->kl_dev, c->kl_part, c->Xk, c->Yk, c->Ytk,
                     c->Y2tk, c->Xmk, c->Xdk, c->Vp, c->Qg, c->Qbg, c->cptr, c->ridx, c->cval, c->Hr, c->Wr, c->c0, c->c3,
                     c->seg_col[0], c->seg_col[1], c->seg_k0[0], c->seg_k0[1], c->seg_k1[0],
                     c->seg_k1[1], c->seg_ptr[0], c->seg_ptr[1], c->Aseg, c->Bseg, c->dseg,
@@ -405,13 +430,8 @@ int alloc_workspace(dna_ctx* c) {
     if (c->Bpart) c->dpart = reinterpret_cast<double*>(static_cast<char*>(c->Bpart) + bp);
     e |= dmalloc(&c->Xmu, sizeof(Tp) * (size_t)(R * M));
     e |= dmalloc(&c->Xdna, sizeof(Tp) * (size_t)(R * M));
-    e |= dmalloc(&c->dfin_h, sizeof(double) * 2 * T);
-    e |= dmalloc(&c->dfin_w, sizeof(double) * 2 * N);
-    e |= dmalloc(&c->choice_h, (size_t)T);
-    e |= dmalloc(&c->choice_w, (size_t)N);
     e |= dmalloc(&c->kl_dev, sizeof(double));
     e |= dmalloc(&c->kl_part, sizeof(double) * (size_t)dna::REDUCE_PARTS);
-    e |= dmalloc(&c->status, sizeof(int));
     if (c->tc) {
         const int64_t mo = std::max(c->pad_o[0], c->pad_o[1]);
         const int64_t ms = std::max(c->pad_s[0], c->pad_s[1]);
@@ -439,12 +459,7 @@ int alloc_workspace(dna_ctx* c) {
         }
     }
     if (e != DNA_OK) return DNA_ERR_ALLOC;
-    if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess) return DNA_ERR_CUDA;
-    if (cudaMemset(c->choice_h, 0, (size_t)T) != cudaSuccess) return DNA_ERR_CUDA;
-    if (cudaMemset(c->choice_w, 0, (size_t)N) != cudaSuccess) return DNA_ERR_CUDA;
-    if (cudaMemset(c->dfin_h, 0, sizeof(double) * 2 * T) != cudaSuccess) return DNA_ERR_CUDA;
-    if (cudaMemset(c->dfin_w, 0, sizeof(double) * 2 * N) != cudaSuccess) return DNA_ERR_CUDA;
-    return DNA_OK;
+    return alloc_state(c);
 }
 
 // Workspace of the sparse-V form: no transposed copy of V (the CSC copy has nnz entries)
@@ -465,26 +480,15 @@ int alloc_sparse_workspace(dna_ctx* c) {
     e |= dmalloc(&c->Xmu, sizeof(Tp) * (size_t)(R4 * M));
     e |= dmalloc(&c->Xdna, sizeof(Tp) * (size_t)(R4 * M));
     e |= dmalloc(&c->dpart, sizeof(double) * (size_t)(2 * M));
-    e |= dmalloc(&c->dfin_h, sizeof(double) * 2 * T);
-    e |= dmalloc(&c->dfin_w, sizeof(double) * 2 * N);
-    e |= dmalloc(&c->choice_h, (size_t)T);
-    e |= dmalloc(&c->choice_w, (size_t)N);
     e |= dmalloc(&c->kl_dev, sizeof(double));
     e |= dmalloc(&c->kl_part, sizeof(double) * (size_t)dna::REDUCE_PARTS);
-    e |= dmalloc(&c->status, sizeof(int));
     e |= dmalloc(&c->cptr, sizeof(int64_t) * (size_t)(T + 1));
     e |= dmalloc(&c->ridx, sizeof(int32_t) * (size_t)std::max<int64_t>(c->nnz, 1));
     e |= dmalloc(&c->cval, sizeof(Tp) * (size_t)std::max<int64_t>(c->nnz, 1));
     e |= dmalloc(&c->Hr, sizeof(Tp) * (size_t)(T * R4));
     e |= dmalloc(&c->Wr, sizeof(Tp) * (size_t)(N * R4));
     if (e != DNA_OK) return DNA_ERR_ALLOC;
-    if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(c->choice_h, 0, (size_t)T) != cudaSuccess ||
-        cudaMemset(c->choice_w, 0, (size_t)N) != cudaSuccess ||
-        cudaMemset(c->dfin_h, 0, sizeof(double) * 2 * T) != cudaSuccess ||
-        cudaMemset(c->dfin_w, 0, sizeof(double) * 2 * N) != cudaSuccess)
-        return DNA_ERR_CUDA;
-    return DNA_OK;
+    return alloc_state(c);
 }
 
 // The CSC copy of V and the row and column sums of V (eq. 10 targets), built on the host
