@@ -650,16 +650,22 @@ void free_lists(dna_group* g) {
     g->tile_allocs.clear();
 }
 
+// A host table into device memory on the group's stream: behind the kernels that still read
+// what it replaces, before those that are queued next (a copy on the default stream is ordered
+// with neither).  The call returns when the host memory has been read.
+int copy_in(dna_group* g, void* dst, const void* src, size_t bytes) {
+    return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, g->gs) == cudaSuccess
+               ? DNA_OK
+               : DNA_ERR_CUDA;
+}
+
 int upload(dna_group* g, const std::vector<GTile>& v, TileList* out) {
     out->n = (int)v.size();
     out->d = nullptr;
     if (v.empty()) return DNA_OK;
     if (cudaMalloc(&out->d, sizeof(GTile) * v.size()) != cudaSuccess) return DNA_ERR_ALLOC;
     g->tile_allocs.push_back(out->d);
-    if (cudaMemcpy(out->d, v.data(), sizeof(GTile) * v.size(), cudaMemcpyHostToDevice) !=
-        cudaSuccess)
-        return DNA_ERR_CUDA;
-    return DNA_OK;
+    return copy_in(g, out->d, v.data(), sizeof(GTile) * v.size());
 }
 
 // Split plan of every problem for rows-per-split `rows`, then all tile lists.
@@ -784,9 +790,7 @@ int build_tiles(dna_group* g) {
             e |= upload(g, tq1[w], &g->tp1[w]);
             e |= upload(g, tq2[w], &g->tp2[w]);
         }
-        if (!e && cudaMemcpy(g->gv, g->hgv.data(), sizeof(dna::TcGView) * g->hgv.size(),
-                             cudaMemcpyHostToDevice) != cudaSuccess)
-            e = DNA_ERR_CUDA;
+        if (!e) e = copy_in(g, g->gv, g->hgv.data(), sizeof(dna::TcGView) * g->hgv.size());
     }
     for (int w = 0; w < 2; ++w) {
         e |= upload(g, t1[w], &g->p1[w]);
@@ -798,9 +802,7 @@ int build_tiles(dna_group* g) {
     }
     e |= upload(g, tk, &g->kl);
     if (e) return e;
-    if (cudaMemcpy(g->dp, g->hp.data(), sizeof(GProb) * g->count, cudaMemcpyHostToDevice) !=
-        cudaSuccess)
-        return DNA_ERR_CUDA;
+    if ((e = copy_in(g, g->dp, g->hp.data(), sizeof(GProb) * g->count))) return e;
     if (g->gexec) {
         cudaGraphExecDestroy(g->gexec);
         g->gexec = nullptr;
@@ -1047,7 +1049,9 @@ int dna_group_create(int count, const int64_t* N, const int64_t* T, const int64_
         e = DNA_ERR_ALLOC;
     if (!e && tc && cudaMalloc(&g->gv, sizeof(dna::TcGView) * 2 * (size_t)count) != cudaSuccess)
         e = DNA_ERR_ALLOC;
-    if (!e && cudaMemset(g->status, 0, sizeof(int)) != cudaSuccess) e = DNA_ERR_CUDA;
+    // on the group's stream, like everything it runs: a clear on the default stream could land
+    // behind the work queued there, over a status that a kernel has set
+    if (!e && cudaMemsetAsync(g->status, 0, sizeof(int), g->gs) != cudaSuccess) e = DNA_ERR_CUDA;
     if (e) {
         cudaGetLastError();
         dna_group_destroy(g);

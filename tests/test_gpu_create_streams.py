@@ -63,3 +63,48 @@ def test_create_beside_a_busy_default_stream(form, fault):
     for got in _run(form, fault, True):
         for a, b in zip(ref[0], got):
             assert np.array_equal(a, b, equal_nan=True)
+
+
+def _run_group(bf16, fault, busy):
+    import torch
+
+    import paper_1301_3389_gb300 as dna
+    probs = [workloads.custom(n, t, r, seed=n) for n, t, r in ((130, 201, 16), (65, 700, 40))]
+    if fault:
+        probs[1].W[7] = 0.0
+    V, W, H = ([torch.from_numpy(np.ascontiguousarray(getattr(p, k))).to("cuda", torch.float32)
+                for p in probs] for k in "VWH")
+    sizes = [[x.shape[d] for x in m] for m, d in ((V, 0), (V, 1), (W, 1))]
+    side = torch.cuda.Stream()
+
+    def state():
+        out = []
+        for q in range(2):
+            choice = np.zeros(sizes[1][q], np.uint8)
+            out += [dna.LIB.dna_group_get_choice(g, q, 0, choice.ctypes.data, len(choice)), choice]
+        return out
+
+    torch.cuda.synchronize()
+    if busy:
+        torch.cuda._sleep(1_000_000_000)
+    g = dna.dna_group_create(*sizes, dna.make_opts(dtype=dna.DNA_BF16 if bf16 else dna.DNA_F32))
+    dna.dna_group_set_stream(g, side)
+    dna.dna_group_bind(g, V, W, H)
+    dna.dna_group_step_H(g)
+    first = state()
+    assert torch.cuda.default_stream().query() != busy
+    torch.cuda.synchronize()
+    second = state()
+    dna.dna_group_destroy(g)
+    return first, second
+
+
+@pytest.mark.parametrize("fault", [False, True])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_group_beside_a_busy_default_stream(bf16, fault):
+    """As above for a group; its tables reach the device in the group's own order too."""
+    import paper_1301_3389_gb300 as dna
+    ref = _run_group(bf16, fault, False)[0]
+    assert ref[0] == (dna.DNA_ERR_NONFINITE if fault else dna.DNA_OK) and ref[1].any()
+    for got in _run_group(bf16, fault, True):
+        assert all(np.array_equal(a, b) for a, b in zip(ref, got))
