@@ -17,8 +17,8 @@ everything from them), so repeated calls allocate nothing; a call that fails des
 context.  ``release_contexts()`` frees the calling thread's contexts.
 
 Work is queued on the current stream and not waited for (``KLDiv``'s forward waits for its
-number): a kept context carries an event after its last call, which a call on another
-stream waits for, and every tensor that the queued kernels use is recorded on their stream.
+number): a kept context carries an event after its last call, which the next call's stream
+waits for, and every tensor that the queued kernels use is recorded on their stream.
 Waiting at the end of each call left the GPU idle while Python prepared the next one
 (N=1024 T=4096 R=64: d_KL forward and backward 590 us -> 442, two unrolled steps forward
 and backward 1300 -> 925).
@@ -44,7 +44,7 @@ def _pool() -> dict:
 def release_contexts() -> None:
     """Destroy the library contexts this thread keeps for the autograd wrappers."""
     pool = _pool()
-    for ctx, _, _ in pool.values():
+    for ctx, _ in pool.values():
         L.dna_destroy(ctx)
     pool.clear()
 
@@ -63,14 +63,17 @@ class _Ctx:
             raise RuntimeError("the autograd wrappers cannot be captured in a CUDA graph")
         stream = self.stream = torch.cuda.current_stream()
         # taken out while in use (re-entrant calls get their own)
-        ctx, last, self.event = _pool().pop(self.key, (None, None, None))
-        if ctx is None:
+        ctx, self.event = _pool().pop(self.key, (None, None))
+        kept = ctx is not None
+        if not kept:
             ctx = L.dna_create(N, T, R, L.make_opts(dtype=dtype))
             self.event = torch.cuda.Event()
         self.ctx = ctx
         try:
-            if last is not None and last != stream:
-                stream.wait_event(self.event)   # the context's workspace is still in use there
+            if kept:
+                # the last call may still use the context's workspace, on whatever stream it
+                # ran (an equal handle may be a new stream that took a destroyed one's place)
+                stream.wait_event(self.event)
             for t in (V, W, H, *others):
                 t.record_stream(stream)
             L.dna_set_stream(ctx, stream)
@@ -86,7 +89,7 @@ class _Ctx:
         pool = _pool()
         if exc_type is None and self.key not in pool:
             self.event.record(self.stream)
-            pool[self.key] = (self.ctx, self.stream, self.event)
+            pool[self.key] = (self.ctx, self.event)
         else:
             L.dna_destroy(self.ctx)
         return False
