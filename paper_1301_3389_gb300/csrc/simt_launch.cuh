@@ -36,16 +36,20 @@ int pass1_rb(const View& v, Tp* A, Tp* B, int splits, int64_t s_per, bool with_b
              cudaStream_t st, double* dcur) {
     const size_t smem = Pass1Cfg<Tp, RB>::smem;
     dim3 grid((unsigned)((v.O + OB - 1) / OB), (unsigned)((v.R + RB - 1) / RB), (unsigned)splits);
-    if (with_b) {
-        auto k = k_pass1<Tp, RB, true>;
+    auto launch = [&](auto k) {
         if (prep_smem(k, smem)) return DNA_ERR_CUDA;
-        dna::launch_pdl(k, grid, dim3(NT), smem, st, v, A, B, s_per, status, dcur);
-    } else {
-        auto k = k_pass1<Tp, RB, false>;
-        if (prep_smem(k, smem)) return DNA_ERR_CUDA;
-        dna::launch_pdl(k, grid, dim3(NT), smem, st, v, A, B, s_per, status, dcur);
-    }
-    return launch_status();
+        // float32 above rank 128: a plain launch.  Its plan fills the SMs in one wave of two CTAs
+        // each, which took longer where programmatic serialisation let it start beside the
+        // operand kernel: N=1000 T=1200, DNA iteration at R = 129 731 us without any, 782 with
+        // it here, 706 as it is (with it in the other kernels); MU at R = 129 289, 340, 282;
+        // DNA at R = 512 1602, 1559, 1566
+        if (sizeof(Tp) == 4 && v.R > f2::MAX_R)
+            k<<<grid, NT, smem, st>>>(v, A, B, s_per, status, dcur);
+        else
+            dna::launch_pdl(k, grid, dim3(NT), smem, st, v, A, B, s_per, status, dcur);
+        return launch_status();
+    };
+    return with_b ? launch(k_pass1<Tp, RB, true>) : launch(k_pass1<Tp, RB, false>);
 }
 
 template <typename Tp, int RB, int NC, bool FULL>
