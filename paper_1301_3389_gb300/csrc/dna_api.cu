@@ -905,16 +905,19 @@ dna::SparseSegs segs(const dna_ctx* c, int w) {
     return dna::SparseSegs{c->seg_col[w], c->seg_k0[w], c->seg_k1[w], c->seg_ptr[w], c->nseg[w]};
 }
 
-// Both factors as rows of R4 values for the sparse kernels: a transposed copy of H, and W
-// itself where its rows are 16-byte words already.
+// The factors as rows of R4 values for the sparse kernels: W itself where its rows are 16-byte
+// words already, and (Hr given) a transposed copy of H.
 template <typename Tp>
 int sparse_rows(dna_ctx* c, const Tp** Wr, const Tp** Hr) {
     using S = dna::Simt<Tp>;
     const bool direct = c->R4 == c->R && reinterpret_cast<uintptr_t>(c->W) % 16 == 0;
     *Wr = static_cast<const Tp*>(direct ? c->W : c->Wr);
-    *Hr = static_cast<const Tp*>(c->Hr);
-    return phase(c, DNA_PHASE_OPERANDS, direct ? 1 : 2, [&] {
-        int e = S::transpose(static_cast<const Tp*>(c->H), c->R, c->T, c->R4,
+    if (Hr) *Hr = static_cast<const Tp*>(c->Hr);
+    if (direct && !Hr) return DNA_OK;
+    return phase(c, DNA_PHASE_OPERANDS, (Hr ? 1 : 0) + (direct ? 0 : 1), [&] {
+        int e = DNA_OK;
+        if (Hr)
+            e = S::transpose(static_cast<const Tp*>(c->H), c->R, c->T, c->R4,
                              static_cast<Tp*>(c->Hr), c->stream);
         if (!e && !direct)
             e = S::pad_rows(static_cast<const Tp*>(c->W), c->N, c->R, c->R4,
@@ -979,13 +982,15 @@ int sparse_kl(dna_ctx* c) {
     using S = dna::Simt<Tp>;
     const View v = make_view(c, false);
     cudaStream_t st = c->stream;
-    const Tp *Wr, *Hr;
-    if (int e = sparse_rows<Tp>(c, &Wr, &Hr)) return e;
+    // a segment reads one column of H, the columns' sums each column once more: a transposed copy
+    // costs more than it saves (36771 x 10212, 1.34 M non-zeros, R = 64: 83 us with it, 81 without)
+    const Tp* Wr;
+    if (int e = sparse_rows<Tp>(c, &Wr, nullptr)) return e;
     return phase(c, DNA_PHASE_KL, 5, [&] {
         int e = S::scale_ops(v, nullptr, false, nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0,
                              c->gpart, st);
         if (!e) e = S::raw_sums(c->gpart, S::glue_parts(v.S), c->R, c->c0, st);
-        if (!e) e = S::sp_kl(v, segs(c, 0), c->ridx, static_cast<const Tp*>(c->cval), Wr, Hr, c->R4,
+        if (!e) e = S::sp_kl(v, segs(c, 0), c->ridx, static_cast<const Tp*>(c->cval), Wr, c->R4,
                              c->c0, c->dseg, c->dpart, c->status, st);
         return e ? e : dna::reduce_sum(c->dpart, c->T, c->kl_dev, c->kl_part, st);
     });

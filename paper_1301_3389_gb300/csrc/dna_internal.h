@@ -213,8 +213,8 @@ template <typename Tp> struct Simt {
                          const Tp* Xd, int64_t R4, const Tp* c3, uint8_t* choice, double* dfin,
                          double* fpart, double reg, bool mu, int* status, cudaStream_t st);
     static int sp_kl(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-                     const Tp* Yr, const Tp* Xr, int64_t R4, const double* c0, double* dseg,
-                     double* part, int* status, cudaStream_t st);
+                     const Tp* Yr, int64_t R4, const double* c0, double* dseg, double* part,
+                     int* status, cudaStream_t st);
     // out (n x ld) = in (n x R) with zeros past R
     static int pad_rows(const Tp* in, int64_t n, int64_t R, int64_t ld, Tp* out, cudaStream_t st);
     // out (cols x ld) = in^t (in rows x cols), zeros past `rows`, all row-major

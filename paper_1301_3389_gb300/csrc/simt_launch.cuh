@@ -613,20 +613,19 @@ int Simt<Tp>::sp_select(const View& v, const SparseSegs& sg, const double* dseg,
 
 template <typename Tp>
 int Simt<Tp>::sp_kl(const View& v, const SparseSegs& sg, const int32_t* idx, const Tp* val,
-                    const Tp* Yr, const Tp* Xr, int64_t R4, const double* c0, double* dseg,
-                    double* part, int* status, cudaStream_t st) {
-    if (sg.n > 0) {
-        const int e = simt::by_lanes(v.R, [&](auto lpn) {
-            sparse::k_sp_kl<Tp, decltype(lpn)::value>
-                <<<simt::sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(R4, sg, idx, val, Yr, Xr,
-                                                                     dseg);
-            return simt::launch_status();
-        });
-        if (e) return e;
-    }
-    sparse::k_sp_reduce_kl<Tp><<<simt::sp_grid(v.O), sparse::WARPS * 32, 0, st>>>(
-        v.O, v.R, R4, sg.sptr, dseg, Xr, c0, part, status);
-    return simt::launch_status();
+                    const Tp* Yr, int64_t R4, const double* c0, double* dseg, double* part,
+                    int* status, cudaStream_t st) {
+    return simt::by_lanes(v.R, [&](auto lpn) {
+        constexpr int LPN = decltype(lpn)::value;
+        if (sg.n > 0) {
+            sparse::k_sp_kl<Tp, LPN><<<simt::sp_grid(sg.n), sparse::WARPS * 32, 0, st>>>(
+                v, R4, sg, idx, val, Yr, dseg);
+            if (simt::launch_status()) return DNA_ERR_CUDA;
+        }
+        sparse::k_sp_reduce_kl<Tp, LPN><<<simt::sp_grid(v.O), sparse::WARPS * 32, 0, st>>>(
+            v, sg.sptr, dseg, c0, part, status);
+        return simt::launch_status();
+    });
 }
 
 template <typename Tp>
