@@ -49,7 +49,10 @@ int pass1_rb(const View& v, Tp* A, Tp* B, int splits, int64_t s_per, bool with_b
             dna::launch_pdl(k, grid, dim3(NT), smem, st, v, A, B, s_per, status, dcur);
         return launch_status();
     };
-    return with_b ? launch(k_pass1<Tp, RB, true>) : launch(k_pass1<Tp, RB, false>);
+    // float32 at ranks up to 128 comes here for descent selection only, which needs B
+    if constexpr (sizeof(Tp) == 8 || RB == 128)
+        if (!with_b) return launch(k_pass1<Tp, RB, false>);
+    return with_b ? launch(k_pass1<Tp, RB, true>) : DNA_ERR_UNSUPPORTED;
 }
 
 template <typename Tp, int RB, int NC, bool FULL>
