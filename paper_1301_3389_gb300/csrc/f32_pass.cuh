@@ -22,9 +22,10 @@
 // Measured against the kernels of simt_kernels.cuh (microseconds, H and W view, with the
 // split plans of each): N=1024 T=11554 R=80 pass 1 304, 459 -> 152, 150 and pass 2 213, 368 ->
 // 117, 119; N=4096 T=165 R=80 pass 1 203, 57 -> 23, 21; N=256 T=512 R=16 pass 1 24, 26 -> 6.6,
-// 6.5.  At N=4096 T=16384 R=128 pass 1 runs at 45.5 TFLOP/s of algorithm, pass 2 at 41.8; the
-// FMA pipe is busy 60 % of the time, the rest is shared-memory bandwidth (two 16-byte loads
-// per 8 packed FMAs in the z tile take as long as the FMAs) and the element-wise part.
+// 6.5.  At N=4096 T=16384 R=128 pass 1 runs at 45.5 TFLOP/s of algorithm, pass 2 at 40.8; the
+// FMA pipe is busy 70 to 73 % of the time in pass 1, the rest is shared-memory bandwidth (two
+// 16-byte loads per 8 packed FMAs in the z tile take as long as the FMAs) and the element-wise
+// part.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(256) k_split_sum(Tp* __restrict__ A, Tp* __res
 // threads, group g adding the contiguous splits [g k, (g + 1) k) (k = ceil(splits / 8), up
 // to eight loads in flight) and the eight group sums added in order.  blockIdx.y picks A or
 // B.  With one thread per value the loads of the splits follow one another in rounds of
-// L2 latency: 64 splits of 80 x 165 values take 16 rounds there and one here.
+// L2 latency: 64 splits of 80 x 165 values take 8 rounds there and one here.
 template <typename Tp, int VEC>
 __global__ void __launch_bounds__(256) k_split_sum_par(Tp* __restrict__ A, Tp* __restrict__ B,
                                                        int64_t n, int splits) {
