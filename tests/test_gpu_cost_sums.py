@@ -79,14 +79,18 @@ class Bound:
 
 
 @pytest.mark.parametrize("which", [0, 1])
-@pytest.mark.parametrize("form", ["f32", "group_f32", "sparse"])
-def test_infinite_mu_cost_keeps_newton(form, which):
+@pytest.mark.parametrize("form,R", [("f32", 2), ("f32", 70), ("f32", 120), ("group_f32", 2),
+                                    ("group_f32", 50), ("sparse", 2), ("sparse", 40),
+                                    ("sparse", 120)])
+def test_infinite_mu_cost_keeps_newton(form, R, which):
     """Column 0 (row 0 for the W step): the MU gain of component a is v y / z = 2e-38, so the
     MU z of row 0, 1e-8 * 2e-38, underflows to 0 where v = 2e-38 > 0: infinite cost.  The
-    Newton gain is floored at eps = 0.01 and its cost is finite."""
+    Newton gain is floored at eps = 0.01 and its cost is finite.  Component b is R - 1 equal
+    components, each an equal share."""
     V = np.array([[2e-38, 0.0, 1.0], [0.0, 1.0, 2.0], [1.0, 1.0, 3.0]])
-    Y = np.array([[1e-8, 0.0], [1.0, 0.0], [0.0, 1.0]])
-    X = np.ones((2, 3))
+    Y = np.array([[1e-8, 0.0], [1.0, 0.0], [0.0, 1.0]])[:, [0] + (R - 1) * [1]]
+    X = np.ones((R, 3))
+    X[1:] /= R - 1
     # the third column needs z > 0 everywhere; its selection does not matter
     with Bound(form, *((V, Y, X) if which == 0 else (V.T, X.T, Y.T))) as b:
         b.step(which)
@@ -98,8 +102,9 @@ def test_infinite_mu_cost_keeps_newton(form, which):
             assert dm[0] == np.inf and np.isfinite(dd[0]) and np.isfinite(dm[1:]).all()
 
 
-@pytest.mark.parametrize("R", [4, 40])
-@pytest.mark.parametrize("form", ["f32", "bf16", "group_f32", "group_bf16", "sparse"])
+@pytest.mark.parametrize("form,R", [(f, R) for f in ("f32", "bf16", "group_f32", "group_bf16",
+                                                    "sparse") for R in (4, 40)] +
+                         [("f32", 90), ("f32", 128), ("bf16", 100), ("sparse", 128)])
 def test_infinite_kl(form, R):
     rng = np.random.default_rng(R)
     V, W, H = rng.random((150, 70)) + 0.1, rng.random((150, R)), rng.random((R, 70))
